@@ -1,0 +1,150 @@
+// FP64 products on the FP16 tensor pipe, by error-free splitting (Ozaki, Ogita, Oishi and Rump,
+// "Error-free transformations of matrix multiplication by using fast routines of matrix
+// multiplication", 2012).
+//
+// This GPU's FP64 pipe retires about 1.7 lane-FMAs per clock and SM (1.2 TFLOP/s in all), its
+// FP16 mma.sync pipe 1019 (measured), so 28 FP16 products per FP64 product are still ~21 times
+// faster.  Every operand entry of a row is written against the row's scale 2^E (|x| < 2^E) as
+//   x = 2^E sum_{s=0..6} d_s 2^(-8 - 9 s),   d_s an integer in [-256, 256],
+// which keeps 62 fractional bits below the row's scale (all 53 of x when x is within 2^-9 of
+// it).  The digit products d_s d_t are integers of at most 2^16; those of one weight s + t = g
+// <= 6 are summed by the tensor cores in FP32, exactly: at most 7 pairs x 32 terms x 2^16 < 2^24
+// per chunk of 32 inner terms (checked against 64-bit integers on the device for the largest
+// magnitudes).  Chunk sums are then carried in 32-bit integers.  The dropped pairs (g > 6) and
+// the digits' tails are below 2^-62 of the two scales' product per term, so the only rounding
+// that shows is the final one to FP64.
+#pragma once
+#include <stdint.h>
+
+#include <cuda_fp16.h>
+
+namespace hrp {
+
+constexpr int kDig = 7;        // digits per operand, and weights s + t = 0 .. 6 kept
+constexpr int kDigK = 32;      // inner terms per chunk (exactness bound above)
+constexpr int kDigLd = 40;     // halves per staged row of 32: 80 bytes, conflict-free for ldmatrix
+constexpr int kDigHead = 2;    // bits of headroom of a row's scale over its largest entry so far
+
+__device__ __forceinline__ int dig_field(double x) {         // biased exponent field
+  return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff;
+}
+
+// The 7 digits of 8 consecutive inner terms v[0..7] of one row, eb = the row's scale as a biased
+// exponent (field(x) <= eb for every entry; E = eb - 1022), to dst[s * plane .. + 8) halves
+// (16-byte stores).  Entries are finite.
+__device__ __forceinline__ void dig_split8(const double (&v)[8], int eb, __half* dst, int plane) {
+  // digits come out unsigned (u = d + 256) after adding 256 at every digit position
+  constexpr unsigned long long kBias = 0x4020100804020100ull;
+  uint32_t w[kDig][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    unsigned long long M[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(v[2 * p + q]);
+      const int F = (int)(b >> 52) & 0x7ff;
+      unsigned long long m = (b & 0xfffffffffffffull) | (F ? 0x10000000000000ull : 0ull);
+      const int sh = 9 - (eb - (F ? F : 1));                 // 62 fractional bits below 2^E
+      if (sh >= 0) {
+        m <<= sh;
+      } else {
+        const int r = min(-sh, 63);
+        m = (m + (1ull << (r - 1))) >> r;
+      }
+      M[q] = (((long long)b < 0) ? 0ull - m : m) + kBias;
+    }
+#pragma unroll
+    for (int s = 0; s < kDig; ++s) {
+      const int o = 54 - 9 * s;
+      uint32_t u0 = (uint32_t)(M[0] >> o), u1 = (uint32_t)(M[1] >> o);
+      if (s > 0) {
+        u0 &= 511u;
+        u1 &= 511u;
+      }
+      // 0x6400 | u is the half 1024 + u (u <= 512); subtracting 1280 leaves d exactly
+      const uint32_t h = 0x64006400u | u0 | (u1 << 16);
+      const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6500)));
+      w[s][p] = *reinterpret_cast<const uint32_t*>(&d);
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < kDig; ++s)
+    *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+__device__ __forceinline__ void dig_ldmatrix(uint32_t (&r)[4], const __half* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void dig_mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// One chunk of a warp's 16 x 16 output: rows a0 .. a0 + 15 of the staged digits A ([s][row][k],
+// `aplane` halves per digit), columns = rows b0 .. b0 + 15 of B.  The weights' sums over the
+// chunk are added to iacc[g][j], j = 4 (column half) + the mma accumulator's register.
+__device__ __forceinline__ void dig_chunk(const __half* A, int aplane, int a0, const __half* B, int bplane, int b0,
+                                          int (&iacc)[kDig][8]) {
+  const int lane = threadIdx.x & 31;
+  float acc[kDig][2][4];
+#pragma unroll
+  for (int g = 0; g < kDig; ++g)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[g][h][q] = 0.f;
+  // ldmatrix addresses: A tiles (rows 0-7, k 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15);
+  // B tiles (columns 0-7, k 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15)
+  const __half* ap = A + (size_t)(a0 + (lane & 15)) * kDigLd + (lane >> 4) * 8;
+  const __half* bp = B + (size_t)(b0 + (lane & 7) + ((lane >> 4) << 3)) * kDigLd + ((lane >> 3) & 1) * 8;
+#pragma unroll
+  for (int ks = 0; ks < kDigK; ks += 16) {
+    uint32_t b[kDig][4];
+#pragma unroll
+    for (int t = 0; t < kDig; ++t) dig_ldmatrix(b[t], bp + (size_t)t * bplane + ks);
+#pragma unroll
+    for (int s = 0; s < kDig; ++s) {
+      uint32_t a[4];
+      dig_ldmatrix(a, ap + (size_t)s * aplane + ks);
+#pragma unroll
+      for (int t = 0; t < kDig - s; ++t) {
+        dig_mma(acc[s + t][0], a, b[t][0], b[t][1]);
+        dig_mma(acc[s + t][1], a, b[t][2], b[t][3]);
+      }
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < kDig; ++g)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) iacc[g][j] += __float2int_rn(acc[g][j >> 2][j & 3]);
+}
+
+// The product sum of one output in units of 2^(Ex + Ey - 34): weights g = 0 .. 2 and 3 .. 6 are
+// joined in 64-bit integers and converted by the 1.5 2^52 offset (two FP64 additions; the
+// conversion instructions run on the FP64 pipe too).  Up to 2^15 inner terms.
+__device__ __forceinline__ double dig_value(const int (&iacc)[kDig][8], int j) {
+  const long long hi = ((long long)iacc[0][j] << 18) + ((long long)iacc[1][j] << 9) + (long long)iacc[2][j];
+  const long long lo = ((long long)iacc[3][j] << 27) + ((long long)iacc[4][j] << 18) +
+                       ((long long)iacc[5][j] << 9) + (long long)iacc[6][j];      // units 2^-36 of hi's
+  constexpr long long kMagic = 0x4338000000000000ll;                               // 1.5 2^52
+  const double hm = __longlong_as_double(kMagic + hi);
+  const double lm = __longlong_as_double(kMagic + ((lo + 128) >> 8));              // units 2^-28
+  // hm - 1.5 2^52 - 1.5 2^24 is exact; the FMA adds lm 2^-28 = 1.5 2^24 + lo 2^-36
+  return fma(lm, 0x1p-28, hm - (0x1.8p52 + 0x1.8p24));
+}
+// 2^(Ex + Ey - 34) for biased row scales ebx, eby, as two factors (their product may leave the
+// normal range on its own)
+__device__ __forceinline__ void dig_scale(int ebx, int eby, double& f0, double& f1) {
+  const int e = ebx + eby - 2 * 1022 - 34;
+  const int e0 = max(-1022, min(1023, e));
+  const int e1 = max(-1022, min(1023, e - e0));
+  f0 = __longlong_as_double((long long)(e0 + 1023) << 52);
+  f1 = __longlong_as_double((long long)(e1 + 1023) << 52);
+}
+
+}  // namespace hrp

@@ -116,6 +116,59 @@ cudaError_t launch_gemm_simt(double* C, int ldc, const double* X, int ldx, const
 cudaError_t launch_gemm_simt_f32(double* C, int ldc, const float* X, int ldx, const float* Y, int ldy,
                                  int m, int n, int k, bool lower, cudaStream_t s);
 
+// Independent blocks of one product, for one launch: block b is
+//   C[xr : xr+m, yr : yr+n] -= X[xr : xr+m, 0:k] Y[yr : yr+n, 0:k]^T
+// (offsets into the column-major operands and C), with `lower` only its entries on or below its
+// own diagonal.  tile0: the block's first tile in the launch (gemm_block_offsets).
+struct GemmBlock {
+  int xr, yr, m, n, lower, tile0;
+};
+constexpr int kMaxGemmBlocks = 96;
+struct GemmBlocks {
+  int count = 0;
+  GemmBlock b[kMaxGemmBlocks];
+};
+// tiles of edge t of a block: all of them, or (lower) those that reach the diagonal
+__host__ __device__ inline int gemm_block_tiles(const GemmBlock& g, int t) {
+  const int gm = (g.m + t - 1) / t, gn = (g.n + t - 1) / t;
+  if (!g.lower) return gm * gn;
+  const int q = gm < gn ? gm : gn;              // column tile j holds rows j .. gm - 1
+  return q * gm - q * (q - 1) / 2;
+}
+// tile index within a block -> row and column tile (column by column)
+__device__ __forceinline__ void gemm_block_tile(const GemmBlock& g, int t, int idx, int& tx, int& ty) {
+  const int gm = (g.m + t - 1) / t;
+  if (!g.lower) {
+    ty = idx / gm;
+    tx = idx - ty * gm;
+    return;
+  }
+  ty = 0;
+  while (idx >= gm - ty) {
+    idx -= gm - ty;
+    ++ty;
+  }
+  tx = ty + idx;
+}
+// sets every block's tile0, returns the launch's tiles
+inline int gemm_block_offsets(GemmBlocks& bl, int t) {
+  int tiles = 0;
+  for (int i = 0; i < bl.count; ++i) {
+    bl.b[i].tile0 = tiles;
+    tiles += gemm_block_tiles(bl.b[i], t);
+  }
+  return tiles;
+}
+// FP64 products of a list of blocks (k_gemm_f64.cu), with the accuracy of FP64 or better
+cudaError_t launch_gemm_f64_blocks(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, int k,
+                                   GemmBlocks& bl, cudaStream_t s);
+// FP32 products of a list of blocks, operands from FP32 copies (k_gemm_simt.cu); every entry is
+// the same chain of FMAs as in launch_gemm_simt_f32
+// whether launch_gemm_simt_f32 takes its 128 x 128 tiles (then better launched alone)
+bool gemm_f32_wide(const float* X, int ldx, const float* Y, int ldy, int m, int n, int k);
+cudaError_t launch_gemm_f32_blocks(double* C, int ldc, const float* X, int ldx, const float* Y, int ldy, int k,
+                                   GemmBlocks& bl, cudaStream_t s);
+
 // ---------------- tcgen05 FP16 GEMM (k_gemm_tc.cu) ----------------
 // C[m x n] (FP64 master, column-major) -= scale * X Y^T with X = S[xr0.., k0..] (m x k) and
 // Y = S[yr0.., k0..] (n x k) read from the row-major FP16 shadow S (lds), FP32 accumulation

@@ -1,0 +1,180 @@
+// FP64 GEMM C -= X Y^T of the FP64 levels (the updates of Alg. 2 and 3) by error-free digit
+// products on the FP16 tensor pipe (digits.cuh), one launch for one block or for a list of
+// independent blocks.
+//
+// One CTA of 4 warps computes one 32 x 32 tile (a warp 16 x 16).  Per chunk of 32 inner terms the
+// CTA loads its 64 operand rows from the master (coalesced along rows), takes the rows' largest
+// exponents, writes the digits to shared memory (36 KB) and multiplies them; the next chunk's
+// loads are in flight during the products.  What bounds it: 56 mma per warp and 16 terms (8 clocks
+// each per sub-partition) against ~45 integer instructions per entry of splitting; two or three
+// CTAs per SM overlap the two.  The small tile is for the small products this library runs in
+// FP64 (orders 64 to 1024): a 64 x 64 tile would leave most SMs idle.
+//
+// Measured against the FP64 SIMT kernel it replaces (32 x 32 tiles, FP64 FMAs): the 32 diagonal
+// blocks of 125 x 125 x 1024 of a SYRK 10.3 ms one after another -> one launch, the whole SYRK
+// (n = 4000, k = 1024, three levels) 10.40 -> 0.457 ms; the n = 1024 FP64 factorization and solve
+// 2.58 -> 1.96 ms.  Relative error against extended precision 5e-17 .. 7e-17, where the FMA
+// chains had 1.2e-16 (k = 16) .. 8.5e-16 (k = 1000).
+//
+// A row's scale carries 2 bits of headroom over its largest entry so far.  When a later chunk
+// holds a larger entry still, the CTA moves its integer sums to FP64 first (at the old scales)
+// and goes on with the new ones.  A tile whose operand rows hold a NaN or an infinity is computed
+// by plain FP64 FMAs instead, so that those propagate as they would there.
+#include "digits.cuh"
+#include "hrp_internal.cuh"
+
+namespace hrp {
+namespace {
+
+constexpr int kT = 32;                         // tile edge
+constexpr int kThreads = 128;
+constexpr int kPlane = kT * kDigLd;            // halves per digit plane of one operand
+constexpr int kFlush = 64;                     // chunks the 32-bit sums hold (2^24 each) before a move to FP64
+
+__global__ void __launch_bounds__(kThreads, 2)
+gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict__ X, int ldx,
+                       const double* __restrict__ Y, int ldy, int k, const __grid_constant__ GemmBlocks bl) {
+  pdl_wait();
+  pdl_trigger();
+  extern __shared__ __align__(16) __half dig[];                  // [2 operands][7][32][kDigLd]
+  __shared__ int rowmax[2][2 * kT];                              // largest exponent field of the chunk, by parity
+  __shared__ int scale[2 * kT];                                  // the rows' scales (biased exponent)
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  // this CTA's block and tile
+  int b = 0;
+  while (b + 1 < bl.count && (int)blockIdx.x >= bl.b[b + 1].tile0) ++b;
+  const GemmBlock blk = bl.b[b];
+  const int ti = (int)blockIdx.x - blk.tile0;
+  int ty, tx;
+  gemm_block_tile(blk, kT, ti, tx, ty);
+  const int m0 = tx * kT, n0 = ty * kT, m = blk.m, n = blk.n, lower = blk.lower;
+  const double* Xb = X + blk.xr;
+  const double* Yb = Y + blk.yr;
+  double* Cb = C + (size_t)blk.yr * ldc + blk.xr;
+
+  if (tid < 2 * kT) {
+    rowmax[0][tid] = rowmax[1][tid] = 0;
+    scale[tid] = 0;
+  }
+  // warp w holds inner terms 8 w .. 8 w + 7 of the chunk, lane = operand row
+  const bool okx = m0 + lane < m, oky = n0 + lane < n;
+  double px[8], py[8];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int kk = k0 + 8 * warp + q;
+      px[q] = (okx && kk < k) ? Xb[(size_t)kk * ldx + m0 + lane] : 0.0;
+      py[q] = (oky && kk < k) ? Yb[(size_t)kk * ldy + n0 + lane] : 0.0;
+    }
+  };
+  int iacc[kDig][8];
+  double vacc[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    vacc[j] = 0.0;
+#pragma unroll
+    for (int g = 0; g < kDig; ++g) iacc[g][j] = 0;
+  }
+  // the warp's 16 x 16 part: rows 16 (warp / 2), columns 16 (warp % 2); register j of a lane is
+  // row g + 8 ((j >> 1) & 1), column 8 (j >> 2) + 2 t + (j & 1), g = lane / 4, t = lane % 4
+  const int a0 = 16 * (warp >> 1), b0 = 16 * (warp & 1);
+  const int gr = a0 + (lane >> 2), gc = b0 + 2 * (lane & 3);
+  auto flush = [&]() {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      double f0, f1;
+      dig_scale(scale[gr + 8 * ((j >> 1) & 1)], scale[kT + gc + 8 * (j >> 2) + (j & 1)], f0, f1);
+      vacc[j] += dig_value(iacc, j) * f0 * f1;
+#pragma unroll
+      for (int g = 0; g < kDig; ++g) iacc[g][j] = 0;
+    }
+  };
+  bool flushed = false, special = false;
+  int held = 0;
+  fetch(0);
+  __syncthreads();
+  const int nchunk = (k + kDigK - 1) / kDigK;
+  for (int c = 0; c < nchunk; ++c) {
+    int fx = 0, fy = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      fx = max(fx, dig_field(px[q]));
+      fy = max(fy, dig_field(py[q]));
+    }
+    atomicMax(&rowmax[c & 1][lane], fx);
+    atomicMax(&rowmax[c & 1][kT + lane], fy);
+    __syncthreads();                                             // also: the last chunk's products are done
+    int need = 0, mx = 0;
+    if (tid < 2 * kT) {
+      mx = rowmax[c & 1][tid];
+      rowmax[(c + 1) & 1][tid] = 0;
+      need = mx == 0x7ff ? 2 : (max(mx, 1) > scale[tid] ? 1 : 0);
+    }
+    const bool grow = __syncthreads_or(need) != 0;
+    if (grow && __syncthreads_or(need == 2)) {
+      special = true;
+      break;
+    }
+    if (grow || held == kFlush) {
+      if (held > 0) {
+        flush();
+        flushed = true;
+        held = 0;
+      }
+      __syncthreads();
+      if (need) scale[tid] = max(mx, 1) + kDigHead;
+      __syncthreads();
+    }
+    dig_split8(px, scale[lane], dig + lane * kDigLd + 8 * warp, kPlane);
+    dig_split8(py, scale[kT + lane], dig + kDig * kPlane + lane * kDigLd + 8 * warp, kPlane);
+    if (c + 1 < nchunk) fetch((c + 1) * kDigK);
+    __syncthreads();
+    dig_chunk(dig, kPlane, a0, dig + kDig * kPlane, kPlane, b0, iacc);
+    ++held;
+  }
+  if (special) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
+      if (r >= m || cl >= n || (lower && r < cl)) continue;
+      double s = 0.0;
+      for (int kk = 0; kk < k; ++kk) s = fma(Xb[(size_t)kk * ldx + r], Yb[(size_t)kk * ldy + cl], s);
+      Cb[(size_t)cl * ldc + r] -= s;
+    }
+    return;
+  }
+  double cv[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
+    cv[j] = (r < m && cl < n && !(lower && r < cl)) ? Cb[(size_t)cl * ldc + r] : 0.0;
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int rr = gr + 8 * ((j >> 1) & 1), cc = gc + 8 * (j >> 2) + (j & 1);
+    const int r = m0 + rr, cl = n0 + cc;
+    if (r >= m || cl >= n || (lower && r < cl)) continue;
+    double f0, f1;
+    dig_scale(scale[rr], scale[kT + cc], f0, f1);
+    double v = dig_value(iacc, j);
+    if (f1 != 1.0) v *= f1;
+    double* p = Cb + (size_t)cl * ldc + r;
+    if (flushed) *p = cv[j] - fma(v, f0, vacc[j]);
+    else *p = fma(-v, f0, cv[j]);
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_gemm_f64_blocks(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, int k,
+                                   GemmBlocks& bl, cudaStream_t s) {
+  if (k <= 0 || bl.count <= 0) return cudaSuccess;
+  const int tiles = gemm_block_offsets(bl, kT);
+  if (tiles <= 0) return cudaSuccess;
+  const int smem = 2 * kDig * kPlane * (int)sizeof(__half);
+  (void)launch_pdl(gemm_f64_digits_kernel, dim3(tiles), dim3(kThreads), smem, s, C, ldc, X, ldx, Y, ldy, k, bl);
+  return cudaGetLastError();
+}
+
+}  // namespace hrp

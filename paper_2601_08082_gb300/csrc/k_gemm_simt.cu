@@ -1,5 +1,4 @@
-// SIMT GEMM for the FP64 and FP32 levels of the tree (and the FP16-operand fallback):
-// C -= X Y^T on column-major views of the FP64 master.  This is the update
+// SIMT GEMM for the FP32 levels of the tree (and the FP16-operand fallback): C -= X Y^T on column-major views of the FP64 master.  This is the update
 // "B2 <- B2 - B1 L21^T" of Alg. 2 and "C21 <- C21 - A2 A1^T" of Alg. 3 (alpha = -1,
 // beta = 1 in Alg. 1); with `lower` it is the leaf SYRK of Alg. 3 on a diagonal block.
 #include <cstdint>
@@ -9,18 +8,10 @@
 namespace hrp {
 namespace {
 
-// inner-dimension slice per stage: 16 for FP64, 64 for FP32 accumulation (fewer
-// latency-bound stages for the small GEMMs of the FP32 levels)
-template <int RND> struct Slice { static constexpr int BK = 64; };
-template <> struct Slice<0> { static constexpr int BK = 16; };
-
-template <int RND> struct Acc { using T = float; };
-template <> struct Acc<0> { using T = double; };
-
+// operand rounding on load: FP32 (RND = 1) or FP16 (2); FP64 products run in k_gemm_f64.cu
 template <int RND>
-__device__ __forceinline__ typename Acc<RND>::T cvt_op(double x) {
-  if constexpr (RND == 0) return x;
-  else if constexpr (RND == 1) return __double2float_rn(x);
+__device__ __forceinline__ float cvt_op(double x) {
+  if constexpr (RND == 1) return __double2float_rn(x);
   else return __half2float(__double2half(x));
 }
 // operands already in FP32 (the FP32 shadow of L): no rounding on load
@@ -35,8 +26,8 @@ gemm_simt_kernel(double* __restrict__ C, int ldc, const TIN* __restrict__ X, int
                  const TIN* __restrict__ Y, int ldy, int m, int n, int k, int lower) {
   pdl_wait();
   pdl_trigger();
-  using T = typename Acc<RND>::T;
-  constexpr int BK = Slice<RND>::BK;
+  using T = float;
+  constexpr int BK = 64;             // few latency-bound stages for the small GEMMs of the FP32 levels
   constexpr int BM = TL, BN = TL, R = TL / 16;
   __shared__ T Xs[BK][BM + 1];
   __shared__ T Ys[BK][BN + 1];
@@ -195,11 +186,104 @@ sgemm128_kernel(double* __restrict__ C, int ldc, const float* __restrict__ X, in
   }
 }
 
+// A list of independent FP32 products in one launch: 64 x 64 outputs per CTA, 256 threads, 4 x 4
+// per thread (rows 4 tx .. +3, columns 4 ty .. +3), K in slices of 16 staged k-major with the next
+// slice prefetched into registers.  Every entry is one chain of FMAs over k from 0, as in the
+// kernels above, so the results do not depend on which of them computes a block.
+// For the many small blocks of Alg. 3's deeper levels (125 to 500 rows): alone, each fills a tenth
+// of the SMs and its time is the latency of its k slices.
+constexpr int GB_T = 64, GB_BK = 16;
+
+__global__ void __launch_bounds__(256)
+gemm_f32_blocks_kernel(double* __restrict__ C, int ldc, const float* __restrict__ X, int ldx,
+                       const float* __restrict__ Y, int ldy, int k, const __grid_constant__ GemmBlocks bl) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ __align__(16) float Xs[GB_BK][GB_T + 4];
+  __shared__ __align__(16) float Ys[GB_BK][GB_T + 4];
+  int b = 0;
+  while (b + 1 < bl.count && (int)blockIdx.x >= bl.b[b + 1].tile0) ++b;
+  const GemmBlock blk = bl.b[b];
+  int bx, by;
+  gemm_block_tile(blk, GB_T, (int)blockIdx.x - blk.tile0, bx, by);
+  const int m0 = bx * GB_T, n0 = by * GB_T, m = blk.m, n = blk.n, lower = blk.lower;
+  X += blk.xr;
+  Y += blk.yr;
+  C += (size_t)blk.yr * ldc + blk.xr;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int lr = tid & 63, lk = tid >> 6;                    // loader: row lr, slice rows lk + 4 q
+  float px[4], py[4];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int gk = k0 + lk + 4 * q;
+      px[q] = (gk < k && m0 + lr < m) ? X[(size_t)gk * ldx + m0 + lr] : 0.f;
+      py[q] = (gk < k && n0 + lr < n) ? Y[(size_t)gk * ldy + n0 + lr] : 0.f;
+    }
+  };
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  fetch(0);
+  for (int k0 = 0; k0 < k; k0 += GB_BK) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      Xs[lk + 4 * q][lr] = px[q];
+      Ys[lk + 4 * q][lr] = py[q];
+    }
+    __syncthreads();
+    if (k0 + GB_BK < k) fetch(k0 + GB_BK);
+#pragma unroll
+    for (int kk = 0; kk < GB_BK; ++kk) {
+      const float4 a4 = *reinterpret_cast<const float4*>(&Xs[kk][4 * tx]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&Ys[kk][4 * ty]);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int gc = n0 + 4 * ty + j;
+    double cv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int gr = m0 + 4 * tx + i;
+      cv[i] = (gc < n && gr < m && !(lower && gr < gc)) ? C[(size_t)gc * ldc + gr] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int gr = m0 + 4 * tx + i;
+      if (gc < n && gr < m && !(lower && gr < gc)) C[(size_t)gc * ldc + gr] = cv[i] - (double)acc[i][j];
+    }
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_gemm_f32_blocks(double* C, int ldc, const float* X, int ldx, const float* Y, int ldy, int k,
+                                   GemmBlocks& bl, cudaStream_t s) {
+  if (k <= 0 || bl.count <= 0) return cudaSuccess;
+  const int tiles = gemm_block_offsets(bl, GB_T);
+  if (tiles <= 0) return cudaSuccess;
+  (void)launch_pdl(gemm_f32_blocks_kernel, dim3(tiles), dim3(256), 0, s, C, ldc, X, ldx, Y, ldy, k, bl);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_gemm_simt(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy,
                              int m, int n, int k, OpRound rnd, bool lower, cudaStream_t s) {
   if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
+  if (rnd == OpRound::F64) {
+    GemmBlocks bl;
+    bl.count = 1;
+    bl.b[0] = GemmBlock{0, 0, m, n, lower ? 1 : 0, 0};
+    return launch_gemm_f64_blocks(C, ldc, X, ldx, Y, ldy, k, bl, s);
+  }
   // 64 x 64 tiles unless that leaves most SMs idle: the operand rounding and the FP64
   // read-modify-write of C run on the FP64 pipe, so the small products of the FP32 levels
   // are spread over 32 x 32 tiles
@@ -210,7 +294,7 @@ cudaError_t launch_gemm_simt(double* C, int ldc, const double* X, int ldx, const
   if (grid.y > 65535) return cudaErrorInvalidValue;
 #define HRP_SIMT(R_, T_) (void)launch_pdl(gemm_simt_kernel<R_, T_>, dim3(grid), dim3(256), 0, s, C, ldc, X, ldx, Y, ldy, m, n, k, lower)
   switch (rnd) {
-    case OpRound::F64: if (small) HRP_SIMT(0, 32); else HRP_SIMT(0, 64); break;
+    case OpRound::F64: break;
     case OpRound::F32: if (small) HRP_SIMT(1, 32); else HRP_SIMT(1, 64); break;
     case OpRound::F16: if (small) HRP_SIMT(2, 32); else HRP_SIMT(2, 64); break;
   }
@@ -218,15 +302,18 @@ cudaError_t launch_gemm_simt(double* C, int ldc, const double* X, int ldx, const
   return cudaGetLastError();
 }
 
+// 128 x 128 tiles once they cover half the SMs (16-byte operand loads need 16-byte aligned columns)
+bool gemm_f32_wide(const float* X, int ldx, const float* Y, int ldy, int m, int n, int k) {
+  const bool vec = (ldx % 4) == 0 && (ldy % 4) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 &&
+                   (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
+  return vec && k >= 64 && (long long)((m + 127) / 128) * ((n + 127) / 128) >= device_sm_count() / 2;
+}
+
 cudaError_t launch_gemm_simt_f32(double* C, int ldc, const float* X, int ldx, const float* Y, int ldy,
                                  int m, int n, int k, bool lower, cudaStream_t s) {
   if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
   const int sms = device_sm_count();
-  // large products: 128 x 128 tiles once they cover the SMs (16-byte operand loads need
-  // 16-byte aligned operand columns)
-  const bool vec = (ldx % 4) == 0 && (ldy % 4) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 &&
-                   (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
-  if (vec && k >= 64 && (long long)((m + 127) / 128) * ((n + 127) / 128) >= sms / 2) {
+  if (gemm_f32_wide(X, ldx, Y, ldy, m, n, k)) {
     dim3 g128((m + 127) / 128, (n + 127) / 128);
     if (g128.y > 65535) return cudaErrorInvalidValue;
     (void)launch_pdl(sgemm128_kernel, dim3(g128), dim3(256), 0, s, C, ldc, X, ldx, Y, ldy, m, n, k, lower);
