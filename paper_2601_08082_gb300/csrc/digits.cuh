@@ -29,10 +29,10 @@ __device__ __forceinline__ int dig_field(double x) {         // biased exponent 
   return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff;
 }
 
-// The 7 digits of 8 consecutive inner terms v[0..7] of one row, eb = the row's scale as a biased
-// exponent (field(x) <= eb for every entry; E = eb - 1022), to dst[s * plane .. + 8) halves
-// (16-byte stores).  Entries are finite.
-__device__ __forceinline__ void dig_split8(const double (&v)[8], int eb, __half* dst, int plane) {
+// The 7 digits of 8 consecutive inner terms v[0..7] of one row, eb[i] = the scale of v[i] as a
+// biased exponent (field(v[i]) <= eb[i]; E = eb - 1022), to dst[s * plane .. + 8) halves (16-byte
+// stores).  Entries are finite.
+__device__ __forceinline__ void dig_split8(const double (&v)[8], const int (&eb)[8], __half* dst, int plane) {
   // digits come out unsigned (u = d + 256) after adding 256 at every digit position
   constexpr unsigned long long kBias = 0x4020100804020100ull;
   uint32_t w[kDig][4];
@@ -44,7 +44,7 @@ __device__ __forceinline__ void dig_split8(const double (&v)[8], int eb, __half*
       const unsigned long long b = (unsigned long long)__double_as_longlong(v[2 * p + q]);
       const int F = (int)(b >> 52) & 0x7ff;
       unsigned long long m = (b & 0xfffffffffffffull) | (F ? 0x10000000000000ull : 0ull);
-      const int sh = 9 - (eb - (F ? F : 1));                 // 62 fractional bits below 2^E
+      const int sh = 9 - (eb[2 * p + q] - (F ? F : 1));      // 62 fractional bits below 2^E
       if (sh >= 0) {
         m <<= sh;
       } else {
@@ -72,8 +72,20 @@ __device__ __forceinline__ void dig_split8(const double (&v)[8], int eb, __half*
     *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
+// the same with one scale for all 8
+__device__ __forceinline__ void dig_split8(const double (&v)[8], int eb, __half* dst, int plane) {
+  const int e[8] = {eb, eb, eb, eb, eb, eb, eb, eb};
+  dig_split8(v, e, dst, plane);
+}
+
 __device__ __forceinline__ void dig_ldmatrix(uint32_t (&r)[4], const __half* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void dig_ldmatrix_t(uint32_t (&r)[4], const __half* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"((uint32_t)__cvta_generic_to_shared(p))
                : "memory");
@@ -127,7 +139,8 @@ __device__ __forceinline__ void dig_chunk(const __half* A, int aplane, int a0, c
 // The product sum of one output in units of 2^(Ex + Ey - 34): weights g = 0 .. 2 and 3 .. 6 are
 // joined in 64-bit integers and converted by the 1.5 2^52 offset (two FP64 additions; the
 // conversion instructions run on the FP64 pipe too).  Up to 2^15 inner terms.
-__device__ __forceinline__ double dig_value(const int (&iacc)[kDig][8], int j) {
+template <int NJ>
+__device__ __forceinline__ double dig_value(const int (&iacc)[kDig][NJ], int j) {
   const long long hi = ((long long)iacc[0][j] << 18) + ((long long)iacc[1][j] << 9) + (long long)iacc[2][j];
   const long long lo = ((long long)iacc[3][j] << 27) + ((long long)iacc[4][j] << 18) +
                        ((long long)iacc[5][j] << 9) + (long long)iacc[6][j];      // units 2^-36 of hi's
@@ -145,6 +158,16 @@ __device__ __forceinline__ void dig_scale(int ebx, int eby, double& f0, double& 
   const int e1 = max(-1022, min(1023, e - e0));
   f0 = __longlong_as_double((long long)(e0 + 1023) << 52);
   f1 = __longlong_as_double((long long)(e1 + 1023) << 52);
+}
+
+// v 2^e by integer addition to the exponent (the FP64 pipe is the slow one); exact unless the
+// result leaves the normal range, where ldexp rounds it
+__device__ __forceinline__ double dig_shift(double v, int e) {
+  const long long b = __double_as_longlong(v);
+  const int F = (int)(b >> 52) & 0x7ff;
+  if (F == 0) return v;                          // a sum of digits: zero, never subnormal
+  if (F + e >= 1 && F + e <= 2046) return __longlong_as_double(b + ((long long)e << 52));
+  return ldexp(v, e);
 }
 
 }  // namespace hrp

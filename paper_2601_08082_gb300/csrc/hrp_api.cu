@@ -59,6 +59,8 @@ struct hrp_handle_s {
   size_t work_cap = 0;
   unsigned char* pwork = nullptr;  // POTRS diagonal-block inverses
   size_t pwork_cap = 0;
+  unsigned char* rwork = nullptr;  // scales and digits of the residual's operands
+  size_t rwork_cap = 0;
   double* d_norms = nullptr;   // 2 * 64 doubles
   double* h_norms = nullptr;   // pinned host mirror
   long long launches = 0;
@@ -810,6 +812,7 @@ hrp_status hrp_destroy(hrp_handle* h) {
   cudaFree(h->work);
   cudaFree(h->d_norms);
   cudaFree(h->pwork);
+  cudaFree(h->rwork);
   if (h->h_norms) cudaFreeHost(h->h_norms);
   for (cudaEvent_t e : h->events) cudaEventDestroy(e);
   for (cudaEvent_t e : h->bevents) cudaEventDestroy(e);
@@ -1046,7 +1049,7 @@ static hrp_status gmres_correction(hrp_handle* h, const double* dA, int lda, int
   while (k < m && e == cudaSuccess) {
     double* vk = V + (size_t)k * n;
     // w = M^{-1} A v_k (the residual kernel gives -A v_k from a zero right-hand side)
-    e = launch_residual(dA, lda, vk, n, zero, n, w, n, n, 1, s);
+    e = launch_residual(dA, lda, vk, n, zero, n, w, n, n, 1, h->rwork, s);
     if (e == cudaSuccess) e = launch_scale(w, w, -1.0, n, false, s);
     if (e != cudaSuccess) break;
     if ((st = potrs_impl(h, n, 1, h->fact, n, w, n, false, s)) != HRP_OK) return st;
@@ -1129,6 +1132,7 @@ hrp_status hrp_posv(hrp_handle* h, const hrp_tree* tree, int n, int nrhs, const 
   if (n == 0 || nrhs == 0) return HRP_OK;
   if ((st = ensure(h, &h->fact, &h->fact_cap, (size_t)n * n)) != HRP_OK) return st;
   if ((st = ensure(h, &h->work, &h->work_cap, (size_t)n * nrhs)) != HRP_OK) return st;
+  if ((st = ensure(h, &h->rwork, &h->rwork_cap, residual_workspace_bytes(n))) != HRP_OK) return st;
   if (!tree) return set_err(h, HRP_ERR_INVALID_ARG, "no tree");
   cudaError_t e;
   hrp_tree fallback;
@@ -1160,7 +1164,7 @@ hrp_status hrp_posv(hrp_handle* h, const hrp_tree* tree, int n, int nrhs, const 
     double prev = 1e300;
     bool diverged = false;
     while (true) {
-      if ((e = launch_residual(dA, lda, dX, ldx, dB, ldb, h->work, n, n, nrhs, s)) != cudaSuccess)
+      if ((e = launch_residual(dA, lda, dX, ldx, dB, ldb, h->work, n, n, nrhs, h->rwork, s)) != cudaSuccess)
         return cuda_status(h, e, "hrp_posv residual");
       if ((e = launch_col_norms2(h->work, n, dB, ldb, n, nrhs, h->d_norms, s)) != cudaSuccess)
         return cuda_status(h, e, "hrp_posv norms");
@@ -1499,7 +1503,7 @@ namespace {
 constexpr int kBatchStreams = 32;
 
 struct SysWork {
-  size_t shadow, w32, pinv, ticket, fact, res;   // byte offsets into h->bwork
+  size_t shadow, w32, pinv, ticket, fact, res, rwork;   // byte offsets into h->bwork
   int lds;
 };
 
@@ -1519,6 +1523,7 @@ hrp_status batch_prepare(hrp_handle* h, int batch, const int* n, std::vector<Sys
     w.ticket = take(sizeof(int));
     w.fact = nrhs_ir ? take(sizeof(double) * (size_t)ni * ni) : 0;
     w.res = nrhs_ir ? take(sizeof(double) * (size_t)ni * nrhs_ir + sizeof(double) * 2 * nrhs_ir) : 0;
+    w.rwork = nrhs_ir ? take(residual_workspace_bytes(ni)) : 0;
   }
   unsigned char* old = h->bwork;
   size_t old_cap = h->bwork_cap;
@@ -2244,7 +2249,7 @@ extern "C" hrp_status hrp_posv_batched(hrp_handle* h, const hrp_tree* const* tre
         note(launch_axpy_matrix(dX[i], ldx[i], R, n[i], n[i], nrhs, si));
         ++its[i];
       }
-      note(launch_residual(dA[i], lda[i], dX[i], ldx[i], dB[i], ldb[i], R, n[i], n[i], nrhs, si));
+      note(launch_residual(dA[i], lda[i], dX[i], ldx[i], dB[i], ldb[i], R, n[i], n[i], nrhs, h->bwork + ws[i].rwork, si));
       note(launch_col_norms2(R, n[i], dB[i], ldb[i], n[i], nrhs, R + (size_t)n[i] * nrhs, si));
     }
     if ((st = join(h, s)) != HRP_OK) break;

@@ -220,9 +220,16 @@ cudaError_t launch_fill_spd_uniform(double* A, int lda, int n, unsigned long lon
 cudaError_t launch_finalize_info(int* info, cudaStream_t s);
 cudaError_t launch_copy_lower(double* dst, int ldd, const double* src, int lds, int n, cudaStream_t s);
 cudaError_t launch_copy_matrix(double* dst, int ldd, const double* src, int lds, int m, int n, cudaStream_t s);
-// R = B - A X with A symmetric from its lower triangle (FP64). R, B, X: n x nrhs.
+// R = B - A X with A symmetric from its lower triangle, with FP64 accuracy (k_residual.cu). R, B,
+// X: n x nrhs.  work: device scratch of residual_workspace_bytes(n), no initial contents needed.
+constexpr int kResBlock = 64, kResRhs = 16;
+constexpr size_t kResFragBytes = (size_t)(kResBlock / 16) * 7 * (kResRhs / 8) * 32 * 8;   // X digits of one block
+constexpr size_t residual_workspace_bytes(int n) {
+  const size_t nb = (size_t)((n + kResBlock - 1) / kResBlock);
+  return nb * (kResFragBytes + sizeof(int) * (kResBlock + kResRhs + 1));
+}
 cudaError_t launch_residual(const double* A, int lda, const double* X, int ldx, const double* B, int ldb,
-                            double* R, int ldr, int n, int nrhs, cudaStream_t s);
+                            double* R, int ldr, int n, int nrhs, void* work, cudaStream_t s);
 // out[j] = ||R[:, j]||_2^2 and out[nrhs + j] = ||B[:, j]||_2^2 (accumulated with atomics; zeroed here)
 cudaError_t launch_col_norms2(const double* R, int ldr, const double* B, int ldb, int n, int nrhs,
                               double* out, cudaStream_t s);

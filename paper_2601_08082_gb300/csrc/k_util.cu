@@ -1,6 +1,5 @@
-// Small device utilities of the solver: info handling, copies, the FP64 residual of the
-// refinement loop (R = B - A X with A read once from its lower triangle), column norms,
-// and the FP64 backward error ||A - L L^T||_F / ||A||_F (Sec. 4.2 accuracy metric).
+// Small device utilities of the solver: info handling, copies, column norms, and the FP64
+// backward error ||A - L L^T||_F / ||A||_F (Sec. 4.2 accuracy metric).
 #include <climits>
 
 #include <algorithm>
@@ -52,57 +51,12 @@ __global__ void axpy_matrix_kernel(double* X, int ldx, const double* D, int ldd,
   }
 }
 
-// ---- residual R -= A X over lower-triangle tiles (R preset to B) ----
-constexpr int RT = 64;
-constexpr int RNRHS = 16;
-
 __device__ __forceinline__ void tri_index(long long t, int& I, int& J) {
   long long i = (long long)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
   while (i * (i + 1) / 2 > t) --i;
   while ((i + 1) * (i + 2) / 2 <= t) ++i;
   I = (int)i;
   J = (int)(t - i * (i + 1) / 2);
-}
-
-__global__ void __launch_bounds__(256)
-residual_tile_kernel(const double* __restrict__ A, int lda, const double* __restrict__ X, int ldx,
-                     double* __restrict__ R, int ldr, int n, int nrhs) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ double As[RT][RT + 1];
-  __shared__ double xI[RNRHS][RT];
-  __shared__ double xJ[RNRHS][RT];
-  int I, J;
-  tri_index(blockIdx.x, I, J);
-  const int I0 = I * RT, J0 = J * RT;
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < RT * RT; idx += 256) {
-    int i = idx % RT, j = idx / RT;
-    int gi = I0 + i, gj = J0 + j;
-    As[i][j] = (gi < n && gj < n && gi >= gj) ? A[(size_t)gj * lda + gi] : 0.0;
-  }
-  for (int idx = tid; idx < RT * nrhs; idx += 256) {
-    int i = idx % RT, c = idx / RT;
-    xI[c][i] = (I0 + i < n) ? X[(size_t)c * ldx + I0 + i] : 0.0;
-    xJ[c][i] = (J0 + i < n) ? X[(size_t)c * ldx + J0 + i] : 0.0;
-  }
-  __syncthreads();
-  const int i = tid % RT, g = tid / RT;          // 4 groups of right-hand sides
-  for (int c = g; c < nrhs; c += 4) {
-    // row i of block I: sum_j A(I0+i, J0+j) x(J0+j), using symmetry inside a diagonal tile
-    double y = 0.0;
-    if (I == J) {
-      for (int j = 0; j < RT; ++j) y += (j <= i ? As[i][j] : As[j][i]) * xJ[c][j];
-    } else {
-      for (int j = 0; j < RT; ++j) y += As[i][j] * xJ[c][j];
-    }
-    if (I0 + i < n) atomicAdd(R + (size_t)c * ldr + I0 + i, -y);
-    if (I != J) {
-      double z = 0.0;                          // row i of block J: sum_r A(I0+r, J0+i) x(I0+r)
-      for (int r = 0; r < RT; ++r) z += As[r][i] * xI[c][r];
-      if (J0 + i < n) atomicAdd(R + (size_t)c * ldr + J0 + i, -z);
-    }
-  }
 }
 
 __global__ void col_norms2_kernel(const double* R, int ldr, const double* B, int ldb, int n, int nrhs, double* out) {
@@ -269,22 +223,6 @@ cudaError_t launch_axpy_matrix(double* X, int ldx, const double* D, int ldd, int
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
   (void)launch_pdl(axpy_matrix_kernel, dim3(grid_for((size_t)n * nrhs, 256)), dim3(256), 0, s, X, ldx, D, ldd, n, nrhs);
   return cudaGetLastError();
-}
-cudaError_t launch_residual(const double* A, int lda, const double* X, int ldx, const double* B, int ldb,
-                            double* R, int ldr, int n, int nrhs, cudaStream_t s) {
-  if (n <= 0 || nrhs <= 0) return cudaSuccess;
-  cudaError_t e = launch_copy_matrix(R, ldr, B, ldb, n, nrhs, s);
-  if (e != cudaSuccess) return e;
-  const long long nt = (n + RT - 1) / RT;
-  const long long tiles = nt * (nt + 1) / 2;
-  for (int c0 = 0; c0 < nrhs; c0 += RNRHS) {
-    int nc = nrhs - c0 < RNRHS ? nrhs - c0 : RNRHS;
-    (void)launch_pdl(residual_tile_kernel, dim3((unsigned)tiles), dim3(256), 0, s, A, lda, X + (size_t)c0 * ldx, ldx, R + (size_t)c0 * ldr,
-                                                         ldr, n, nc);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
 }
 cudaError_t launch_col_norms2(const double* R, int ldr, const double* B, int ldb, int n, int nrhs, double* out,
                               cudaStream_t s) {
