@@ -29,43 +29,48 @@ __device__ __forceinline__ int dig_field(double x) {         // biased exponent 
   return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff;
 }
 
+// x in units of 2^(E - 62), E = eb - 1022 (the fixed point the digits are cut from), |x| < 2^E;
+// bits below the unit are rounded.  x finite.
+__device__ __forceinline__ long long dig_fix(double x, int eb) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int F = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = (b & 0xfffffffffffffull) | (F ? 0x10000000000000ull : 0ull);
+  const int sh = 9 - (eb - (F ? F : 1));
+  if (sh >= 0) {
+    m <<= sh;
+  } else {
+    const int r = min(-sh, 63);
+    m = (m + (1ull << (r - 1))) >> r;
+  }
+  return ((long long)b < 0) ? (long long)(0ull - m) : (long long)m;
+}
+// the s-th digits of two fixed-point values as a pair of halves.  M must already hold kDigBias
+// (256 at every digit position), which makes the digits come out unsigned, u = d + 256.
+constexpr unsigned long long kDigBias = 0x4020100804020100ull;
+__device__ __forceinline__ uint32_t dig_pair(unsigned long long M0, unsigned long long M1, int s) {
+  const int o = 54 - 9 * s;
+  uint32_t u0 = (uint32_t)(M0 >> o), u1 = (uint32_t)(M1 >> o);
+  if (s > 0) {
+    u0 &= 511u;
+    u1 &= 511u;
+  }
+  // 0x6400 | u is the half 1024 + u (u <= 512); subtracting 1280 leaves d exactly
+  const uint32_t h = 0x64006400u | u0 | (u1 << 16);
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6500)));
+  return *reinterpret_cast<const uint32_t*>(&d);
+}
+
 // The 7 digits of 8 consecutive inner terms v[0..7] of one row, eb[i] = the scale of v[i] as a
 // biased exponent (field(v[i]) <= eb[i]; E = eb - 1022), to dst[s * plane .. + 8) halves (16-byte
 // stores).  Entries are finite.
 __device__ __forceinline__ void dig_split8(const double (&v)[8], const int (&eb)[8], __half* dst, int plane) {
-  // digits come out unsigned (u = d + 256) after adding 256 at every digit position
-  constexpr unsigned long long kBias = 0x4020100804020100ull;
   uint32_t w[kDig][4];
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
-    unsigned long long M[2];
+    const unsigned long long M0 = (unsigned long long)dig_fix(v[2 * p], eb[2 * p]) + kDigBias;
+    const unsigned long long M1 = (unsigned long long)dig_fix(v[2 * p + 1], eb[2 * p + 1]) + kDigBias;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(v[2 * p + q]);
-      const int F = (int)(b >> 52) & 0x7ff;
-      unsigned long long m = (b & 0xfffffffffffffull) | (F ? 0x10000000000000ull : 0ull);
-      const int sh = 9 - (eb[2 * p + q] - (F ? F : 1));      // 62 fractional bits below 2^E
-      if (sh >= 0) {
-        m <<= sh;
-      } else {
-        const int r = min(-sh, 63);
-        m = (m + (1ull << (r - 1))) >> r;
-      }
-      M[q] = (((long long)b < 0) ? 0ull - m : m) + kBias;
-    }
-#pragma unroll
-    for (int s = 0; s < kDig; ++s) {
-      const int o = 54 - 9 * s;
-      uint32_t u0 = (uint32_t)(M[0] >> o), u1 = (uint32_t)(M[1] >> o);
-      if (s > 0) {
-        u0 &= 511u;
-        u1 &= 511u;
-      }
-      // 0x6400 | u is the half 1024 + u (u <= 512); subtracting 1280 leaves d exactly
-      const uint32_t h = 0x64006400u | u0 | (u1 << 16);
-      const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6500)));
-      w[s][p] = *reinterpret_cast<const uint32_t*>(&d);
-    }
+    for (int s = 0; s < kDig; ++s) w[s][p] = dig_pair(M0, M1, s);
   }
 #pragma unroll
   for (int s = 0; s < kDig; ++s)
@@ -158,6 +163,24 @@ __device__ __forceinline__ void dig_scale(int ebx, int eby, double& f0, double& 
   const int e1 = max(-1022, min(1023, e - e0));
   f0 = __longlong_as_double((long long)(e0 + 1023) << 52);
   f1 = __longlong_as_double((long long)(e1 + 1023) << 52);
+}
+
+// a fixed-point value M 2^u (|M| < 2^63) as the nearest double, by integer operations; results
+// outside the normal range go through ldexp
+__device__ __forceinline__ double dig_to_double(long long M, int u) {
+  if (M == 0) return 0.0;
+  const unsigned long long sgn = (unsigned long long)M & 0x8000000000000000ull;
+  unsigned long long a = (unsigned long long)(M < 0 ? -M : M);
+  const int z = __clzll((long long)a);                        // a 2^z in [2^63, 2^64)
+  a <<= z;
+  // leading 53 bits, rounded to nearest even at the 11 below
+  unsigned long long q = a >> 11;
+  const unsigned rest = (unsigned)a & 0x7ffu;
+  q += (rest > 0x400u) | ((rest == 0x400u) & (unsigned)(q & 1));
+  const int e = 63 - z + u;                                   // value in [2^e, 2^(e+1)) (2^(e+1) after a carry)
+  if (e >= -1021 && e <= 1021)
+    return __longlong_as_double((long long)(sgn | (((unsigned long long)(e + 1022) << 52) + q)));
+  return ldexp(sgn ? -(double)q : (double)q, e - 52);
 }
 
 // v 2^e by integer addition to the exponent (the FP64 pipe is the slow one); exact unless the

@@ -236,6 +236,12 @@ void apply_tuned(const hrp_handle* h, hrp_tree* t, int n) {
 // allocation, barrier set-up, pipeline fill); smaller ones stay on the SIMT pipe
 bool split_tc_worth(int m, int n, int k) { return k >= 32 && (double)m * n * k >= 2.0e6; }
 
+// FP64 leaf TRSMs of at least this many columns run by refinement (k_trsm64.cu); narrower ones are
+// a short enough substitution.  Factorizations of order n with leaves of n / 2, refinement against
+// substitution: n = 80 164 / 156 us, 96 100 / 96, 112 113 / 117, 128 125 / 128; n = 1024 with leaf
+// 64 1663 / 2020 us, with leaf 128 1419 / 1860.
+constexpr int kRefineMin = 56;
+
 struct Fact {
   hrp_handle* h;
   const hrp_tree* t;
@@ -246,7 +252,7 @@ struct Fact {
   cudaStream_t s;
   __half* shadow;       // null if no F16 level
   int lds;
-  float* w32;           // null if every level is F64
+  float* w32;           // FP32 inverses of the diagonal leaves (n x 128)
   __half* shadow8;      // null if no F8 level, or if the F8 GEMMs read bytes8
   unsigned char* bytes8 = nullptr;   // E4M3 codes for the block-scaled F8 GEMMs
   int* tile_exp;
@@ -338,7 +344,7 @@ struct Fact {
       return;
     }
     float* W = nullptr;
-    if (w32) {
+    if (w32 && (nb >= kRefineMin || tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || tree_has(t, HRP_F8E4M3))) {
       W = w32 + (size_t)off * 128;
       leaves[off] = nb;
       inv_by[off] = {s, launch_no[s] + 1};
@@ -356,7 +362,12 @@ struct Fact {
     __half* sh = shadow;
     begin(CLS_TRSM, (double)m * nc * nc);
     if (p == HRP_F64 || t->trsm_compute == 1) {
-      chk(launch_trsm_leaf64(Ab, lda, r0, m, c0, nc, sh, lds, shadow32, ld32, info, h->d_err, s));
+      const auto lf = leaves.find(c0);
+      if (w32 && nc >= kRefineMin && lf != leaves.end() && lf->second == nc)
+        chk(launch_trsm_refine64(Ab, lda, r0, m, c0, nc, w32 + (size_t)c0 * 128, 128, sh, lds, shadow32, ld32, info,
+                                 h->d_err, s));
+      else
+        chk(launch_trsm_leaf64(Ab, lda, r0, m, c0, nc, sh, lds, shadow32, ld32, info, h->d_err, s));
       quant8(r0, m, c0, nc, p);
       split_block(r0, m, c0, nc, p);
       return;
@@ -643,7 +654,7 @@ hrp_status potrf_enqueue(hrp_handle* h, const hrp_tree* t, int n, double* dA, in
     f.shadow8 = h->shadow8;
     f.tile_exp = h->tile_exp;
   }
-  if (tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || has8) {
+  if (n > t->leaf) {
     if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128 + 128 * 128)) != HRP_OK) return st;
     f.w32 = h->w32;
   }
@@ -1648,7 +1659,7 @@ hrp_status enqueue_persistent(hrp_handle* h, const std::vector<PSys>& sys, cudaS
       s16 = reinterpret_cast<__half*>(shadow_bytes + 1);
       shadow_bytes += ((size_t)q.n * q.n * sizeof(__half) + 255) / 256 * 256;
     }
-    bs.push_back(BatchSys{q.A, q.lda, q.n, op0, (int)ops.size(), q.info, q.src, q.ldsrc, s32, s16});
+    bs.push_back(BatchSys{q.A, q.lda, q.n, op0, (int)ops.size(), q.info, q.src, q.ldsrc, 0, s32, s16});
   }
   // systems of order 0: info = 0
   for (const PSys& q : sys)
@@ -1768,8 +1779,7 @@ hrp_status hrp_potrf_batched(hrp_handle* h, const hrp_tree* const* trees_in, int
     f.shadow = tree_has(f.t, HRP_F16) ? reinterpret_cast<__half*>(h->bwork + ws[i].shadow) : nullptr;
     f.shadow8 = nullptr;
     f.tile_exp = nullptr;
-    f.w32 = (tree_has(f.t, HRP_F32) || tree_has(f.t, HRP_F16)) ? reinterpret_cast<float*>(h->bwork + ws[i].w32)
-                                                                : nullptr;
+    f.w32 = f.n > f.t->leaf ? reinterpret_cast<float*>(h->bwork + ws[i].w32) : nullptr;
     f.begin(CLS_OTHER, 0.0);
     f.chk(launch_fill_int(f.info, INT_MAX, 1, f.s));
     f.potrf(0, f.n, 0);
@@ -2457,8 +2467,21 @@ struct TrsmRun : Blas3 {
   bool tc;
   int* info;
   int tleaf() const { return t->trsm_leaf ? t->trsm_leaf : t->leaf; }
+  float* w32 = nullptr;                          // FP32 inverses of L's FP64 leaves (n x 128)
+  // the diagonal blocks of the FP64 base cases that run by refinement, in recursion order
+  void leaves(int c0, int nc, int depth, std::vector<std::pair<int, int>>& out) const {
+    if (std::min(m, nc) <= tleaf()) {
+      if ((prec(depth, nc) == HRP_F64 || t->trsm_compute == 1) && nc >= kRefineMin && nc <= 128) out.push_back({c0, nc});
+      return;
+    }
+    const int n1 = split(nc);
+    leaves(c0, n1, depth + 1, out);
+    leaves(c0 + n1, nc - n1, depth + 1, out);
+  }
   void leaf(int c0, int nc, int p) {
-    if (p == HRP_F64 || t->trsm_compute == 1)
+    if ((p == HRP_F64 || t->trsm_compute == 1) && w32 && nc >= kRefineMin && nc <= 128)
+      chk(launch_trsm_refine64(B, ldb, 0, m, c0, nc, w32 + (size_t)c0 * 128, 128, S16, lds, B32, m, info, h->d_err, s, L, ldl));
+    else if (p == HRP_F64 || t->trsm_compute == 1)
       chk(launch_trsm_leaf64(B, ldb, 0, m, c0, nc, S16, lds, B32, m, info, h->d_err, s, L, ldl));
     else
       chk(launch_trsm_leaf32_subst(B, ldb, 0, m, c0, nc, S16, lds, B32, m, info, h->d_err, s, L, ldl));
@@ -2601,6 +2624,21 @@ hrp_status hrp_trsm(hrp_handle* h, const hrp_tree* tree, int m, int n, const dou
     r.B32 = h->shadow32;
     r.L32 = h->shadow32 + (size_t)m * n;
     r.chk(launch_cast_f32(dL, ldl, n, n, h->shadow32 + (size_t)m * n, n, r.s));
+  }
+  std::vector<std::pair<int, int>> lv;
+  r.leaves(0, n, 0, lv);
+  if (!lv.empty()) {                             // all inverses at once, one CTA each
+    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128 + 128 * 128)) != HRP_OK) return st;
+    r.w32 = h->w32;
+    LeafList list;
+    for (size_t i = 0; i < lv.size(); ++i) {
+      list.c0[list.count] = lv[i].first;
+      list.n[list.count++] = lv[i].second;
+      if (list.count == 256 || i + 1 == lv.size()) {
+        r.chk(launch_trtri_leaves(dL, ldl, r.w32, list, r.s));
+        list.count = 0;
+      }
+    }
   }
   r.rec(0, n, 0);
   launch_ctx() = LaunchCtx{};

@@ -105,6 +105,18 @@ cudaError_t launch_trsm_leaf32_subst(double* A, int ld, int r0, int m, int c0, i
                                      __half* shadow16, int lds, float* shadow32, int ld32, const int* info,
                                      unsigned* err, cudaStream_t s, const double* Lm = nullptr, int ldl = 0);
 
+// FP64 leaf TRSM by refinement on the tensor pipe (k_trsm64.cu), nc <= 128, with the FP32 inverse
+// W of the leaf (ldw): the accuracy of FP64 substitution or better; outputs as launch_trsm_leaf64.
+cudaError_t launch_trsm_refine64(double* A, int ld, int r0, int m, int c0, int nc, const float* W, int ldw,
+                                 __half* shadow16, int lds, float* shadow32, int ld32, const int* info, unsigned* err,
+                                 cudaStream_t s, const double* Lm = nullptr, int ldl = 0);
+// FP32 inverses of diagonal blocks of a given lower triangle (a standalone TRSM)
+struct LeafList {
+  int count = 0;
+  int c0[256], n[256];
+};
+cudaError_t launch_trtri_leaves(const double* Lm, int ldl, float* W, const LeafList& list, cudaStream_t s);
+
 // ---------------- SIMT GEMM (k_gemm_simt.cu) ----------------
 // C[m x n] -= X[m x k] * Y[n x k]^T, all FP64 column-major views of the master, with
 // operands rounded per `rnd` and accumulated in FP64 (rnd == F64) or FP32.  lower: C is a
@@ -299,6 +311,7 @@ struct BatchSys {
   int* info;          // device int: 0 or the failing column
   const double* src;  // when non-null, A's lower triangle is first copied from src (ldsrc)
   int ldsrc;
+  int pad;            // explicit (0): the struct's bytes are part of the key of a batch's plan
   float* s32;         // FP32 and FP16 copies of the finished off-diagonal entries (column-
   __half* s16;        // major, leading dimension n), read by the FP32 and FP16 GEMMs; null
                       // when the system's tree has neither precision

@@ -529,7 +529,44 @@ trsm_inv32_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int nc,
   }
 }
 
+// FP32 inverses of independent diagonal blocks of a lower triangle Lm, one CTA per block: block b
+// (order n[b] <= 128 at offset c0[b]) to W + 128 c0[b], column-major with leading dimension 128,
+// zeros above the diagonal.
+__global__ void __launch_bounds__(256, 1)
+trtri_leaves_kernel(const double* __restrict__ Lm, int ldl, float* __restrict__ W, const __grid_constant__ LeafList list) {
+  pdl_wait();
+  pdl_trigger();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* Lf = reinterpret_cast<float*>(smem_raw);
+  float* Wt = Lf + 128 * kInvLD;
+  const int c0 = list.c0[blockIdx.x], n = list.n[blockIdx.x];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nb32 = ((n + 31) / 32) * 32;
+  for (int j = warp; j < nb32; j += 8)
+    for (int i = lane; i < nb32; i += 32)
+      Lf[j * kInvLD + i] = (i < n && j < n && i >= j) ? (float)Lm[(size_t)(c0 + j) * ldl + c0 + i] : 0.f;
+  __syncthreads();
+  trtri32_blocked(Lf, Wt, n);
+  float* Wb = W + (size_t)c0 * 128;
+  for (int j = warp; j < n; j += 8)
+    for (int i = lane; i < n; i += 32) Wb[(size_t)j * 128 + i] = (i >= j) ? Wt[j * kInvLD + i] : 0.f;
+}
+
 }  // namespace
+
+cudaError_t launch_trtri_leaves(const double* Lm, int ldl, float* W, const LeafList& list, cudaStream_t s) {
+  if (list.count <= 0) return cudaSuccess;
+  const int smem = 2 * 128 * kInvLD * 4;
+  static unsigned long long attr_mask = 0;
+  const unsigned long long attr_bit = dev_bit();
+  if (!(attr_mask & attr_bit)) {
+    cudaError_t e = cudaFuncSetAttribute(trtri_leaves_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    attr_mask |= attr_bit;
+  }
+  (void)launch_pdl(trtri_leaves_kernel, dim3(list.count), dim3(256), smem, s, Lm, ldl, W, list);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_potrf_leaf(double* A, int ld, int n, int col0, bool compute64, bool round16,
                               float* W32, int ldw, int* info, unsigned* err, cudaStream_t s) {

@@ -70,12 +70,12 @@ residual_prologue_kernel(const double* __restrict__ A, int lda, const double* __
     if (in) R[(size_t)c * ldr + gi] = B[(size_t)c * ldb + gi];
     const int F = dig_field(v[q]);
     bad |= F == 0x7ff;
-    if (v[q] != 0.0) mx = max(mx, max(F, 1) + se[r0 + q]);
+    if (__double_as_longlong(v[q]) << 1) mx = max(mx, max(F, 1) + se[r0 + q]);
   }
   atomicMax(&top[c], mx);
   bad = __syncthreads_or(bad);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) eb[q] = v[q] != 0.0 ? top[c] - se[r0 + q] : 1;
+  for (int q = 0; q < 8; ++q) eb[q] = (__double_as_longlong(v[q]) << 1) ? top[c] - se[r0 + q] : 1;
   if (!bad) dig_split8(v, eb, dx + (size_t)c * kLd + r0, kResRhs * kLd);
   if (tid < kResRhs) xs[blk * kResRhs + tid] = top[tid];
   if (tid == 0) flag[blk] = bad;
@@ -219,7 +219,7 @@ residual_tile_kernel(const double* __restrict__ A, int lda, const double* __rest
       if (c >= nrhs || row >= n) continue;
       const int sh = (((j >> 1) & 1) ? e1 : e0) + 1 + xs[kb * kResRhs + c] - 1022 - 34;
       const double v = dig_shift(dig_value(iacc, j), sh);
-      if (v != 0.0) atomicAdd(R + (size_t)c * ldr + row, -v);
+      if (__double_as_longlong(v) << 1) atomicAdd(R + (size_t)c * ldr + row, -v);
     }
   }
 }
