@@ -177,16 +177,16 @@ hrp_status hrp_potrf_host(hrp_handle* h, const hrp_tree* tree, int n, const doub
 
 /*
  * Arithmetic of the FP64 leaves (Alg. 1 base case, the 128 x 128 leaf on an 8-CTA cluster).
- * The leaf's pivot chains, TRSM substitutions and rank-16 updates lie on the critical path of
- * the whole factorization, and FP64 operations take ~64 cycles on this GPU.
- *   mode 1: the leaf runs in double-float arithmetic (pairs of binary32, Dekker 1971; about
- *     48 significant bits, relative error of each operation a few units of 2^-48) on the FP32
- *     pipe.  The leaf is scaled by a power of two and converted exactly (hi) and to 2^-48
- *     (lo) from FP64 on load, and L is rounded back to FP64 on store.  A leaf with an entry
- *     that is not finite, or a diagonal entry or pivot that is not positive or falls below
- *     2^-36 times its largest diagonal entry, is factored again by the FP64 schedule in the
- *     same launch (bitwise the mode-0 result; a failing column is reported as in mode 0).
- *   mode 0: the leaf in FP64.
+ * A leaf is first factored in binary32 and refined to FP64 accuracy with exact residuals (its
+ * error against 64 bits is below a direct FP64 factorization's).  A leaf that cannot be refined (a
+ * pivot that is not positive in binary32, an entry that is not finite or above
+ * sqrt(a_ii a_jj), a condition number above about 10^5) is factored directly, in the same launch:
+ *   mode 1: in double-float arithmetic (pairs of binary32, Dekker 1971; about 48 significant bits,
+ *     relative error of each operation a few units of 2^-48) on the FP32 pipe, and again in FP64
+ *     where an entry that is not finite, or a diagonal entry or pivot that is not positive or falls
+ *     below 2^-36 times the largest diagonal entry, is met (a failing column is reported as in
+ *     mode 0).
+ *   mode 0: in FP64.
  *   mode -1 (default): mode 1 for trees with a level below FP64, mode 0 for all-FP64 trees.
  * Applies to hrp_potrf, hrp_potrf_async, hrp_posv and the stream-pool batched calls.
  */

@@ -253,6 +253,7 @@ struct Fact {
   __half* shadow;       // null if no F16 level
   int lds;
   float* w32;           // FP32 inverses of the diagonal leaves (n x 128)
+  float* scratch = nullptr;   // kLeafScratch floats for the leaves' refinement
   __half* shadow8;      // null if no F8 level, or if the F8 GEMMs read bytes8
   unsigned char* bytes8 = nullptr;   // E4M3 codes for the block-scaled F8 GEMMs
   int* tile_exp;
@@ -344,13 +345,14 @@ struct Fact {
       return;
     }
     float* W = nullptr;
-    if (w32 && (nb >= kRefineMin || tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || tree_has(t, HRP_F8E4M3))) {
+    if (w32 && nb < n && (nb >= kRefineMin || tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || tree_has(t, HRP_F8E4M3))) {
       W = w32 + (size_t)off * 128;
       leaves[off] = nb;
       inv_by[off] = {s, launch_no[s] + 1};
     }
     begin(CLS_POTRF, (double)nb * nb * nb / 3.0);
-    chk(launch_potrf_leaf(A + (size_t)off * lda + off, lda, nb, off, p == HRP_F64, p == HRP_F16, W, 128, info, h->d_err, s));
+    chk(launch_potrf_leaf(A + (size_t)off * lda + off, lda, nb, off, p == HRP_F64, p == HRP_F16, W, 128, info, h->d_err,
+                          scratch, s));
   }
 
   void leaf_trsm(int r0, int m, int c0, int nc, int p) {
@@ -654,9 +656,10 @@ hrp_status potrf_enqueue(hrp_handle* h, const hrp_tree* t, int n, double* dA, in
     f.shadow8 = h->shadow8;
     f.tile_exp = h->tile_exp;
   }
-  if (n > t->leaf) {
-    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128 + 128 * 128)) != HRP_OK) return st;
+  if (n > 0) {
+    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128 + kLeafScratch)) != HRP_OK) return st;
     f.w32 = h->w32;
+    f.scratch = h->w32 + (size_t)n * 128;
   }
   f.shadow32 = nullptr;
   f.ld32 = n;
@@ -1529,7 +1532,7 @@ hrp_status batch_prepare(hrp_handle* h, int batch, const int* n, std::vector<Sys
     SysWork& w = ws[i];
     w.lds = (ni + 63) / 64 * 64;
     w.shadow = need_factor_ws ? take((size_t)ni * w.lds * sizeof(__half)) : 0;
-    w.w32 = need_factor_ws ? take(((size_t)ni * 128 + 128 * 128) * sizeof(float)) : 0;
+    w.w32 = need_factor_ws ? take(((size_t)ni * 128 + kLeafScratch) * sizeof(float)) : 0;
     w.pinv = take(potrs_workspace_bytes(ni));
     w.ticket = take(sizeof(int));
     w.fact = nrhs_ir ? take(sizeof(double) * (size_t)ni * ni) : 0;
@@ -1779,7 +1782,8 @@ hrp_status hrp_potrf_batched(hrp_handle* h, const hrp_tree* const* trees_in, int
     f.shadow = tree_has(f.t, HRP_F16) ? reinterpret_cast<__half*>(h->bwork + ws[i].shadow) : nullptr;
     f.shadow8 = nullptr;
     f.tile_exp = nullptr;
-    f.w32 = f.n > f.t->leaf ? reinterpret_cast<float*>(h->bwork + ws[i].w32) : nullptr;
+    f.w32 = reinterpret_cast<float*>(h->bwork + ws[i].w32);
+    f.scratch = f.w32 + (size_t)f.n * 128;
     f.begin(CLS_OTHER, 0.0);
     f.chk(launch_fill_int(f.info, INT_MAX, 1, f.s));
     f.potrf(0, f.n, 0);
@@ -2215,6 +2219,7 @@ extern "C" hrp_status hrp_posv_batched(hrp_handle* h, const hrp_tree* const* tre
       f.lds = ws[i].lds;
       f.shadow = tree_has(f.t, HRP_F16) ? reinterpret_cast<__half*>(h->bwork + ws[i].shadow) : nullptr;
       f.w32 = reinterpret_cast<float*>(h->bwork + ws[i].w32);
+      f.scratch = f.w32 + (size_t)n[i] * 128;
       f.begin(CLS_OTHER, 0.0);
       f.chk(launch_fill_int(f.info, INT_MAX, 1, si));
       f.potrf(0, n[i], 0);
@@ -2320,6 +2325,7 @@ extern "C" hrp_status hrp_posv_batched(hrp_handle* h, const hrp_tree* const* tre
         f.lds = ws[i].lds;
         f.shadow = nullptr;
         f.w32 = reinterpret_cast<float*>(h->bwork + ws[i].w32);
+        f.scratch = f.w32 + (size_t)n[i] * 128;
         f.begin(CLS_OTHER, 0.0);
         f.chk(launch_fill_int(f.info, INT_MAX, 1, si));
         f.potrf(0, n[i], 0);
@@ -2628,7 +2634,7 @@ hrp_status hrp_trsm(hrp_handle* h, const hrp_tree* tree, int m, int n, const dou
   std::vector<std::pair<int, int>> lv;
   r.leaves(0, n, 0, lv);
   if (!lv.empty()) {                             // all inverses at once, one CTA each
-    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128 + 128 * 128)) != HRP_OK) return st;
+    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128)) != HRP_OK) return st;
     r.w32 = h->w32;
     LeafList list;
     for (size_t i = 0; i < lv.size(); ++i) {

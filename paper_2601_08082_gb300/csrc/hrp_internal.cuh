@@ -76,13 +76,16 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // 1-based global column (col0 + k + 1) of the first failing pivot (INT_MAX = none).
 // err: device status word; an F16 leaf whose input or factor exceeds kF16Max sets
 // DEV_ERR_RANGE16.
+// scratch: kLeafScratch floats of device memory, 16-byte aligned, for the FP64 leaves' refinement (no
+// initial contents needed; calls that may overlap need one each), or nullptr to do without it.
+constexpr int kLeafScratch = 2 * 36 * 256;
 cudaError_t launch_potrf_leaf(double* A, int ld, int n, int col0, bool compute64, bool round16,
-                              float* W32, int ldw, int* info, unsigned* err, cudaStream_t s);
+                              float* W32, int ldw, int* info, unsigned* err, float* scratch, cudaStream_t s);
 
 // The same FP64 leaf POTRF (no FP16 rounding) on a cluster of 8 CTAs holding 16 x 16
 // tiles in shared memory (k_leaf_cluster.cu); launch_potrf_leaf uses it for n > 32.
 cudaError_t launch_potrf_leaf_cluster(double* A, int ld, int n, int col0, float* W32, int ldw, int* info,
-                                      cudaStream_t s);
+                                      float* scratch, cudaStream_t s);
 
 // Leaf TRSM B <- B L^{-T} with B = A[r0.., c0..] (m x nc) and L = A[c0.., c0..] (nc x nc),
 // in FP64 by substitution.  shadow16 (row-major, lds) receives FP16(X) and shadow32

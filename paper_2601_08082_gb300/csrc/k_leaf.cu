@@ -568,11 +568,15 @@ cudaError_t launch_trtri_leaves(const double* Lm, int ldl, float* W, const LeafL
   return cudaGetLastError();
 }
 
+// FP64 leaves above this order run on the cluster (refinement, k_leaf_cluster.cu); below it the
+// single CTA's register schedule is as fast (order 7: 30 us)
+constexpr int kLeafClusterMin = 8;
+
 cudaError_t launch_potrf_leaf(double* A, int ld, int n, int col0, bool compute64, bool round16,
-                              float* W32, int ldw, int* info, unsigned* err, cudaStream_t s) {
+                              float* W32, int ldw, int* info, unsigned* err, float* scratch, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (n > 128) return cudaErrorInvalidValue;
-  if (compute64 && !round16 && n > 32) return launch_potrf_leaf_cluster(A, ld, n, col0, W32, ldw, info, s);
+  if (compute64 && !round16 && n > kLeafClusterMin) return launch_potrf_leaf_cluster(A, ld, n, col0, W32, ldw, info, scratch, s);
   const size_t smem = W32 ? (size_t)2 * 128 * kInvLD * 4 : 0;
   static unsigned long long attr_mask = 0;     // one opt-in to the largest footprint (n = 128, with W)
   const unsigned long long attr_bit = dev_bit();

@@ -1,5 +1,9 @@
-// Leaf POTRF (Alg. 1 base case) spread over a cluster of 8 CTAs, in FP64 or in
-// double-float arithmetic on the FP32 pipe.
+// Leaf POTRF (Alg. 1 base case) spread over a cluster of 8 CTAs: by refinement of a binary32
+// factor (leaf_refine.cuh), and, for the leaves that cannot be refined, by the direct schedules
+// below in FP64 or in double-float arithmetic on the FP32 pipe.
+//
+// Order 128, one leaf alone in a call with copy and info kernels: 95 us (FP64 schedule) and 60 us
+// (double-float) -> 47 us refined, 68 us for kernel matrices that take a third and fourth step.
 //
 // FP64 on this GPU: each SM sub-partition issues one FP64 warp instruction per ~64
 // cycles (also the dependent latency), the SM as a whole about one per 19 cycles
@@ -49,6 +53,7 @@
 #include <type_traits>
 
 #include "hrp_internal.cuh"
+#include "leaf_refine.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -903,10 +908,14 @@ __device__ int leaf_body(double* __restrict__ A, int ld, int n, int col0, float*
 
 __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCThreads, 1)
 potrf_leaf_cluster_kernel(double* __restrict__ A, int ld, int n, int col0, float* __restrict__ W32, int ldw,
-                          int* __restrict__ info, int df) {
+                          int* __restrict__ info, int df, float* scratch) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  // an earlier block failed: stop like LAPACK (every CTA reads the same value: nothing in this
+  // kernel writes info before a cluster barrier)
+  if (*(volatile int*)info != INT_MAX) return;
+  if (scratch != nullptr && leafref::leaf_refine(A, ld, n, W32, ldw, scratch, smem_raw)) return;
   if (df) {
     if (leaf_body<dfloat>(A, ld, n, col0, W32, ldw, info, smem_raw) != kFallback) return;
     cg::this_cluster().sync();          // every CTA has left the double-float attempt
@@ -914,22 +923,28 @@ potrf_leaf_cluster_kernel(double* __restrict__ A, int ld, int n, int col0, float
   (void)leaf_body<double>(A, ld, n, col0, W32, ldw, info, smem_raw);
 }
 
+constexpr size_t kLeafSmem =
+    sizeof(LeafSmem<double>) > sizeof(leafref::Smem) ? sizeof(LeafSmem<double>) : sizeof(leafref::Smem);
+static_assert(kLeafSmem <= 227 * 1024, "shared memory of one CTA");
+static_assert(leafref::kScratch == kLeafScratch, "scratch of the callers");
+static_assert(leafref::kThreads == kCThreads && leafref::kCtas == kCL, "one launch shape");
+
 }  // namespace
 
 cudaError_t launch_potrf_leaf_cluster(double* A, int ld, int n, int col0, float* W32, int ldw, int* info,
-                                      cudaStream_t s) {
+                                      float* scratch, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (n > 128) return cudaErrorInvalidValue;
   static unsigned long long attr_mask = 0;
   const unsigned long long attr_bit = dev_bit();
   if (!(attr_mask & attr_bit)) {
     cudaError_t e = cudaFuncSetAttribute(potrf_leaf_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(LeafSmem<double>));
+                                         (int)kLeafSmem);
     if (e != cudaSuccess) return e;
     attr_mask |= attr_bit;
   }
-  (void)launch_pdl(potrf_leaf_cluster_kernel, dim3(kCL), dim3(kCThreads), sizeof(LeafSmem<double>), s, A, ld, n, col0,
-                   W32, ldw, info, launch_ctx().leaf_df ? 1 : 0);
+  (void)launch_pdl(potrf_leaf_cluster_kernel, dim3(kCL), dim3(kCThreads), kLeafSmem, s, A, ld, n, col0,
+                   W32, ldw, info, launch_ctx().leaf_df ? 1 : 0, scratch);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,879 @@
+// The leaf POTRF by refinement: an FP32 Cholesky corrected to FP64 accuracy with exact residuals
+// (used by potrf_leaf_cluster_kernel before its direct schedules, see there).
+//
+// The direct schedules of k_leaf_cluster.cu carry the accuracy of the result through all 128
+// pivots, in FP64 (~820 cycles a column) or in pairs of binary32 (~420).  Here the chain runs in
+// plain binary32 (about 60 cycles a column, one warp, two columns at a time) and the digits come
+// afterwards, from products:
+//   L0 = chol_32(A), W0 = L0^{-1}                       binary32, every CTA of the cluster the same
+//   repeat  R  = A - L L^T                              exact (digit products, digits.cuh)
+//           E  = W0 R W0^T,  F = its lower triangle with half the diagonal
+//           L += L0 F                                   binary16 pairs (22 bits) on the tensor pipe
+// (L (I + F) (I + F)^T L^T = A to first order in F.)  Each step multiplies the error by the relative
+// error of L0 and W0, about 2^-21 for the leaves of dominant matrices, so two steps pass FP64's
+// unit roundoff; the loop stops when the next error is below 2^-57.  L is held in 62-bit fixed
+// point against the scales 2^e_i, e_i = ceil(ex_i / 2) for a_ii < 2^ex_i, so that |l_ij| < 2^e_i
+// exactly, whatever the range of A (the fixed point keeps one more bit for binary32's rounding).
+//
+// Work split: the 36 residual tiles (I, J) belong to CTA (I + J) mod 8; the corrections of column
+// block J to CTA J.  Every CTA needs all residuals and all corrections; they are exchanged through
+// a scratch array in global memory (36 KB each, L2 resident; distributed shared memory was
+// measured at ~9 bytes per clock and SM for this all-to-all pattern), two cluster barriers a step;
+// nothing else waits.
+//
+// A leaf whose diagonal is not positive, with |a_ij| > sqrt(a_ii a_jj), a binary32 pivot that is not
+// positive, or that does not converge (condition number above ~10^5) is left untouched and
+// factored by the direct schedules in the same launch.
+#pragma once
+#include <cooperative_groups.h>
+
+#include "digits.cuh"
+#include "hrp_internal.cuh"
+
+namespace hrp {
+namespace leafref {
+
+namespace cg = cooperative_groups;
+
+constexpr int kThreads = 256;
+constexpr int kCtas = 8;
+constexpr int kTiles = 36;
+constexpr int kTtLd = 136;             // halves per row of the staged column block
+constexpr int kMaxStep = 6;
+constexpr float kTol = 0x1p-57f;
+
+struct Smem {
+  unsigned long long Lx[kTiles][256];  // L in units of 2^(e_i - 62) plus kByteBias, rows swizzled
+  union {
+    float f[kTiles][256];              // binary32 tiles not yet eliminated, row-major with ft()
+    __half h[kTiles][2][256];          // L0 as binary16 pairs hi + lo 2^-11, row-major with ht()
+  } L0;
+  __half W0[kTiles][2][256];           // L0^{-1}, pairs
+  __half R[kTiles][2][256];            // R (lower tiles), scaled, pairs
+  __half Tt[2][16][kTtLd];             // T = R W0_J^T, then F, transposed: [column][row]; rows of H
+  float Wrow[16][132];                 // rows 16 rank .. of the inverse, binary32
+  __half Sbuf[12][2][256];             // phase 1: sums for the off-diagonal blocks of W0, pairs
+  float4 xy[16][16];                   // phase 1: the diagonal block's column pairs, rows 2 j, 2 j + 1
+  float4 rr[16];                       // phase 1: 1 / l_kk, 1 / l_{k+1,k+1}, l_{k+1,k} of a pair
+  int e[128];                          // scales
+  unsigned char tI[kTiles], tJ[kTiles];   // row and column of each lower tile
+  unsigned rmax[2], emax[2];           // largest |R| and scaled |E| here (bits), by step parity
+};
+
+// Digits of 8 bits: byte s of a fixed-point value with kByteBias (128 at every byte) added is d + 128,
+// weight 2^(8 (7 - s)); a pair of digits takes a byte permutation, a mask and a subtraction, less
+// than half of digits.cuh's 9-bit ones, which matters here where every value is split once per use.
+// Eight digits, weights s + t <= 7 kept; a product of 128 terms sums to at most 8 x 128 x 2^14 =
+// 2^24 per weight, exact in binary32 without intermediate moves.
+constexpr unsigned long long kByteBias = 0x8080808080808080ull;
+// digits s of M0 and M1 as a pair of halves
+__device__ __forceinline__ uint32_t byte_pair(unsigned long long M0, unsigned long long M1, int s) {
+  const int byte = 7 - s;                // from the low end
+  const uint32_t w0 = byte >= 4 ? (uint32_t)(M0 >> 32) : (uint32_t)M0, w1 = byte >= 4 ? (uint32_t)(M1 >> 32) : (uint32_t)M1;
+  const uint32_t b = byte & 3;
+  const uint32_t x = (__byte_perm(w0, w1, b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12)) & 0x00ff00ffu) | 0x64006400u;
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&x), __half2half2(__ushort_as_half(0x6480)));   // 1152
+  return *reinterpret_cast<const uint32_t*>(&d);
+}
+
+__device__ __forceinline__ int tix(int I, int J) { return I * (I + 1) / 2 + J; }
+// element (i, j) of a binary32 tile: 16-byte groups swizzled so that 8 rows read without conflicts
+__device__ __forceinline__ int ft(int i, int j) { return i * 16 + ((((j >> 2) ^ (i >> 1)) & 3) << 2) + (j & 3); }
+// element (i, j) of a binary16 tile: the two 16-byte halves of a row swapped on rows 4-7 and 12-15
+__device__ __forceinline__ int ht(int i, int j) { return i * 16 + ((((j >> 3) ^ (i >> 2)) & 1) << 3) + (j & 7); }
+// element (i, k) of a fixed-point tile: halves of a row swapped on odd rows
+__device__ __forceinline__ int lx(int i, int k) { return i * 16 + (k ^ ((i & 1) << 3)); }
+
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// x as hi + lo 2^-11, both binary16 (22 bits of x; lo keeps binary16's normal range)
+__device__ __forceinline__ void half_pair(float x, __half& hi, __half& lo) {
+  hi = __float2half_rn(x);
+  lo = __float2half_rn((x - __half2float(hi)) * 2048.f);
+}
+__device__ __forceinline__ void half_pair2(float2 x, __half2& hi, __half2& lo) {
+  hi = __float22half2_rn(x);
+  const float2 b = __half22float2(hi);
+  lo = __float22half2_rn(make_float2((x.x - b.x) * 2048.f, (x.y - b.y) * 2048.f));
+}
+// x (|x| < 1 up to rounding) in units of 2^-62, truncated
+__device__ __forceinline__ unsigned long long fix62(float x) {
+  const unsigned b = __float_as_uint(x);
+  const int F = (int)(b >> 23) & 0xff, sh = F - 88;          // x = m 2^(F - 150)
+  const long long m = F ? (long long)((b & 0x7fffffu) | 0x800000u) : 0;
+  const long long M = sh >= 0 ? m << min(sh, 39) : (sh > -24 ? m >> -sh : 0);
+  return (unsigned long long)((int)b < 0 ? -M : M);
+}
+
+// fragments of a 16 x 16 binary16 tile: as the A operand (rows x terms), its transpose as A, as the B
+// operand (columns x terms), its transpose as B
+enum class Op { A, At, B, Bt };
+template <Op O>
+__device__ __forceinline__ void frag(uint32_t (&r)[4], const __half* t, int lane) {
+  if constexpr (O == Op::A) {
+    const int i = lane & 15;
+    dig_ldmatrix(r, t + ht(i, (lane >> 4) * 8));
+  } else if constexpr (O == Op::At) {
+    const int i = ((lane >> 4) & 1) * 8 + (lane & 7);
+    dig_ldmatrix_t(r, t + ht(i, ((lane >> 3) & 1) * 8));
+  } else if constexpr (O == Op::B) {
+    const int i = (lane & 7) + ((lane >> 4) << 3);
+    dig_ldmatrix(r, t + ht(i, ((lane >> 3) & 1) * 8));
+  } else {
+    const int i = ((lane >> 3) & 1) * 8 + (lane & 7);
+    dig_ldmatrix_t(r, t + ht(i, (lane >> 4) * 8));
+  }
+}
+// acc0 += hi hi, acc1 += hi lo + lo hi (weight 2^-11) for a 16 x 16 output and 16 terms
+__device__ __forceinline__ void pair_mm(float (&acc0)[2][4], float (&acc1)[2][4], const uint32_t (&ah)[4],
+                                        const uint32_t (&al)[4], const uint32_t (&bh)[4], const uint32_t (&bl)[4]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    dig_mma(acc0[h], ah, bh[2 * h], bh[2 * h + 1]);
+    dig_mma(acc1[h], ah, bl[2 * h], bl[2 * h + 1]);
+    dig_mma(acc1[h], al, bh[2 * h], bh[2 * h + 1]);
+  }
+}
+// the value of a pair product
+__device__ __forceinline__ float pair_value(float c0, float c1) { return fmaf(c1, 0x1p-11f, c0); }
+// a warp's 16 x 16 result (scaled by f) as pairs to a tile
+__device__ __forceinline__ void put_pairs(__half (*t)[256], const float (&c0)[2][4], const float (&c1)[2][4], float f,
+                                          int lane) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+      const int i = (lane >> 2) + 4 * q, j = 8 * h + 2 * (lane & 3);
+      __half2 hi, lo;
+      half_pair2(make_float2(f * pair_value(c0[h][q], c1[h][q]), f * pair_value(c0[h][q + 1], c1[h][q + 1])), hi, lo);
+      *reinterpret_cast<__half2*>(t[0] + ht(i, j)) = hi;
+      *reinterpret_cast<__half2*>(t[1] + ht(i, j)) = lo;
+    }
+}
+// A-operand fragments of a binary32 tile, split into pairs in registers
+__device__ __forceinline__ void frag_f32(uint32_t (&ah)[4], uint32_t (&al)[4], const float* t, int lane) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = (lane >> 2) + 8 * (q & 1), j = 2 * (lane & 3) + 8 * (q >> 1);
+    __half2 hi, lo;
+    half_pair2(*reinterpret_cast<const float2*>(t + ft(i, j)), hi, lo);
+    ah[q] = *reinterpret_cast<const uint32_t*>(&hi);
+    al[q] = *reinterpret_cast<const uint32_t*>(&lo);
+  }
+}
+template <Op OA, Op OB>
+__device__ __forceinline__ void tile_pair_mm(float (&c0)[2][4], float (&c1)[2][4], const __half (*A)[256],
+                                             const __half (*B)[256], int lane) {
+  uint32_t ah[4], al[4], bh[4], bl[4];
+  frag<OA>(ah, A[0], lane);
+  frag<OA>(al, A[1], lane);
+  frag<OB>(bh, B[0], lane);
+  frag<OB>(bl, B[1], lane);
+  pair_mm(c0, c1, ah, al, bh, bl);
+}
+
+// Cholesky of the 32 x 32 diagonal block p (tiles 2p, 2p + 1) by warp 0, and its inverse W by warp 1.
+// Warp 0's lane i holds row i; columns two at a time: every lane forms the pair's pivots (both
+// reciprocal square roots at once, 1 / l_11 = l_00 (a_00 a_11 - a_10^2)^{-1/2}), the lanes' entries of
+// the two columns go through shared memory (16-byte broadcast reads; a shuffle costs four issue slots of the
+// sub-partition) and update the rest.  The next pair's 2 x 2 block is fetched before it is needed,
+// so the chain of a pair is one reciprocal square root and one exchange.  Warp 1's lane c holds column
+// c of W and applies the same column pairs to it one step behind, told by named barriers 1 .. 15
+// (one per pair: the producer only arrives).  False (warp 0) when a pivot is not positive and finite;
+// both warps pass every barrier in any case.
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_wait(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ bool potrf32(Smem& sm, int p, int lane) {
+  const unsigned full = 0xffffffffu;
+  const int ti = lane >> 4, ri = lane & 15;
+  float a[32];
+#pragma unroll
+  for (int j4 = 0; j4 < 8; ++j4) {
+    const int tj = j4 >> 2;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tj <= ti) v = *reinterpret_cast<const float4*>(&sm.L0.f[tix(2 * p + ti, 2 * p + tj)][ft(ri, 4 * (j4 & 3))]);
+    a[4 * j4] = v.x;
+    a[4 * j4 + 1] = v.y;
+    a[4 * j4 + 2] = v.z;
+    a[4 * j4 + 3] = v.w;
+  }
+  bool ok = true;
+  float d0 = __shfl_sync(full, a[0], 0), q = __shfl_sync(full, a[0], 1), s = __shfl_sync(full, a[1], 1);
+#pragma unroll
+  for (int k = 0; k < 32; k += 2) {
+    float nd0 = 0.f, nq = 0.f, ns = 0.f;         // the next pair's block before this pair's update
+    if (k + 2 < 32) {
+      nd0 = __shfl_sync(full, a[k + 2], k + 2);
+      nq = __shfl_sync(full, a[k + 2], k + 3);
+      ns = __shfl_sync(full, a[k + 3], k + 3);
+    }
+    const float det = fmaf(s, d0, -q * q);
+    const float r0 = rsqrt_fast(d0), rd = rsqrt_fast(det);
+    ok = ok && d0 > 1e-12f && det > 1e-12f * d0;   // scaled pivots: false for NaN too
+    const float m = q * r0, r1 = d0 * r0 * rd;
+    const float x = a[k] * r0;                   // column k of L (rows >= k)
+    const float y = fmaf(-x, m, a[k + 1]) * r1;  // column k + 1 (rows > k)
+    a[k] = x;
+    a[k + 1] = y;
+    reinterpret_cast<float2*>(sm.xy[k >> 1])[lane] = make_float2(x, y);
+    if (lane == 0) sm.rr[k >> 1] = make_float4(r0, r1, m, 0.f);
+    __syncwarp();
+    if (k < 28) pair_arrive((k >> 1) + 1);       // 15 is the caller's, after the last two pairs
+    if (k + 2 < 32) {
+#pragma unroll
+      for (int j = k + 2; j < 32; j += 2) {
+        const float4 v = sm.xy[k >> 1][j >> 1];  // rows j and j + 1 of the two columns
+        if (j == k + 2) {
+          d0 = fmaf(-v.y, v.y, fmaf(-v.x, v.x, nd0));
+          q = fmaf(-v.w, v.y, fmaf(-v.z, v.x, nq));
+          s = fmaf(-v.w, v.w, fmaf(-v.z, v.z, ns));
+        }
+        a[j] = fmaf(-y, v.y, fmaf(-x, v.x, a[j]));
+        a[j + 1] = fmaf(-y, v.w, fmaf(-x, v.z, a[j + 1]));
+      }
+    }
+  }
+  // L as pairs (zero above the diagonal), in place of the binary32 tiles
+#pragma unroll
+  for (int tj = 0; tj < 2; ++tj) {
+    if (tj > ti) continue;
+    __half (*t)[256] = sm.L0.h[tix(2 * p + ti, 2 * p + tj)];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      __half2 hi[4], lo[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = 16 * tj + 8 * c + 2 * u;
+        half_pair2(make_float2(j <= lane ? a[j] : 0.f, j + 1 <= lane ? a[j + 1] : 0.f), hi[u], lo[u]);
+      }
+      *reinterpret_cast<uint4*>(t[0] + ht(ri, 8 * c)) = *reinterpret_cast<const uint4*>(hi);
+      *reinterpret_cast<uint4*>(t[1] + ht(ri, 8 * c)) = *reinterpret_cast<const uint4*>(lo);
+    }
+  }
+  return ok;
+}
+// warp 1: W = L^{-1} of the block as pairs
+__device__ __forceinline__ void inverse32(Smem& sm, int p, int lane) {
+  float w[32];
+#pragma unroll
+  for (int r = 0; r < 32; ++r) w[r] = r == lane ? 1.f : 0.f;
+#pragma unroll
+  for (int k = 0; k < 32; k += 2) {
+    if (k < 30) pair_wait((k >> 1) + 1);         // barrier 15 covers the last two pairs
+    const float4 rr = sm.rr[k >> 1];
+    w[k] *= rr.x;
+    w[k + 1] = fmaf(-rr.z, w[k], w[k + 1]) * rr.y;
+#pragma unroll
+    for (int j = k + 2; j < 32; j += 2) {
+      const float4 v = sm.xy[k >> 1][j >> 1];
+      w[j] = fmaf(-v.y, w[k + 1], fmaf(-v.x, w[k], w[j]));
+      w[j + 1] = fmaf(-v.w, w[k + 1], fmaf(-v.z, w[k], w[j + 1]));
+    }
+  }
+  const int ti = lane >> 4, ri = lane & 15;
+#pragma unroll
+  for (int r = 0; r < 32; ++r) {
+    const int I = r >> 4;
+    if (ti > I) continue;
+    __half (*t)[256] = sm.W0[tix(2 * p + I, 2 * p + ti)];
+    __half hi, lo;
+    half_pair(w[r], hi, lo);
+    t[0][ht(r & 15, ri)] = hi;
+    t[1][ht(r & 15, ri)] = lo;
+  }
+}
+
+// C (binary32 tile) -= the pair products
+__device__ __forceinline__ void sub_tile(float* C, const float (&c0)[2][4], const float (&c1)[2][4], int lane) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+      float2* o = reinterpret_cast<float2*>(C + ft((lane >> 2) + 4 * q, 8 * h + 2 * (lane & 3)));
+      float2 v = *o;
+      v.x -= pair_value(c0[h][q], c1[h][q]);
+      v.y -= pair_value(c0[h][q + 1], c1[h][q + 1]);
+      *o = v;
+    }
+}
+
+// L0 and W0 of the scaled leaf in L0.f (NB blocks of 32), both as pairs; false when a pivot failed.  Right-looking by blocks of 32 columns; the products run on
+// the tensor pipe from the pairs (22 bits: a little below binary32, which the refinement makes up
+// for; in binary32 FMAs they were bound by shared-memory reads, 36000 of 51000 cycles).
+__device__ __forceinline__ bool factor32(Smem& sm, int NB, int tid) {
+  const int warp = tid >> 5, lane = tid & 31;
+  for (int p = 0; p < NB; ++p) {
+    // the diagonal block's update with panel p - 1
+    if (p > 0) {
+      if (warp < 3) {
+        const int I = 2 * p + (warp > 0), J = 2 * p + (warp == 2);
+        float c0[2][4] = {}, c1[2][4] = {};
+        tile_pair_mm<Op::A, Op::B>(c0, c1, sm.L0.h[tix(I, 2 * p - 2)], sm.L0.h[tix(J, 2 * p - 2)], lane);
+        tile_pair_mm<Op::A, Op::B>(c0, c1, sm.L0.h[tix(I, 2 * p - 1)], sm.L0.h[tix(J, 2 * p - 1)], lane);
+        sub_tile(sm.L0.f[tix(I, J)], c0, c1, lane);
+      }
+      __syncthreads();
+    }
+    int fail = 0;
+    if (warp == 0) {
+      fail = !potrf32(sm, p, lane);
+      pair_arrive(15);
+    } else if (warp == 1) {
+      inverse32(sm, p, lane);
+    } else if (p > 0) {
+      // the other tiles' update with panel p - 1, and the sums S(I, J) = sum_K L(I, K) W(K, J) of
+      // tile rows 2p, 2p + 1
+      int u = 0;
+      for (int J = 2 * p; J < 2 * NB; ++J)
+        for (int I = max(J, 2 * p + 2); I < 2 * NB; ++I)
+          if (u++ % 6 == warp - 2) {
+            float c0[2][4] = {}, c1[2][4] = {};
+            tile_pair_mm<Op::A, Op::B>(c0, c1, sm.L0.h[tix(I, 2 * p - 2)], sm.L0.h[tix(J, 2 * p - 2)], lane);
+            tile_pair_mm<Op::A, Op::B>(c0, c1, sm.L0.h[tix(I, 2 * p - 1)], sm.L0.h[tix(J, 2 * p - 1)], lane);
+            sub_tile(sm.L0.f[tix(I, J)], c0, c1, lane);
+          }
+      for (int h = 0; h < 2; ++h)
+        for (int J = 0; J < 2 * p; ++J)
+          if (u++ % 6 == warp - 2) {
+            float c0[2][4] = {}, c1[2][4] = {};
+            for (int K = J; K < 2 * p; ++K)
+              tile_pair_mm<Op::A, Op::Bt>(c0, c1, sm.L0.h[tix(2 * p + h, K)], sm.W0[tix(K, J)], lane);
+            put_pairs(sm.Sbuf[2 * J + h], c0, c1, 1.f, lane);
+          }
+    }
+    if (__syncthreads_or(fail)) return false;
+    // panel: L(I, 2p), L(I, 2p + 1) = A(I, ..) Wpp^T, a warp per tile row; and the blocks of W left of
+    // the diagonal block, W(I, J) = -sum_K Wpp(I, K) S(K, J)
+    int u = 0;
+    for (int I = 2 * p + 2; I < 2 * NB; ++I)
+      if (u++ % 8 == warp) {
+        float x0[2][4] = {}, x1[2][4] = {}, y0[2][4] = {}, y1[2][4] = {};
+        uint32_t ah[4], al[4], bh[4], bl[4];
+        frag_f32(ah, al, sm.L0.f[tix(I, 2 * p)], lane);
+        frag<Op::B>(bh, sm.W0[tix(2 * p, 2 * p)][0], lane);
+        frag<Op::B>(bl, sm.W0[tix(2 * p, 2 * p)][1], lane);
+        pair_mm(x0, x1, ah, al, bh, bl);
+        frag<Op::B>(bh, sm.W0[tix(2 * p + 1, 2 * p)][0], lane);
+        frag<Op::B>(bl, sm.W0[tix(2 * p + 1, 2 * p)][1], lane);
+        pair_mm(y0, y1, ah, al, bh, bl);
+        frag_f32(ah, al, sm.L0.f[tix(I, 2 * p + 1)], lane);
+        frag<Op::B>(bh, sm.W0[tix(2 * p + 1, 2 * p + 1)][0], lane);
+        frag<Op::B>(bl, sm.W0[tix(2 * p + 1, 2 * p + 1)][1], lane);
+        pair_mm(y0, y1, ah, al, bh, bl);
+        __syncwarp();                                       // every lane has read both tiles
+        put_pairs(sm.L0.h[tix(I, 2 * p)], x0, x1, 1.f, lane);
+        put_pairs(sm.L0.h[tix(I, 2 * p + 1)], y0, y1, 1.f, lane);
+      }
+    for (int J = 0; J < 2 * p; ++J)
+      for (int h = 0; h < 2; ++h)
+        if (u++ % 8 == warp) {
+          float c0[2][4] = {}, c1[2][4] = {};
+          for (int K = 0; K <= h; ++K)
+            tile_pair_mm<Op::A, Op::Bt>(c0, c1, sm.W0[tix(2 * p + h, 2 * p + K)], sm.Sbuf[2 * J + K], lane);
+          put_pairs(sm.W0[tix(2 * p + h, J)], c0, c1, -1.f, lane);
+        }
+    __syncthreads();
+  }
+  return true;
+}
+
+// B fragments of the staged column block (columns x rows 16 k ..), hi or lo plane
+__device__ __forceinline__ void frag_tt(uint32_t (&r)[4], const __half (*t)[kTtLd], int kt, int lane) {
+  dig_ldmatrix(r, &t[(lane & 7) + ((lane >> 4) << 3)][16 * kt + ((lane >> 3) & 1) * 8]);
+}
+// a warp's 16 x 16 result (rows 16 I ..) into the staged column block
+__device__ __forceinline__ void put_tt(Smem& sm, int I, const float (&v)[2][4], int lane) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = 8 * h + 2 * (lane & 3) + (q & 1), r = 16 * I + (lane >> 2) + 8 * (q >> 1);
+      __half hi, lo;
+      half_pair(v[h][q], hi, lo);
+      sm.Tt[0][c][r] = hi;
+      sm.Tt[1][c][r] = lo;
+    }
+}
+
+// sum over the 16 (J + 1) inner terms of L(I, :) L(J, :)^T for one half tile (rows 0 .. 15, columns
+// j0 .. + 7), in units of 2^-60 of the fixed points' scales, modulo 2^64.  ND digits, weights s + t <
+// ND kept: 8 is exact to the fixed point; 6 (an error of 2^-49) is enough for the first residual,
+// whose L carries binary32's error (with 5 the loop takes a third step).
+template <int ND>
+__device__ __forceinline__ void half_tile_product(const Smem& sm, int I, int J, int j0, int lane, long long (&sum)[4]) {
+  float acc[ND][4];
+#pragma unroll
+  for (int w = 0; w < ND; ++w)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[w][q] = 0.f;
+  const int ra = lane >> 2, kk = 2 * (lane & 3);
+  const unsigned long long* la = sm.Lx[tix(I, 0)];
+  const unsigned long long* lb = sm.Lx[tix(J, 0)];
+#pragma unroll 1
+  for (int kt = 0; kt <= J; ++kt, la += 256, lb += 256) {
+    const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(la + lx(ra, kk));
+    const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(la + lx(ra + 8, kk));
+    const ulonglong2 a2 = *reinterpret_cast<const ulonglong2*>(la + lx(ra, kk + 8));
+    const ulonglong2 a3 = *reinterpret_cast<const ulonglong2*>(la + lx(ra + 8, kk + 8));
+    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(lb + lx(j0 + ra, kk));
+    const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(lb + lx(j0 + ra, kk + 8));
+    uint32_t bf[ND][2];
+#pragma unroll
+    for (int s = 0; s < ND; ++s) {
+      bf[s][0] = byte_pair(b0.x, b0.y, s);
+      bf[s][1] = byte_pair(b1.x, b1.y, s);
+    }
+#pragma unroll
+    for (int s = 0; s < ND; ++s) {
+      const uint32_t af[4] = {byte_pair(a0.x, a0.y, s), byte_pair(a1.x, a1.y, s), byte_pair(a2.x, a2.y, s),
+                              byte_pair(a3.x, a3.y, s)};
+#pragma unroll
+      for (int t = 0; t < ND - s; ++t) dig_mma(acc[s + t], af, bf[t][0], bf[t][1]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    // weights 2^(-14 - 8 w): w = 0 .. 2 joined in units of 2^-30, the others of 2^(-14 - 8 (ND - 1))
+    long long hi = 0, lo = 0;
+#pragma unroll
+    for (int w = 0; w < 3; ++w) hi = (hi << 8) + __float2int_rn(acc[w][q]);
+#pragma unroll
+    for (int w = 3; w < ND; ++w) lo = (lo << 8) + __float2int_rn(acc[w][q]);
+    constexpr int kLo = 60 - 14 - 8 * (ND - 1);
+    sum[q] = (hi << 30) + (kLo >= 0 ? lo << (kLo >= 0 ? kLo : 0) : lo >> (kLo < 0 ? -kLo : 0));
+  }
+}
+
+// x 2^e truncated to binary32 (0 below its normal range)
+__device__ __forceinline__ float scaled_float(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int F = ((int)(b >> 52) & 0x7ff) - 1023 + 127 + e;
+  if (F <= 0) return 0.f;
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | ((unsigned)min(F, 254) << 23) | ((unsigned)(b >> 29) & 0x7fffffu));
+}
+
+// the largest of the CTAs' words (bits of non-negative floats)
+__device__ __forceinline__ float cluster_max(cg::cluster_group& cluster, unsigned* w) {
+  unsigned q[kCtas], m = 0;
+#pragma unroll
+  for (int u = 0; u < kCtas; ++u) q[u] = *(volatile unsigned*)cluster.map_shared_rank(w, u);
+#pragma unroll
+  for (int u = 0; u < kCtas; ++u) m = max(m, q[u]);
+  return __uint_as_float(m);
+}
+
+// floats of global scratch the refinement exchanges through: residual tiles, then corrections
+constexpr int kScratch = 2 * kTiles * 256;
+
+// The leaf.  Returns true when A holds L (and W32 its FP32 inverse); false, the same in every CTA,
+// with nothing written, when the direct schedules must factor it.  Every thread of the cluster
+// takes the same path through the cluster barriers.
+__device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __restrict__ W32, int ldw,
+                            float* scratch, unsigned char* smem_raw) {
+  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int NB = (n + 31) / 32, T = 2 * NB, NTL = T * (T + 1) / 2;
+  float* xR = scratch;                        // residual tiles
+  float* xD = scratch + kTiles * 256;         // corrections of L
+
+  // this warp's residual units: half tiles (16 rows, 8 columns) of the CTA's tiles, longest products
+  // first; the tile's entries in fixed point (unit 2^(e_i + e_j - 58)) stay in registers
+  int uI[2] = {-1, -1}, uJ[2] = {0, 0}, uH[2] = {0, 0};
+  {
+    int slot = 0;
+    for (int J = T - 1; J >= 0; --J) {
+      const int I = (rank - J) & 7;
+      if (I < J || I >= T) continue;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int u = 2 * slot + h;
+        if (u == warp) {
+          uI[0] = I;
+          uJ[0] = J;
+          uH[0] = h;
+        } else if (15 - u == warp) {
+          uI[1] = I;
+          uJ[1] = J;
+          uH[1] = h;
+        }
+      }
+      ++slot;
+    }
+  }
+  // ---- load: every lower tile (one entry per thread and tile, all loads in flight), the
+  // diagonal's scales, then scaled binary32 ----
+  int bad = 0;
+  const int li = tid & 15, lk = tid >> 4;
+  double araw[2][4];
+  {
+    double v[kTiles];
+    int t = 0;
+#pragma unroll
+    for (int I = 0; I < 8; ++I)
+#pragma unroll
+      for (int J = 0; J <= I; ++J, ++t) {
+        const int gi = 16 * I + li, gk = 16 * J + lk;
+        v[t] = (gi < n && gk <= gi) ? A[(size_t)gk * ld + gi] : 0.0;
+      }
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int gi = 16 * uI[x] + (lane >> 2) + 8 * (q >> 1), gj = 16 * uJ[x] + 8 * uH[x] + 2 * (lane & 3) + (q & 1);
+        araw[x][q] = (uI[x] >= 0 && gi < n && gj <= gi) ? A[(size_t)gj * ld + gi] : 0.0;
+      }
+    if (tid < 2) sm.rmax[tid] = sm.emax[tid] = 0;
+    if (tid < kTiles) {
+      int I = 0;
+      while ((I + 1) * (I + 2) / 2 <= tid) ++I;
+      sm.tI[tid] = (unsigned char)I;
+      sm.tJ[tid] = (unsigned char)(tid - I * (I + 1) / 2);
+    }
+    if (tid < 128) {
+      int e = 0;
+      if (tid < n) {
+        const long long b = __double_as_longlong(A[(size_t)tid * ld + tid]);
+        const int F = (int)(b >> 52);                          // negative for a negative entry
+        bad = F <= 0 || F >= 0x7ff;
+        e = bad ? 0 : (F - 1022 + 1) >> 1;
+      }
+      sm.e[tid] = e;
+    }
+    if (__syncthreads_or(bad)) return false;
+    t = 0;
+#pragma unroll
+    for (int I = 0; I < 8; ++I) {
+      if (I >= T) break;
+      const int gi = 16 * I + li, ei = sm.e[gi];
+#pragma unroll
+      for (int J = 0; J <= I; ++J) {
+        const int gk = 16 * J + lk, ee = ei + sm.e[gk];
+        const double x = v[I * (I + 1) / 2 + J];
+        // a positive definite leaf has |a_ij| < 2^(e_i + e_j)
+        bad |= dig_field(x) > ee + 1022;
+        float f = scaled_float(x, -ee);
+        if (gi >= n) f = gi == gk ? 0.5f : 0.f;                // rows past n: a unit block of its own
+        sm.L0.f[I * (I + 1) / 2 + J][ft(li, lk)] = f;
+      }
+    }
+  }
+  if (__syncthreads_or(bad)) return false;
+  long long afix[2][4];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    if (uI[x] < 0) continue;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int gi = 16 * uI[x] + (lane >> 2) + 8 * (q >> 1), gj = 16 * uJ[x] + 8 * uH[x] + 2 * (lane & 3) + (q & 1);
+      afix[x][q] = 0;
+      if (gi < n && gj <= gi) afix[x][q] = dig_fix(araw[x][q], sm.e[gi] + sm.e[gj] + 2 + 1022) >> 2;
+      if (gi >= n && gi == gj) afix[x][q] = 1ll << 57;         // 0.5
+    }
+  }
+  if (!factor32(sm, NB, tid)) return false;                    // the same in every CTA
+  // ---- L to fixed point: a lane takes two adjacent columns of a row ----
+  for (int t = warp; t < NTL; t += 8) {
+    const int j = 2 * (lane & 7), ib = lane >> 3;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = 4 * q + ib, at = ht(i, j);
+      const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&sm.L0.h[t][0][at]));
+      const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&sm.L0.h[t][1][at]));
+      *reinterpret_cast<ulonglong2*>(&sm.Lx[t][lx(i, j)]) =
+          make_ulonglong2(fix62(pair_value(hi.x, lo.x)) + kByteBias, fix62(pair_value(hi.y, lo.y)) + kByteBias);
+    }
+  }
+  __syncthreads();
+
+  float first = 1.f, last = 1.f;
+  const bool mine = rank < T;                                  // this CTA's column block exists
+  bool good = false;
+  for (int step = 0; step < kMaxStep; ++step) {
+    // ---- R = A - L L^T: this CTA's tiles, to the scratch ----
+    const int par = step & 1;
+    float mx = 0.f;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      if (uI[x] < 0) continue;
+      const int I = uI[x], J = uJ[x], j0 = 8 * uH[x];
+      long long sum[4];
+      if (step == 0) half_tile_product<6>(sm, I, J, j0, lane, sum);
+      else half_tile_product<8>(sm, I, J, j0, lane, sum);
+      float res[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = (lane >> 2) + 8 * (q >> 1), j = j0 + 2 * (lane & 3) + (q & 1);
+        const long long d = afix[x][q] - sum[q];
+        const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
+        res[q] = fmaf((float)(unsigned)(a >> 32), 0x1p32f, (float)(unsigned)a) * (d < 0 ? -0x1p-58f : 0x1p-58f);
+        if (I == J && j > i) res[q] = 0.f;                     // above the diagonal (mirrored below)
+        mx = fmaxf(mx, fabsf(res[q]));
+      }
+      float* o = xR + tix(I, J) * 256 + (lane >> 2) * 16 + j0 + 2 * (lane & 3);
+      __stcg(reinterpret_cast<float2*>(o), make_float2(res[0], res[1]));
+      __stcg(reinterpret_cast<float2*>(o + 128), make_float2(res[2], res[3]));
+    }
+    {
+      // non-negative floats order as their bits
+      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+      if (lane == 0) atomicMax(&sm.rmax[par], m);
+    }
+    cluster.sync();                                            // B1: the residual tiles are written
+    // ---- all of R, scaled by a power of two, as pairs ----
+    float4 g[9];
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+      const int idx = tid + kThreads * u;
+      g[u] = (idx >> 6) < NTL ? __ldcg(reinterpret_cast<const float4*>(xR) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    mx = cluster_max(cluster, &sm.rmax[par]);
+    // scale 2^s with max |R| 2^s in [0.5, 1)
+    const int xe = max((int)(__float_as_uint(mx) >> 23) & 0xff, 1) - 126;
+    const int s = min(-xe, 100);
+    const float fs = __uint_as_float((unsigned)(s + 127) << 23), fsi = __uint_as_float((unsigned)(127 - s) << 23);
+    if (mx > 0.f) {
+#pragma unroll
+      for (int u = 0; u < 9; ++u) {
+        const int idx = tid + kThreads * u, t = idx >> 6, i = (idx & 63) >> 2, j = 4 * (idx & 3);
+        if (t >= NTL) continue;
+        __half2 h0, l0, h1, l1;
+        half_pair2(make_float2(g[u].x * fs, g[u].y * fs), h0, l0);
+        half_pair2(make_float2(g[u].z * fs, g[u].w * fs), h1, l1);
+        if (sm.tI[t] != sm.tJ[t]) {
+          __half2* p = reinterpret_cast<__half2*>(&sm.R[t][0][ht(i, j)]);
+          p[0] = h0;
+          p[1] = h1;
+          p = reinterpret_cast<__half2*>(&sm.R[t][1][ht(i, j)]);
+          p[0] = l0;
+          p[1] = l1;
+        } else {
+          const __half hi[4] = {__low2half(h0), __high2half(h0), __low2half(h1), __high2half(h1)};
+          const __half lo[4] = {__low2half(l0), __high2half(l0), __low2half(l1), __high2half(l1)};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (j + q <= i) {
+              sm.R[t][0][ht(i, j + q)] = hi[q];
+              sm.R[t][1][ht(i, j + q)] = lo[q];
+              sm.R[t][0][ht(j + q, i)] = hi[q];
+              sm.R[t][1][ht(j + q, i)] = lo[q];
+            }
+        }
+      }
+    }
+    __syncthreads();
+    const int J = rank;
+    const int I = warp;
+    float em = 0.f;
+    float dl[2][4] = {};                                       // this warp's corrections L0 F
+    const bool below = mine && mx > 0.f && I >= J && I < T;
+    if (mine && mx > 0.f) {
+      uint32_t ah[4], al[4], bh[4], bl[4];
+      // T = R W0_J^T, row tile I
+      if (I < T) {
+        float c0[2][4] = {}, c1[2][4] = {};
+        for (int k = 0; k <= J; ++k) {
+          if (k <= I) {
+            frag<Op::A>(ah, sm.R[tix(I, k)][0], lane);
+            frag<Op::A>(al, sm.R[tix(I, k)][1], lane);
+          } else {
+            frag<Op::At>(ah, sm.R[tix(k, I)][0], lane);
+            frag<Op::At>(al, sm.R[tix(k, I)][1], lane);
+          }
+          frag<Op::B>(bh, sm.W0[tix(J, k)][0], lane);
+          frag<Op::B>(bl, sm.W0[tix(J, k)][1], lane);
+          pair_mm(c0, c1, ah, al, bh, bl);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) c0[h][q] = fmaf(c1[h][q], 0x1p-11f, c0[h][q]);
+        put_tt(sm, I, c0, lane);
+      }
+      __syncthreads();
+      // E = W0 T (row tiles I >= J), F: lower triangle with half the diagonal
+      float f0[2][4] = {}, f1[2][4] = {};
+      if (below) {
+        for (int k = 0; k <= I; ++k) {
+          frag<Op::A>(ah, sm.W0[tix(I, k)][0], lane);
+          frag<Op::A>(al, sm.W0[tix(I, k)][1], lane);
+          frag_tt(bh, sm.Tt[0], k, lane);
+          frag_tt(bl, sm.Tt[1], k, lane);
+          pair_mm(f0, f1, ah, al, bh, bl);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float E = fmaf(f1[h][q], 0x1p-11f, f0[h][q]);
+            if (!(fabsf(E) < 1e30f)) em = __uint_as_float(0x7f800000u);   // not finite: gives up
+            em = fmaxf(em, fabsf(E));
+            const int c = 8 * h + 2 * (lane & 3) + (q & 1), r = (lane >> 2) + 8 * (q >> 1);
+            if (I == J) E = r > c ? E : (r == c ? 0.5f * E : 0.f);
+            f0[h][q] = E;
+          }
+      }
+      __syncthreads();
+      if (below) put_tt(sm, I, f0, lane);
+      __syncthreads();
+      // the correction of column block J, L0 F
+      if (below) {
+        float c1[2][4] = {};
+        for (int k = J; k <= I; ++k) {
+          frag<Op::A>(ah, sm.L0.h[tix(I, k)][0], lane);
+          frag<Op::A>(al, sm.L0.h[tix(I, k)][1], lane);
+          frag_tt(bh, sm.Tt[0], k, lane);
+          frag_tt(bl, sm.Tt[1], k, lane);
+          pair_mm(dl, c1, ah, al, bh, bl);
+        }
+        float* o = xD + tix(I, J) * 256 + (lane >> 2) * 16 + 2 * (lane & 3);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int c = 8 * h + 2 * (lane & 3) + (q & 1), r = (lane >> 2) + 8 * (q >> 1);
+            dl[h][q] = (I > J || r >= c) ? fmaf(c1[h][q], 0x1p-11f, dl[h][q]) * fsi : 0.f;
+          }
+          __stcg(reinterpret_cast<float2*>(o + 8 * h), make_float2(dl[h][0], dl[h][1]));
+          __stcg(reinterpret_cast<float2*>(o + 8 * h + 128), make_float2(dl[h][2], dl[h][3]));
+        }
+      }
+    }
+    {
+      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(em));
+      if (lane == 0) atomicMax(&sm.emax[par], m);
+      // the other parity's words were read before the last barrier and are used again after this one
+      if (tid == 0) sm.rmax[par ^ 1] = sm.emax[par ^ 1] = 0;
+    }
+    cluster.sync();                                            // B2: the corrections are written
+    em = cluster_max(cluster, &sm.emax[par]) * fsi;          // the scale is the same in every CTA
+    if (!(em < 0.25f)) break;
+    if (step == 0) first = fmaxf(em, 0x1p-24f);
+    else if (em > 0.25f * last && em > 0x1p-50f) break;
+    last = em;
+    good = em * first <= kTol;
+    if (good) {
+      // no further residual: the last correction goes into this CTA's own columns only
+      if (below) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int c = 8 * h + 2 * (lane & 3) + (q & 1), r = (lane >> 2) + 8 * (q >> 1);
+            sm.Lx[tix(I, J)][lx(r, c)] += fix62(dl[h][q]);
+          }
+      }
+    } else if (mx > 0.f) {
+#pragma unroll
+      for (int u = 0; u < 9; ++u) {
+        const int idx = tid + kThreads * u;
+        g[u] = (idx >> 6) < NTL ? __ldcg(reinterpret_cast<const float4*>(xD) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 9; ++u) {
+        const int idx = tid + kThreads * u, t = idx >> 6, i = (idx & 63) >> 2, j = 4 * (idx & 3);
+        if (t >= NTL) continue;
+        ulonglong2* p = reinterpret_cast<ulonglong2*>(&sm.Lx[t][lx(i, j)]);   // 4 terms stay together
+        ulonglong2 y0 = p[0], y1 = p[1];
+        y0.x += fix62(g[u].x);
+        y0.y += fix62(g[u].y);
+        y1.x += fix62(g[u].z);
+        y1.y += fix62(g[u].w);
+        p[0] = y0;
+        p[1] = y1;
+        if (step == 0 && W32 != nullptr) {                      // for the inverse below, times 2^22
+          __half2* o = reinterpret_cast<__half2*>(&sm.R[t][0][ht(i, j)]);
+          o[0] = __float22half2_rn(make_float2(g[u].x * 0x1p22f, g[u].y * 0x1p22f));
+          o[1] = __float22half2_rn(make_float2(g[u].z * 0x1p22f, g[u].w * 0x1p22f));
+        }
+      }
+    }
+    __syncthreads();
+    if (step == 0 && W32 != nullptr && mine) {
+      // W = W0 + H W0, H = I - W0 L (a Newton step on the inverse), rows 16 rank ..: L = L0 plus the
+      // first correction; every product down to 2^-32, the sums of magnitude 1 start from -I
+      const int C = warp;
+      if (C <= rank) {
+        float c0[2][4] = {}, c1[2][4] = {}, c2[2][4] = {};
+        uint32_t ah[4], al[4], bh[4], bl[4], bd[4];
+        if (C == rank) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if ((lane >> 2) + 8 * (q >> 1) == 8 * h + 2 * (lane & 3) + (q & 1)) c0[h][q] = -1.f;
+        }
+        for (int K = C; K <= rank; ++K) {
+          frag<Op::A>(ah, sm.W0[tix(rank, K)][0], lane);
+          frag<Op::A>(al, sm.W0[tix(rank, K)][1], lane);
+          frag<Op::Bt>(bh, sm.L0.h[tix(K, C)][0], lane);
+          frag<Op::Bt>(bl, sm.L0.h[tix(K, C)][1], lane);
+          pair_mm(c0, c1, ah, al, bh, bl);
+          if (mx > 0.f) frag<Op::Bt>(bd, sm.R[tix(K, C)][0], lane);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            dig_mma(c2[h], al, bl[2 * h], bl[2 * h + 1]);
+            if (mx > 0.f) dig_mma(c2[h], ah, bd[2 * h], bd[2 * h + 1]);
+          }
+        }
+        // -H times 2^16 as one binary16 plane, rows of H
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < 4; q += 2) {
+            const float x0 = fmaf(c2[h][q], 0x1p-22f, pair_value(c0[h][q], c1[h][q])) * -0x1p16f;
+            const float x1 = fmaf(c2[h][q + 1], 0x1p-22f, pair_value(c0[h][q + 1], c1[h][q + 1])) * -0x1p16f;
+            *reinterpret_cast<__half2*>(&sm.Tt[0][(lane >> 2) + 4 * q][16 * C + 8 * h + 2 * (lane & 3)]) =
+                __float22half2_rn(make_float2(x0, x1));
+          }
+      }
+      __syncthreads();
+      if (C <= rank) {
+        float c0[2][4] = {};
+        uint32_t ah[4], bh[4];
+        for (int K = C; K <= rank; ++K) {
+          dig_ldmatrix(ah, &sm.Tt[0][lane & 15][16 * K + (lane >> 4) * 8]);
+          frag<Op::Bt>(bh, sm.W0[tix(K, C)][0], lane);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) dig_mma(c0[h], ah, bh[2 * h], bh[2 * h + 1]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int c = 8 * h + 2 * (lane & 3) + (q & 1), r = (lane >> 2) + 8 * (q >> 1), at = ht(r, c);
+            const float w = pair_value(__half2float(sm.W0[tix(rank, C)][0][at]), __half2float(sm.W0[tix(rank, C)][1][at]));
+            sm.Wrow[r][16 * C + c] = fmaf(c0[h][q], 0x1p-16f, w);
+          }
+      }
+    }
+    __syncthreads();
+    if (good) break;
+  }
+  if (good && mine) {
+    // this CTA's column block of L, and its rows of W
+    const int J = rank, gj = 16 * J + lk;
+#pragma unroll
+    for (int I = 0; I < 8; ++I) {
+      const int gi = 16 * I + li;
+      if (I >= J && I < T && gi < n && gj <= gi)
+        A[(size_t)gj * ld + gi] = dig_to_double((long long)(sm.Lx[tix(I, J)][lx(li, lk)] - kByteBias), sm.e[gi] - 62);
+    }
+    if (W32 != nullptr) {
+      const int gi = 16 * rank + li;
+      if (gi < n)
+        for (int c = lk; c < n; c += 16)
+          W32[(size_t)c * ldw + gi] = c <= gi ? ldexpf(sm.Wrow[li][c], -sm.e[c]) : 0.f;
+    }
+  }
+  cluster.sync();                       // no CTA leaves (or reuses its memory) while others may read it
+  return good;
+}
+
+}  // namespace leafref
+}  // namespace hrp
