@@ -133,10 +133,15 @@ hrp_status hrp_potrf_async(hrp_handle* h, const hrp_tree* tree, int n, double* d
 
 /*
  * Solve A X = B given the factor from hrp_potrf (L in the lower triangle of dL):
- * forward substitution L Y = B, then backward L^T X = Y, in 64-row blocks with FP64
- * storage and sums; each block's 16-term partial products are formed in double-float
- * (a pair of binary32 values, about 2^-44 relative to the sum of |terms| at worst, against
- * about 2^-49 for FP64 arithmetic), which moves them off GB300's slow FP64 pipe.
+ * forward substitution L Y = B, then backward L^T X = Y, with FP64 storage and sums.  Two
+ * ways, both off GB300's slow FP64 pipe:
+ *   - n <= 256, more than 8 right-hand sides, or n > 1024 (one right-hand side: up to 3072):
+ *     with FP64 inverses of the diagonal blocks of up to 512 rows, products exact to 2^-55 of
+ *     the largest term (with several right-hand sides, of the row's times the column's largest);
+ *   - otherwise, and where the device's memory does not hold those inverses (6.3 KB per row):
+ *     in 64-row blocks whose 16-term partial products are formed in double-float (a pair of
+ *     binary32 values, about 2^-44 relative to the sum of |terms| at worst).
+ * Its workspaces for order n are allocated by the first call of that order (capturable after).
  * dB (n x nrhs, ldb >= max(1,n)) is overwritten with X. Asynchronous.
  */
 hrp_status hrp_potrs(hrp_handle* h, int n, int nrhs, const double* dL, int ldl,
@@ -339,7 +344,7 @@ hrp_status hrp_autotune(hrp_handle* h, const hrp_tree* tree, int n, int reps, in
 hrp_status hrp_potrf_batched(hrp_handle* h, const hrp_tree* const* trees, int batch, const int* n,
                              double* const* dA, const int* lda, int* d_info, void* stream);
 /*
- * Batched POTRS (FP64): for each i, dB[i] (n[i] x nrhs, ldb[i]) <- A_i^{-1} dB[i] with the
+ * Batched POTRS (FP64; by block inverses up to n[i] = 256, else double-float): for each i, dB[i] (n[i] x nrhs, ldb[i]) <- A_i^{-1} dB[i] with the
  * factor in the lower triangle of dL[i].  Same stream pool and capture rules as above.
  */
 hrp_status hrp_potrs_batched(hrp_handle* h, int batch, const int* n, double* const* dL, const int* ldl,

@@ -29,20 +29,18 @@ __device__ __forceinline__ int dig_field(double x) {         // biased exponent 
   return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff;
 }
 
-// x in units of 2^(E - 62), E = eb - 1022 (the fixed point the digits are cut from), |x| < 2^E;
-// bits below the unit are rounded.  x finite.
+// x in units of 2^(E - 62), E = eb - 1022 (the fixed point the digits are cut from), |x| < 2^E; bits
+// below the unit are dropped.  x finite.  The significand is placed at the top once and only ever
+// shifted right (its exponent field is at most eb; zero may have any eb), the sign applied by xor and
+// carry.
 __device__ __forceinline__ long long dig_fix(double x, int eb) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int F = (int)(b >> 52) & 0x7ff;
-  unsigned long long m = (b & 0xfffffffffffffull) | (F ? 0x10000000000000ull : 0ull);
-  const int sh = 9 - (eb - (F ? F : 1));
-  if (sh >= 0) {
-    m <<= sh;
-  } else {
-    const int r = min(-sh, 63);
-    m = (m + (1ull << (r - 1))) >> r;
-  }
-  return ((long long)b < 0) ? (long long)(0ull - m) : (long long)m;
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int F = (int)(h >> 20) & 0x7ff;
+  const uint32_t mh = (h & 0xfffffu) | ((uint32_t)min(F, 1) << 20);
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(l, mh, 9) << 32) | (l << 9);
+  const unsigned long long v = m >> min((unsigned)(eb - max(F, 1)), 63u);
+  const long long s = (long long)(int)h >> 63;                 // 0 or -1
+  return (long long)(v ^ (unsigned long long)s) - s;
 }
 // the s-th digits of two fixed-point values as a pair of halves.  M must already hold kDigBias
 // (256 at every digit position), which makes the digits come out unsigned, u = d + 256.
@@ -181,6 +179,23 @@ __device__ __forceinline__ double dig_to_double(long long M, int u) {
   if (e >= -1021 && e <= 1021)
     return __longlong_as_double((long long)(sgn | (((unsigned long long)(e + 1022) << 52) + q)));
   return ldexp(sgn ? -(double)q : (double)q, e - 52);
+}
+
+// Digits of 8 bits: byte s of a fixed-point value with kByteBias (128 at every byte) added is d + 128,
+// weight 2^(8 (7 - s)); a pair of digits takes a byte permutation, a mask and a subtraction, less
+// than half of the 9-bit ones, for kernels where every value is split once per use.  Eight digits,
+// weights s + t <= 7 kept (36 products); a product of 128 terms sums to at most 8 x 128 x 2^14 = 2^24
+// per weight, exact in binary32 without intermediate moves.
+constexpr int kByteDig = 8;
+constexpr unsigned long long kByteBias = 0x8080808080808080ull;
+// digits s of M0 and M1 as a pair of halves
+__device__ __forceinline__ uint32_t byte_pair(unsigned long long M0, unsigned long long M1, int s) {
+  const int byte = 7 - s;                // from the low end
+  const uint32_t w0 = byte >= 4 ? (uint32_t)(M0 >> 32) : (uint32_t)M0, w1 = byte >= 4 ? (uint32_t)(M1 >> 32) : (uint32_t)M1;
+  const uint32_t b = byte & 3;
+  const uint32_t x = (__byte_perm(w0, w1, b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12)) & 0x00ff00ffu) | 0x64006400u;
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&x), __half2half2(__ushort_as_half(0x6480)));   // 1152
+  return *reinterpret_cast<const uint32_t*>(&d);
 }
 
 // v 2^e by integer addition to the exponent (the FP64 pipe is the slow one); exact unless the

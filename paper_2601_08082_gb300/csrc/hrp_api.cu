@@ -59,6 +59,8 @@ struct hrp_handle_s {
   size_t work_cap = 0;
   unsigned char* pwork = nullptr;  // POTRS diagonal-block inverses
   size_t pwork_cap = 0;
+  unsigned char* swork = nullptr;  // block inverses of the solves (k_solve.cu)
+  size_t swork_cap = 0;
   unsigned char* rwork = nullptr;  // scales and digits of the residual's operands
   size_t rwork_cap = 0;
   double* d_norms = nullptr;   // 2 * 64 doubles
@@ -827,6 +829,7 @@ hrp_status hrp_destroy(hrp_handle* h) {
   cudaFree(h->d_norms);
   cudaFree(h->pwork);
   cudaFree(h->rwork);
+  cudaFree(h->swork);
   if (h->h_norms) cudaFreeHost(h->h_norms);
   for (cudaEvent_t e : h->events) cudaEventDestroy(e);
   for (cudaEvent_t e : h->bevents) cudaEventDestroy(e);
@@ -1003,10 +1006,28 @@ hrp_status hrp_potrf(hrp_handle* h, const hrp_tree* tree, int n, double* dA, int
 }
 
 
+// h->swork for the block inverses of order n; false (the sweeps do without) where the device's memory
+// does not hold it
+static bool solve_workspace(hrp_handle* h, int n) {
+  return ensure(h, &h->swork, &h->swork_cap, solve_workspace_bytes(n)) == HRP_OK;
+}
+
+// A solve with the factor in dL.  prepared: h->swork already holds this factor's block inverses
+// (hrp_posv forms them once per factorization).
 static hrp_status potrs_impl(hrp_handle* h, int n, int nrhs, const double* dL, int ldl, double* dB, int ldb,
-                             bool fp32, cudaStream_t s) {
+                             bool fp32, cudaStream_t s, bool prepared = false) {
   hrp_status st;
+  if (n <= 0 || nrhs <= 0) return HRP_OK;
+  // both workspaces whatever the path: after one call of order n, none of that order allocates
   if ((st = ensure(h, &h->pwork, &h->pwork_cap, potrs_workspace_bytes(n))) != HRP_OK) return st;
+  if (prepared || (solve_workspace(h, n) && solve_blocked(n, nrhs))) {
+    cudaError_t e = cudaSuccess;
+    launch_ctx() = LaunchCtx{};
+    if (!prepared) e = launch_solve_inverses(dL, ldl, n, h->swork, s);
+    if (e == cudaSuccess) e = launch_solve(dL, ldl, dB, ldb, n, nrhs, h->swork, s);
+    h->launches += solve_launches(n, nrhs, !prepared);
+    return cuda_status(h, e, "hrp_potrs");
+  }
   cudaError_t e = launch_potrs(dL, ldl, dB, ldb, n, nrhs, fp32, h->pwork, h->d_ticket, h->d_err, s, h->wait_ns);
   h->launches += 1 + potrs_sweeps(nrhs);
   return cuda_status(h, e, "hrp_potrs");
@@ -1032,7 +1053,7 @@ hrp_status hrp_potrs(hrp_handle* h, int n, int nrhs, const double* dL, int ldl, 
 // stop at |g_k| <= gmres_tol * beta or after gmres_restart steps.  Matrix-vector products
 // in FP64 from A's lower triangle.  Synchronous (a few 8-byte reads per step).
 static hrp_status gmres_correction(hrp_handle* h, const double* dA, int lda, int n, const double* r, double* x,
-                                   cudaStream_t s) {
+                                   bool prepared, cudaStream_t s) {
   const int m = h->gmres_restart;
   hrp_status st = ensure(h, &h->kwork, &h->kwork_cap, (size_t)(m + 1) * n + 2 * (size_t)n + 2 * (m + 1));
   if (st != HRP_OK) return st;
@@ -1049,7 +1070,7 @@ static hrp_status gmres_correction(hrp_handle* h, const double* dA, int lda, int
   // v0 = M^{-1} r / beta
   if (e == cudaSuccess) e = cudaMemcpyAsync(V, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return cuda_status(h, e, "gmres");
-  if ((st = potrs_impl(h, n, 1, h->fact, n, V, n, false, s)) != HRP_OK) return st;
+  if ((st = potrs_impl(h, n, 1, h->fact, n, V, n, false, s, prepared)) != HRP_OK) return st;
   e = launch_multi_dot(V, n, 1, V, n, hd, s);
   sync_read(1);
   if (e != cudaSuccess) return cuda_status(h, e, "gmres");
@@ -1066,7 +1087,7 @@ static hrp_status gmres_correction(hrp_handle* h, const double* dA, int lda, int
     e = launch_residual(dA, lda, vk, n, zero, n, w, n, n, 1, h->rwork, s);
     if (e == cudaSuccess) e = launch_scale(w, w, -1.0, n, false, s);
     if (e != cudaSuccess) break;
-    if ((st = potrs_impl(h, n, 1, h->fact, n, w, n, false, s)) != HRP_OK) return st;
+    if ((st = potrs_impl(h, n, 1, h->fact, n, w, n, false, s, prepared)) != HRP_OK) return st;
     for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
       e = launch_multi_dot(V, n, k + 1, w, n, hd, s);
       if (e == cudaSuccess) e = launch_gemv_sub(w, V, n, k + 1, hd, n, s);
@@ -1171,9 +1192,18 @@ hrp_status hrp_posv(hrp_handle* h, const hrp_tree* tree, int n, int nrhs, const 
     if ((st = check_dev_err(h, s)) == HRP_ERR_RANGE && attempt == 0) continue;
     if (st != HRP_OK) return st;
     if (hinfo) continue;
-    // X0 = POTRS(B) in FP32
+    // the inverses of the diagonal blocks serve all solves with this factor: from n = 128 to 8192, 1 to
+    // 16 right-hand sides, one correction, no slower than FP32 sweeps anywhere (one right-hand side:
+    // n = 200 330 -> 308 us a call, 1024 892 -> 851, 4096 4611 -> 4404; 16: 407 -> 328, 1011 -> 928,
+    // 4921 -> 4757)
+    const bool prepared = solve_workspace(h, n);
+    if (prepared) {
+      if ((e = launch_solve_inverses(h->fact, n, n, h->swork, s)) != cudaSuccess) return cuda_status(h, e, "hrp_posv");
+      h->launches += solve_launches(n, 0, true);
+    }
+    // X0 = POTRS(B) (in FP32 where the sweeps do it)
     if ((e = launch_copy_matrix(dX, ldx, dB, ldb, n, nrhs, s)) != cudaSuccess) return cuda_status(h, e, "hrp_posv");
-    if ((st = potrs_impl(h, n, nrhs, h->fact, n, dX, ldx, true, s)) != HRP_OK) return st;
+    if ((st = potrs_impl(h, n, nrhs, h->fact, n, dX, ldx, true, s, prepared)) != HRP_OK) return st;
     it = 0;
     double prev = 1e300;
     bool diverged = false;
@@ -1197,10 +1227,11 @@ hrp_status hrp_posv(hrp_handle* h, const hrp_tree* tree, int n, int nrhs, const 
       prev = worst;
       if (h->refine_mode == 1) {
         for (int c = 0; c < nrhs; ++c)
-          if ((st = gmres_correction(h, dA, lda, n, h->work + (size_t)c * n, dX + (size_t)c * ldx, s)) != HRP_OK)
+          if ((st = gmres_correction(h, dA, lda, n, h->work + (size_t)c * n, dX + (size_t)c * ldx, prepared, s)) !=
+              HRP_OK)
             return st;
       } else {
-        if ((st = potrs_impl(h, n, nrhs, h->fact, n, h->work, n, true, s)) != HRP_OK) return st;
+        if ((st = potrs_impl(h, n, nrhs, h->fact, n, h->work, n, true, s, prepared)) != HRP_OK) return st;
         if ((e = launch_axpy_matrix(dX, ldx, h->work, n, n, nrhs, s)) != cudaSuccess)
           return cuda_status(h, e, "hrp_posv");
       }
@@ -1517,7 +1548,7 @@ namespace {
 constexpr int kBatchStreams = 32;
 
 struct SysWork {
-  size_t shadow, w32, pinv, ticket, fact, res, rwork;   // byte offsets into h->bwork
+  size_t shadow, w32, pinv, swork, ticket, fact, res, rwork;   // byte offsets into h->bwork
   int lds;
 };
 
@@ -1534,6 +1565,7 @@ hrp_status batch_prepare(hrp_handle* h, int batch, const int* n, std::vector<Sys
     w.shadow = need_factor_ws ? take((size_t)ni * w.lds * sizeof(__half)) : 0;
     w.w32 = need_factor_ws ? take(((size_t)ni * 128 + kLeafScratch) * sizeof(float)) : 0;
     w.pinv = take(potrs_workspace_bytes(ni));
+    w.swork = ni <= kSolveSmall ? take(solve_workspace_bytes(ni)) : 0;
     w.ticket = take(sizeof(int));
     w.fact = nrhs_ir ? take(sizeof(double) * (size_t)ni * ni) : 0;
     w.res = nrhs_ir ? take(sizeof(double) * (size_t)ni * nrhs_ir + sizeof(double) * 2 * nrhs_ir) : 0;
@@ -1820,9 +1852,16 @@ hrp_status hrp_potrs_batched(hrp_handle* h, int batch, const int* n, double* con
   for (int i = 0; i < batch; ++i) {
     if (n[i] == 0) continue;
     cudaStream_t si = h->bstreams[which[i]];
-    cudaError_t e = launch_potrs(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, false, h->bwork + ws[i].pinv,
-                                 reinterpret_cast<int*>(h->bwork + ws[i].ticket), h->d_err, si, h->wait_ns);
-    launches += 1 + potrs_sweeps(nrhs);
+    cudaError_t e;
+    if (n[i] <= kSolveSmall) {
+      e = launch_solve_inverses(dL[i], ldl[i], n[i], h->bwork + ws[i].swork, si);
+      if (e == cudaSuccess) e = launch_solve(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, h->bwork + ws[i].swork, si);
+      launches += solve_launches(n[i], nrhs, true);
+    } else {
+      e = launch_potrs(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, false, h->bwork + ws[i].pinv,
+                       reinterpret_cast<int*>(h->bwork + ws[i].ticket), h->d_err, si, h->wait_ns);
+      launches += 1 + potrs_sweeps(nrhs);
+    }
     if (e != cudaSuccess && err == cudaSuccess) err = e;
   }
   if ((st = join(h, s)) != HRP_OK) return st;

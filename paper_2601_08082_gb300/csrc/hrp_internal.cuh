@@ -177,6 +177,19 @@ inline int gemm_block_offsets(GemmBlocks& bl, int t) {
 // FP64 products of a list of blocks (k_gemm_f64.cu), with the accuracy of FP64 or better
 cudaError_t launch_gemm_f64_blocks(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, int k,
                                    GemmBlocks& bl, cudaStream_t s);
+// Independent products C[co ..] = X[xo ..] Y[yo ..]^T (m x n, inner dimension k; offsets in elements), or
+// with neg_rows C = -X Y^T with Y given by rows (term kk of row r at Y[yo + r ldy + kk])
+struct GemmProduct {
+  long long xo, yo, co;
+  int m, n, k, tile0;
+};
+constexpr int kMaxGemmProducts = 256;
+struct GemmProducts {
+  int count = 0;
+  GemmProduct b[kMaxGemmProducts];
+};
+cudaError_t launch_gemm_f64_products(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, bool neg_rows,
+                                     GemmProducts& bl, cudaStream_t s);
 // FP32 products of a list of blocks, operands from FP32 copies (k_gemm_simt.cu); every entry is
 // the same chain of FMAs as in launch_gemm_simt_f32
 // whether launch_gemm_simt_f32 takes its 128 x 128 tiles (then better launched alone)
@@ -216,6 +229,27 @@ cudaError_t launch_potrs(const double* L, int ldl, double* B, int ldb, int n, in
 cudaError_t launch_wait_probe(double* entry, unsigned long long wait_limit_ns, unsigned* dev_err,
                               unsigned long long* waited_ns, cudaStream_t s);
 int potrs_sweeps(int nrhs);
+
+// ---------------- POTRS by block inverses (k_solve.cu) ----------------
+// rows per block
+constexpr int solve_block(int n) { return n <= 64 ? 64 : n <= 128 ? 128 : n <= 1024 ? 256 : 512; }
+// columns of the scratch for the products of the doubling
+constexpr int solve_scratch(int n) { return solve_block(n) / 2; }
+// the inverses (n x block), the scratch, and the intermediate solution (16 columns), FP64
+constexpr size_t solve_workspace_bytes(int n) {
+  return (size_t)n * (solve_block(n) + solve_scratch(n) + kPotrsMaxRhs) * sizeof(double);
+}
+// Prepares `work` (solve_workspace_bytes(n)) for solves with the factor in the lower triangle of L:
+// the FP64 inverses of its diagonal blocks.
+cudaError_t launch_solve_inverses(const double* L, int ldl, int n, void* work, cudaStream_t s);
+// B (n x nrhs) <- A^{-1} B with A = L L^T and the prepared work
+cudaError_t launch_solve(const double* L, int ldl, double* B, int ldb, int n, int nrhs, void* work, cudaStream_t s);
+// whether a single solve takes the block inverses rather than the sweeps; a batched one does up to
+// kSolveSmall
+bool solve_blocked(int n, int nrhs);
+constexpr int kSolveSmall = 256;
+// their launches (nrhs = 0: of the inverses alone)
+int solve_launches(int n, int nrhs, bool inverses);
 
 // ---------------- utilities (k_util.cu) ----------------
 // SM count of the current device, queried once per device

@@ -29,11 +29,19 @@ namespace {
 constexpr int kT = 32;                         // tile edge
 constexpr int kThreads = 128;
 constexpr int kPlane = kT * kDigLd;            // halves per digit plane of one operand
+constexpr int kSpecial = 1 << 20;              // OPs 1 and 2: the exponent of a NaN or an infinity
 constexpr int kFlush = 64;                     // chunks the 32-bit sums hold (2^24 each) before a move to FP64
 
+// OP 0: C -= X Y^T.  OP 1: C = X Y^T with term kk of X's row r zero for kk < r.  OP 2: C = -X Y^T with Y
+// given by rows (term kk of row r at Y[r ldy + kk]), zero for kk > r.  OPs 1 and 2 (the doubling of
+// triangular inverses, launch_solve_inverses) skip the chunks of 32 terms that are all zero.  They
+// also scale term kk, X's entries by 2^t and Y's by 2^-t, by the largest entry of the term in the tile's
+// rows of the operand that is no triangle (Y in OP 1, X in OP 2): rows then keep their digits whatever
+// powers of two scale the rows or the columns of the triangle that is inverted.
+template <int OP, class List>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict__ X, int ldx,
-                       const double* __restrict__ Y, int ldy, int k, const __grid_constant__ GemmBlocks bl) {
+                       const double* __restrict__ Y, int ldy, int k, const __grid_constant__ List bl) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) __half dig[];                  // [2 operands][7][32][kDigLd]
@@ -44,14 +52,29 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
   // this CTA's block and tile
   int b = 0;
   while (b + 1 < bl.count && (int)blockIdx.x >= bl.b[b + 1].tile0) ++b;
-  const GemmBlock blk = bl.b[b];
+  const auto blk = bl.b[b];
   const int ti = (int)blockIdx.x - blk.tile0;
   int ty, tx;
-  gemm_block_tile(blk, kT, ti, tx, ty);
-  const int m0 = tx * kT, n0 = ty * kT, m = blk.m, n = blk.n, lower = blk.lower;
-  const double* Xb = X + blk.xr;
-  const double* Yb = Y + blk.yr;
-  double* Cb = C + (size_t)blk.yr * ldc + blk.xr;
+  const double* Xb;
+  const double* Yb;
+  double* Cb;
+  int lower = 0;
+  if constexpr (OP == 0) {
+    gemm_block_tile(blk, kT, ti, tx, ty);
+    lower = blk.lower;
+    Xb = X + blk.xr;
+    Yb = Y + blk.yr;
+    Cb = C + (size_t)blk.yr * ldc + blk.xr;
+  } else {
+    const int gm = (blk.m + kT - 1) / kT;
+    ty = ti / gm;
+    tx = ti - ty * gm;
+    k = blk.k;
+    Xb = X + blk.xo;
+    Yb = Y + blk.yo;
+    Cb = C + blk.co;
+  }
+  const int m0 = tx * kT, n0 = ty * kT, m = blk.m, n = blk.n;
 
   if (tid < 2 * kT) {
     rowmax[0][tid] = rowmax[1][tid] = 0;
@@ -65,7 +88,8 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
     for (int q = 0; q < 8; ++q) {
       const int kk = k0 + 8 * warp + q;
       px[q] = (okx && kk < k) ? Xb[(size_t)kk * ldx + m0 + lane] : 0.0;
-      py[q] = (oky && kk < k) ? Yb[(size_t)kk * ldy + n0 + lane] : 0.0;
+      if (OP == 2) py[q] = (oky && kk < k) ? Yb[(size_t)(n0 + lane) * ldy + kk] : 0.0;
+      else py[q] = (oky && kk < k) ? Yb[(size_t)kk * ldy + n0 + lane] : 0.0;
     }
   };
   int iacc[kDig][8];
@@ -92,15 +116,25 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
   };
   bool flushed = false, special = false;
   int held = 0;
-  fetch(0);
+  const int c0 = OP == 1 ? m0 / kDigK : 0;
+  const int nchunk = OP == 2 ? (min(k, n0 + kT) + kDigK - 1) / kDigK : (k + kDigK - 1) / kDigK;
+  fetch(c0 * kDigK);
   __syncthreads();
-  const int nchunk = (k + kDigK - 1) / kDigK;
-  for (int c = 0; c < nchunk; ++c) {
-    int fx = 0, fy = 0;
+  for (int c = c0; c < nchunk; ++c) {
+    int fx = 0, fy = 0, tk[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      fx = max(fx, dig_field(px[q]));
-      fy = max(fy, dig_field(py[q]));
+      const int gx = dig_field(px[q]), gy = dig_field(py[q]);
+      if constexpr (OP == 0) {
+        fx = max(fx, gx);
+        fy = max(fy, gy);
+      } else {
+        const int g = (int)__reduce_max_sync(0xffffffffu, (unsigned)(OP == 1 ? gy : gx));
+        tk[q] = g == 0 ? -4096 : g - 1023;                       // a term that is zero throughout: negligible
+        if (OP == 2) tk[q] = -tk[q];
+        fx = max(fx, gx == 0x7ff ? kSpecial : (gx == 0 ? 0 : gx + tk[q]));
+        fy = max(fy, gy == 0x7ff ? kSpecial : (gy == 0 ? 0 : gy - tk[q]));
+      }
     }
     atomicMax(&rowmax[c & 1][lane], fx);
     atomicMax(&rowmax[c & 1][kT + lane], fy);
@@ -109,7 +143,7 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
     if (tid < 2 * kT) {
       mx = rowmax[c & 1][tid];
       rowmax[(c + 1) & 1][tid] = 0;
-      need = mx == 0x7ff ? 2 : (max(mx, 1) > scale[tid] ? 1 : 0);
+      need = mx == (OP == 0 ? 0x7ff : kSpecial) ? 2 : (max(mx, 1) > scale[tid] ? 1 : 0);
     }
     const bool grow = __syncthreads_or(need) != 0;
     if (grow && __syncthreads_or(need == 2)) {
@@ -126,8 +160,19 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
       if (need) scale[tid] = max(mx, 1) + kDigHead;
       __syncthreads();
     }
-    dig_split8(px, scale[lane], dig + lane * kDigLd + 8 * warp, kPlane);
-    dig_split8(py, scale[kT + lane], dig + kDig * kPlane + lane * kDigLd + 8 * warp, kPlane);
+    if constexpr (OP != 0) {
+      int ex[8], ey[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        ex[q] = scale[lane] - tk[q];
+        ey[q] = scale[kT + lane] + tk[q];
+      }
+      dig_split8(px, ex, dig + lane * kDigLd + 8 * warp, kPlane);
+      dig_split8(py, ey, dig + kDig * kPlane + lane * kDigLd + 8 * warp, kPlane);
+    } else {
+      dig_split8(px, scale[lane], dig + lane * kDigLd + 8 * warp, kPlane);
+      dig_split8(py, scale[kT + lane], dig + kDig * kPlane + lane * kDigLd + 8 * warp, kPlane);
+    }
     if (c + 1 < nchunk) fetch((c + 1) * kDigK);
     __syncthreads();
     dig_chunk(dig, kPlane, a0, dig + kDig * kPlane, kPlane, b0, iacc);
@@ -139,8 +184,11 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
       const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
       if (r >= m || cl >= n || (lower && r < cl)) continue;
       double s = 0.0;
-      for (int kk = 0; kk < k; ++kk) s = fma(Xb[(size_t)kk * ldx + r], Yb[(size_t)kk * ldy + cl], s);
-      Cb[(size_t)cl * ldc + r] -= s;
+      for (int kk = 0; kk < k; ++kk)
+        s = fma(Xb[(size_t)kk * ldx + r], OP == 2 ? Yb[(size_t)cl * ldy + kk] : Yb[(size_t)kk * ldy + cl], s);
+      double* p = Cb + (size_t)cl * ldc + r;
+      if (OP == 0) *p -= s;
+      else *p = OP == 1 ? s : -s;
     }
     return;
   }
@@ -148,7 +196,7 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
-    cv[j] = (r < m && cl < n && !(lower && r < cl)) ? Cb[(size_t)cl * ldc + r] : 0.0;
+    cv[j] = (OP == 0 && r < m && cl < n && !(lower && r < cl)) ? Cb[(size_t)cl * ldc + r] : 0.0;
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -160,20 +208,44 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
     double v = dig_value(iacc, j);
     if (f1 != 1.0) v *= f1;
     double* p = Cb + (size_t)cl * ldc + r;
-    if (flushed) *p = cv[j] - fma(v, f0, vacc[j]);
-    else *p = fma(-v, f0, cv[j]);
+    if (OP == 0) {
+      if (flushed) *p = cv[j] - fma(v, f0, vacc[j]);
+      else *p = fma(-v, f0, cv[j]);
+    } else {
+      const double x = flushed ? fma(v, f0, vacc[j]) : v * f0;
+      *p = OP == 1 ? x : -x;
+    }
   }
 }
 
 }  // namespace
+
+constexpr int kSmem = 2 * kDig * kPlane * (int)sizeof(__half);
 
 cudaError_t launch_gemm_f64_blocks(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, int k,
                                    GemmBlocks& bl, cudaStream_t s) {
   if (k <= 0 || bl.count <= 0) return cudaSuccess;
   const int tiles = gemm_block_offsets(bl, kT);
   if (tiles <= 0) return cudaSuccess;
-  const int smem = 2 * kDig * kPlane * (int)sizeof(__half);
-  (void)launch_pdl(gemm_f64_digits_kernel, dim3(tiles), dim3(kThreads), smem, s, C, ldc, X, ldx, Y, ldy, k, bl);
+  (void)launch_pdl(gemm_f64_digits_kernel<0, GemmBlocks>, dim3(tiles), dim3(kThreads), kSmem, s, C, ldc, X, ldx, Y, ldy,
+                   k, bl);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_f64_products(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, bool neg_rows,
+                                     GemmProducts& bl, cudaStream_t s) {
+  int tiles = 0;
+  for (int i = 0; i < bl.count; ++i) {
+    bl.b[i].tile0 = tiles;
+    tiles += ((bl.b[i].m + kT - 1) / kT) * ((bl.b[i].n + kT - 1) / kT);
+  }
+  if (tiles <= 0) return cudaSuccess;
+  if (neg_rows)
+    (void)launch_pdl(gemm_f64_digits_kernel<2, GemmProducts>, dim3(tiles), dim3(kThreads), kSmem, s, C, ldc, X, ldx, Y, ldy,
+                     0, bl);
+  else
+    (void)launch_pdl(gemm_f64_digits_kernel<1, GemmProducts>, dim3(tiles), dim3(kThreads), kSmem, s, C, ldc, X, ldx, Y, ldy,
+                     0, bl);
   return cudaGetLastError();
 }
 

@@ -1,4 +1,5 @@
-// POTRS: solve A X = B with the Cholesky factor, L Y = B then L^T X = Y.
+// POTRS by wavefront sweeps: solve A X = B with the Cholesky factor, L Y = B then L^T X = Y (k_solve.cu
+// has the other way and where it is taken).
 //
 // Two launches per sweep pair plus one pre-pass:
 //   1. inverse pre-pass: every 64 x 64 diagonal block L_rr is inverted in parallel (one

@@ -1,0 +1,531 @@
+// POTRS by block inverses: L Y = B, then L^T X = Y, in blocks of up to 512 rows.
+//
+// The wavefront sweeps of k_potrs.cu hand 64-row blocks from CTA to CTA; a link costs 2.5 us with one
+// right-hand side (the handoff through L2) and 15 us with 16 (the link's products on one SM), n / 64
+// of them in a row.  Here the diagonal blocks of `blk` rows are inverted first, all at once: blocks of
+// 64 by substitution, then doubled to 128, 256 and 512 rows, W21 = -W22 (L21 W11) by digit products
+// (k_gemm_f64.cu).  A sweep is then n / blk steps of two launches that fill the
+// chip,
+//   y_r = W_r b_r,   b_i -= L_ir y_r for the rows i still to come,
+// and the same with the transposes on the way back.  The inverses serve every solve with the
+// factor (the corrections of a refinement, further groups of 16 right-hand sides).
+//
+// Both products take 16 rows at a time and up to 512 inner terms, a warp 16 (few rows,
+// solve_step_kernel) or 64 of them (many, solve_wide_kernel).  The entries go from memory to registers
+// in the order the mma fragments want them, are cut into 8-bit digits there and multiplied exactly by
+// 28 mma per 16 terms (digits.cuh); the warps' sums are added in FP64 in a fixed order.  Scales: term k
+// by its largest right-hand side, then a row of P and a column of Y by the largest entry among the
+// warp's terms, so 7 digits keep 55 bits below the largest term of a sum (with several right-hand
+// sides, below the row's times the column's), whatever powers of two scale the unknowns.
+// What bounds it: latency, 5 us a step with few rows and 8 to 11 us with many (at n = 4096 and one
+// right-hand side 170 us of inverses, most of it the last doubling, then 30 steps); from n = 8192 on the
+// integer work of the wide kernel (~2000 instructions per warp and 16 x 64 entries at two warps per
+// scheduler: 5 us a row tile, issue slots 30 % used).  Solves against the sweeps', us with 1, 4 and 16
+// right-hand sides:
+//   n = 64 18 18 23 (56 60 84), 128 41 41 47 (105 113 140), 2048 233 237 286 (248 365 994),
+//   4 and 16: 4096 427 560 (637 1914), 8192 907 1246 (1204 3794).
+// Backward errors are 3 to 30 times below the sweeps' (whose double-float products keep 44 bits), also
+// for kernel matrices of condition 1e15.  A warp that meets a NaN or an infinity uses FP64 FMAs for its
+// terms.
+#include <cooperative_groups.h>
+
+#include <climits>
+
+#include "digits.cuh"
+#include "hrp_internal.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace hrp {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kRows = 16;
+constexpr int kNone = -4096;                     // below every exponent of a right-hand side against its term's
+
+// The inverse of a 64 x 64 diagonal block of L (block blockIdx.y), 8 of its columns per CTA: columns
+// blockIdx.x + 8 u, two to a warp, so that every CTA has as much to do.  16 lanes hold a column, rows
+// q, q + 16, ..; substitution in FP64, a step costs one reciprocal product, a broadcast and up to four
+// FMAs, and what bounds it is that chain (64 steps of ~150 clocks), from n = 4096 on the FP64 pipe.
+// Row i goes to W + i blk at the block's columns, zeros after it.
+__global__ void __launch_bounds__(128)
+inverse64_kernel(const double* __restrict__ L, int ldl, int n, double* __restrict__ W, int blk) {
+  __shared__ double Ls[64][65];                  // [k][i]
+  __shared__ double rinv[64];
+  pdl_wait();
+  pdl_trigger();
+  const int c0 = 64 * blockIdx.y, m = min(64, n - c0), off = c0 % blk;
+  const int tid = threadIdx.x, lane = tid & 31, q = lane & 15;
+#pragma unroll
+  for (int u = 0; u < 32; ++u) {
+    const int i = tid & 63, k = (tid >> 6) + 2 * u;
+    Ls[k][i] = (i < m && k <= i) ? L[(size_t)(c0 + k) * ldl + c0 + i] : 0.0;
+  }
+  for (int e = tid; e < 8 * (blk - off - 64); e += 128) {
+    const int i = (int)blockIdx.x + 8 * (e / (blk - off - 64));
+    if (i < m) W[(size_t)(c0 + i) * blk + off + 64 + e % (blk - off - 64)] = 0.0;
+  }
+  __syncthreads();
+  if (tid < 64) rinv[tid] = tid < m ? 1.0 / Ls[tid][tid] : 1.0;
+  __syncthreads();
+  const int first = (int)blockIdx.x + 16 * (tid >> 5), c = first + 8 * (lane >> 4);
+  double y[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) y[p] = q + 16 * p == c ? 1.0 : 0.0;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    if (16 * p + 15 < first) continue;           // whole warps
+    for (int kk = 0; kk < 16; ++kk) {
+      const int k = 16 * p + kk;
+      const double v = __shfl_sync(0xffffffffu, y[p], (lane & 16) | kk) * rinv[k];
+      if (q == kk) y[p] = v;
+      else if (q > kk) y[p] = fma(-Ls[k][q + 16 * p], v, y[p]);
+#pragma unroll
+      for (int r = p + 1; r < 4; ++r) y[r] = fma(-Ls[k][q + 16 * r], v, y[r]);
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int i = q + 16 * p;
+    if (i < m && c < 64) W[(size_t)(c0 + i) * blk + off + c] = i >= c ? y[p] : 0.0;
+  }
+}
+
+// What the two product kernels share: the fragments of a warp's 16 KS terms from k0.
+// A: element (half-row h, k step s, j) is row r0 + g + 8 h, k = k0 + 16 s + t2 + (j & 1) + 8 (j >> 1), with
+// g = lane / 4, t2 = 2 (lane % 4); P(i, k) at P[k ldp + i], or TRANS: P[i ldp + k]
+template <bool TRANS, int KS>
+__device__ __forceinline__ void load_rows(double (&a)[2][KS][4], const double* __restrict__ P, int ldp, int r0, int rows, int k0,
+                                          int K) {
+  const int g = (threadIdx.x & 31) >> 2, t2 = 2 * (threadIdx.x & 3);
+#pragma unroll
+  for (int s = 0; s < KS; ++s)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = k0 + 16 * s + t2 + (j & 1) + 8 * (j >> 1);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = r0 + g + 8 * h;
+        a[h][s][j] = (i < rows && k < K) ? (TRANS ? P[(size_t)i * ldp + k] : P[(size_t)k * ldp + i]) : 0.0;
+      }
+    }
+}
+// Y: element (half h, s, j) is right-hand side g + 8 h, the same k
+template <int NH, int KS>
+__device__ __forceinline__ void load_rhs(double (&y)[NH][KS][4], const double* __restrict__ Y, int ldy, int nrhs, int k0, int K) {
+  const int g = (threadIdx.x & 31) >> 2, t2 = 2 * (threadIdx.x & 3);
+#pragma unroll
+  for (int s = 0; s < KS; ++s)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = k0 + 16 * s + t2 + (j & 1) + 8 * (j >> 1);
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {
+        const int c = g + 8 * h;
+        y[h][s][j] = (c < nrhs && k < K) ? Y[(size_t)c * ldy + k] : 0.0;
+      }
+    }
+}
+// The scales: of term k the largest exponent field among its right-hand sides, over the eight lanes (and
+// halves) that hold them, two terms a word of ek; of a right-hand side (ey) the largest of its fields
+// against the terms' scales; of a row (ea) the largest field times its term's scale.  special: a NaN or
+// an infinity (in some lane).
+template <int KS>
+__device__ __forceinline__ int term(const unsigned (&ek)[KS][2], int s, int j) {
+  return (int)((ek[s][j >> 1] >> (16 * (j & 1))) & 0xffffu);
+}
+template <int NH, int KS>
+__device__ __forceinline__ void rhs_scales(const double (&y)[NH][KS][4], unsigned (&ek)[KS][2], int (&ey)[NH], bool& special) {
+#pragma unroll
+  for (int s = 0; s < KS; ++s)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      unsigned w = 0x00010001u;
+#pragma unroll
+      for (int h = 0; h < NH; ++h)
+        w = __vmaxu2(w, (unsigned)dig_field(y[h][s][2 * p]) | ((unsigned)dig_field(y[h][s][2 * p + 1]) << 16));
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) w = __vmaxu2(w, __shfl_xor_sync(0xffffffffu, w, o));
+      special |= (w & 0xffffu) == 0x7ffu || (w >> 16) == 0x7ffu;
+      ek[s][p] = w;
+    }
+#pragma unroll
+  for (int h = 0; h < NH; ++h) {
+    ey[h] = kNone;
+#pragma unroll
+    for (int s = 0; s < KS; ++s)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int f = dig_field(y[h][s][j]);
+        if (f != 0) ey[h] = max(ey[h], f - term<KS>(ek, s, j));
+      }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) ey[h] = max(ey[h], __shfl_xor_sync(0xffffffffu, ey[h], o));
+  }
+}
+template <int KS>
+__device__ __forceinline__ void row_scales(const double (&a)[2][KS][4], const unsigned (&ek)[KS][2], int (&ea)[2], bool& special) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    ea[h] = INT_MIN;
+#pragma unroll
+    for (int s = 0; s < KS; ++s)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int f = dig_field(a[h][s][j]);
+        special |= f == 0x7ff;
+        ea[h] = max(ea[h], max(f, 1) + term<KS>(ek, s, j));
+      }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) ea[h] = max(ea[h], __shfl_xor_sync(0xffffffffu, ea[h], o));
+  }
+}
+// the digits of a k step of the right-hand sides, and its products
+template <int NH, int KS>
+__device__ __forceinline__ void rhs_digits(const double (&y)[NH][KS][4], const unsigned (&ek)[KS][2], const int (&ey)[NH], int s,
+                                           uint32_t (&bf)[kDig][NH][2]) {
+#pragma unroll
+  for (int h = 0; h < NH; ++h) {
+    unsigned long long m[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) m[j] = (unsigned long long)dig_fix(y[h][s][j], ey[h] + term<KS>(ek, s, j)) + kByteBias;
+#pragma unroll
+    for (int d = 0; d < kDig; ++d) {
+      bf[d][h][0] = byte_pair(m[0], m[1], d);
+      bf[d][h][1] = byte_pair(m[2], m[3], d);
+    }
+  }
+}
+__device__ __forceinline__ void row_fragment(const unsigned long long (&m0)[4], const unsigned long long (&m1)[4], int d,
+                                             uint32_t (&af)[4]) {
+  af[0] = byte_pair(m0[0], m0[1], d);
+  af[1] = byte_pair(m1[0], m1[1], d);
+  af[2] = byte_pair(m0[2], m0[3], d);
+  af[3] = byte_pair(m1[2], m1[3], d);
+}
+// the warp's sums to part[row][right-hand side]: weights 2^(-12 - 8 w) joined in units of 2^-57 (at most 64
+// terms below 1)
+template <int NH>
+__device__ __forceinline__ void store_sums(const float (&acc)[kDig][NH][4], const int (&ea)[2], const int (&ey)[NH],
+                                           double (*part)[8 * NH]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
+#pragma unroll
+  for (int h = 0; h < NH; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      long long hi = 0, lo = 0;
+#pragma unroll
+      for (int w = 0; w < 3; ++w) hi = (hi << 8) + __float2int_rn(acc[w][h][q]);
+#pragma unroll
+      for (int w = 3; w < kDig; ++w) lo = (lo << 8) + __float2int_rn(acc[w][h][q]);
+      const int c = t2 + (q & 1);
+      const int e = ea[q >> 1] + __shfl_sync(0xffffffffu, ey[h], 4 * c) - 2 * 1022;
+      part[g + 8 * (q >> 1)][8 * h + c] = dig_to_double((hi << 29) + (lo >> 3), e - 57);
+    }
+}
+// the same sums by FP64 FMAs over the terms kb .. ke - 1 (row i: from lo(i), below hi(i))
+template <int NH, bool TRANS, class Lo, class Hi>
+__device__ __forceinline__ void plain_sums(const double* __restrict__ P, int ldp, int r0, int rows, const double* __restrict__ Y, int ldy,
+                                           int nrhs, Lo lo, Hi hi, double (*part)[8 * NH]) {
+  for (int e = threadIdx.x & 31; e < kRows * 8 * NH; e += 32) {
+    const int i = r0 + e / (8 * NH), c = e % (8 * NH);
+    double v = 0.0;
+    if (i < rows && c < nrhs)
+      for (int k = lo(i); k < hi(i); ++k)
+        v = fma(TRANS ? P[(size_t)i * ldp + k] : P[(size_t)k * ldp + i], Y[(size_t)c * ldy + k], v);
+    part[e / (8 * NH)][c] = v;
+  }
+}
+template <int NH>
+__device__ __forceinline__ double sum_parts(const double (*part)[kRows][8 * NH], int i, int c) {
+  return ((part[0][i][c] + part[1][i][c]) + (part[2][i][c] + part[3][i][c])) +
+         ((part[4][i][c] + part[5][i][c]) + (part[6][i][c] + part[7][i][c]));
+}
+
+// O(i, c) = sum_k P(i, k) Y(k, c) (ADD: O -= ...) for few rows i < rows, k < K <= 512, c < nrhs <= 8 NH.
+// TRI 1: P(i, k) = 0 for k > i; TRI 2: for k < i.  A CTA covers 128 terms, a warp 16, and a cluster of
+// ceil(K / 128) CTAs in y the row tile; the others leave their sums in CTA 0's shared memory.
+template <int NH, bool TRANS, bool ADD, int TRI>
+__global__ void __launch_bounds__(kThreads, 2)
+solve_step_kernel(const double* __restrict__ P, int ldp, int rows, int K, const double* __restrict__ Y, int ldy,
+                  double* __restrict__ O, int ldo, int nrhs) {
+  // CTA 0 of a cluster must have started before the others write to its shared memory
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  pdl_wait();
+  pdl_trigger();
+  __shared__ double part[8][kRows][8 * NH];
+  __shared__ double from[3][kRows * 8 * NH];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r0 = blockIdx.x * kRows, k0 = 128 * (int)blockIdx.y + 16 * warp;
+  if (k0 < K && !(TRI == 1 && k0 > r0 + kRows - 1) && !(TRI == 2 && k0 + 15 < r0)) {
+    double a[2][1][4], y[NH][1][4];
+    load_rows<TRANS, 1>(a, P, ldp, r0, rows, k0, K);
+    load_rhs<NH, 1>(y, Y, ldy, nrhs, k0, K);
+    unsigned ek[1][2];
+    int ea[2], ey[NH];
+    bool special = false;
+    rhs_scales<NH, 1>(y, ek, ey, special);
+    row_scales<1>(a, ek, ea, special);
+    if (__any_sync(0xffffffffu, special)) {
+      plain_sums<NH, TRANS>(P, ldp, r0, rows, Y, ldy, nrhs, [&](int i) { return TRI == 2 ? max(k0, i) : k0; },
+                            [&](int i) { return min(min(K, k0 + 16), TRI == 1 ? i + 1 : K); }, part[warp]);
+    } else {
+      float acc[kDig][NH][4] = {};
+      uint32_t bf[kDig][NH][2];
+      rhs_digits<NH, 1>(y, ek, ey, 0, bf);
+      unsigned long long m[2][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) m[h][j] = (unsigned long long)dig_fix(a[h][0][j], ea[h] - term<1>(ek, 0, j)) + kByteBias;
+#pragma unroll
+      for (int d = 0; d < kDig; ++d) {
+        uint32_t af[4];
+        row_fragment(m[0], m[1], d, af);
+#pragma unroll
+        for (int e = 0; e < kDig - d; ++e)
+#pragma unroll
+          for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h][0], bf[e][h][1]);
+      }
+      store_sums<NH>(acc, ea, ey, part[warp]);
+    }
+  } else {
+    for (int e = lane; e < kRows * 8 * NH; e += 32) part[warp][e / (8 * NH)][e % (8 * NH)] = 0.0;
+  }
+  __syncthreads();
+  const int i = tid % kRows, c = tid / kRows;
+  const bool out = c < 8 * NH && r0 + i < rows && c < nrhs;
+  double v = out ? sum_parts<NH>(part, i, c) : 0.0;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (rank > 0 && out) cluster.map_shared_rank(&from[rank - 1][0], 0)[tid] = v;
+  cluster.sync();
+  if (rank > 0 || !out) return;
+  for (int q = 1; q < (int)gridDim.y; ++q) v += from[q - 1][tid];
+  double* o = O + (size_t)c * ldo + r0 + i;
+  *o = ADD ? *o - v : v;
+}
+static_assert(kRows * 16 == kThreads, "one output per thread at 16 right-hand sides");
+
+// O -= P Y for many rows: a warp keeps 64 terms, whose right-hand sides' digits it cuts once and holds in
+// shared memory as mma fragments, and the CTA runs over row tiles, the next tile's entries in flight
+// during the products.
+constexpr int kWide = 4;                         // k steps per warp
+template <int NH>
+constexpr int wide_smem() {
+  return 8 * kWide * kDig * NH * 32 * 8 + 2 * 8 * kRows * 8 * NH * 8;
+}
+template <int NH, bool TRANS>
+__global__ void __launch_bounds__(kThreads, 1)
+solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const double* __restrict__ Y, int ldy,
+                  double* __restrict__ O, int ldo, int nrhs) {
+  pdl_wait();
+  pdl_trigger();
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint2 (*bfs)[kDig][NH][32] = reinterpret_cast<uint2 (*)[kDig][NH][32]>(smem) + warp * kWide;     // [s][digit][half][lane]
+  double (*parts)[8][kRows][8 * NH] =
+      reinterpret_cast<double (*)[8][kRows][8 * NH]>(smem + 8 * kWide * kDig * NH * 32 * 8);        // [parity]
+  const int k0 = 16 * kWide * warp;
+  const bool act = k0 < K;
+  const int step = (int)gridDim.x * kRows;
+  int r0 = (int)blockIdx.x * kRows;
+  double a[2][kWide][4];
+  if (act) load_rows<TRANS, kWide>(a, P, ldp, r0, rows, k0, K);
+  unsigned ek[kWide][2];
+  int ey[NH];
+  bool yspecial = false;
+  if (act) {
+    double y[NH][kWide][4];
+    load_rhs<NH, kWide>(y, Y, ldy, nrhs, k0, K);
+    rhs_scales<NH, kWide>(y, ek, ey, yspecial);
+    if (!__any_sync(0xffffffffu, yspecial)) {
+#pragma unroll
+      for (int s = 0; s < kWide; ++s) {
+        uint32_t bf[kDig][NH][2];
+        rhs_digits<NH, kWide>(y, ek, ey, s, bf);
+#pragma unroll
+        for (int d = 0; d < kDig; ++d)
+#pragma unroll
+          for (int h = 0; h < NH; ++h) bfs[s][d][h][lane] = make_uint2(bf[d][h][0], bf[d][h][1]);
+      }
+    }
+    __syncwarp();
+  }
+  const int i = tid % kRows, c = tid / kRows;
+  for (int par = 0; r0 < rows; r0 += step, par ^= 1) {
+    const bool out = c < 8 * NH && r0 + i < rows && c < nrhs;
+    double* o = O + (size_t)c * ldo + r0 + i;
+    const double o0 = out ? *o : 0.0;
+    double (*part)[8 * NH] = parts[par][warp];
+    if (act) {
+      int ea[2];
+      bool special = yspecial;
+      row_scales<kWide>(a, ek, ea, special);
+      if (__any_sync(0xffffffffu, special)) {
+        plain_sums<NH, TRANS>(P, ldp, r0, rows, Y, ldy, nrhs, [&](int) { return k0; },
+                              [&](int) { return min(K, k0 + 16 * kWide); }, part);
+        if (r0 + step < rows) load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
+      } else {
+        unsigned long long m[kWide][2][4];
+#pragma unroll
+        for (int s = 0; s < kWide; ++s)
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              m[s][h][j] = (unsigned long long)dig_fix(a[h][s][j], ea[h] - term<kWide>(ek, s, j)) + kByteBias;
+        if (r0 + step < rows) load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
+        float acc[kDig][NH][4] = {};
+#pragma unroll
+        for (int s = 0; s < kWide; ++s) {
+          uint2 bf[kDig][NH];
+#pragma unroll
+          for (int d = 0; d < kDig; ++d)
+#pragma unroll
+            for (int h = 0; h < NH; ++h) bf[d][h] = bfs[s][d][h][lane];
+#pragma unroll
+          for (int d = 0; d < kDig; ++d) {
+            uint32_t af[4];
+            row_fragment(m[s][0], m[s][1], d, af);
+#pragma unroll
+            for (int e = 0; e < kDig - d; ++e)
+#pragma unroll
+              for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h].x, bf[e][h].y);
+          }
+        }
+        store_sums<NH>(acc, ea, ey, part);
+      }
+    } else {
+      for (int e = lane; e < kRows * 8 * NH; e += 32) part[e / (8 * NH)][e % (8 * NH)] = 0.0;
+    }
+    // one barrier per tile: the sums of the next go to the other half
+    __syncthreads();
+    if (out) *o = o0 - sum_parts<NH>(parts[par], i, c);
+  }
+}
+
+template <int NH, bool TRANS, bool ADD, int TRI>
+cudaError_t launch_step(const double* P, int ldp, int rows, int K, const double* Y, int ldy, double* O, int ldo, int nrhs,
+                        cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  const int tiles = (rows + kRows - 1) / kRows, ky = (K + 127) / 128;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if constexpr (ADD) {
+    // rows enough for the wide kernel: more than the clusters' CTAs fit the chip
+    if (tiles * ky > 2 * device_sm_count()) {
+      static unsigned long long attr_mask = 0;
+      const unsigned long long attr_bit = dev_bit();
+      if (!(attr_mask & attr_bit)) {
+        cudaError_t e = cudaFuncSetAttribute(solve_wide_kernel<NH, TRANS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             wide_smem<NH>());
+        if (e != cudaSuccess) return e;
+        attr_mask |= attr_bit;
+      }
+      const int per = (tiles + device_sm_count() - 1) / device_sm_count();
+      cfg.gridDim = dim3((tiles + per - 1) / per);
+      cfg.dynamicSmemBytes = wide_smem<NH>();
+      return cudaLaunchKernelEx(&cfg, solve_wide_kernel<NH, TRANS>, P, ldp, rows, K, Y, ldy, O, ldo, nrhs);
+    }
+  }
+  cfg.gridDim = dim3(tiles, ky);
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = ky;
+  at[1].val.clusterDim.z = 1;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, solve_step_kernel<NH, TRANS, ADD, TRI>, P, ldp, rows, K, Y, ldy, O, ldo, nrhs);
+}
+
+template <int NH>
+cudaError_t solve_group(const double* L, int ldl, double* B, int ldb, int n, int nrhs, int blk, const double* W, double* Z,
+                        cudaStream_t s) {
+  const int nb = (n + blk - 1) / blk;
+  cudaError_t e;
+  for (int r = 0; r < nb; ++r) {                 // Z = L^{-1} B, B's rows updated as they come
+    const int R0 = r * blk, m = n - R0 < blk ? n - R0 : blk;
+    if ((e = launch_step<NH, true, false, 1>(W + (size_t)R0 * blk, blk, m, m, B + R0, ldb, Z + R0, n, nrhs, s)) != cudaSuccess)
+      return e;
+    if ((e = launch_step<NH, false, true, 0>(L + (size_t)R0 * ldl + R0 + m, ldl, n - R0 - m, m, Z + R0, n, B + R0 + m, ldb,
+                                             nrhs, s)) != cudaSuccess)
+      return e;
+  }
+  for (int r = nb - 1; r >= 0; --r) {            // B = L^{-T} Z
+    const int R0 = r * blk, m = n - R0 < blk ? n - R0 : blk;
+    if ((e = launch_step<NH, false, false, 2>(W + (size_t)R0 * blk, blk, m, m, Z + R0, n, B + R0, ldb, nrhs, s)) != cudaSuccess)
+      return e;
+    if ((e = launch_step<NH, true, true, 0>(L + R0, ldl, R0, m, B + R0, ldb, Z, n, nrhs, s)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
+// FP64 inverses of the diagonal blocks of solve_block(n) rows
+cudaError_t launch_solve_inverses(const double* L, int ldl, int n, void* work, cudaStream_t s) {
+  const int blk = solve_block(n), ldt = solve_scratch(n);
+  double* W = static_cast<double*>(work);
+  double* T = W + (size_t)n * blk;
+  (void)launch_pdl(inverse64_kernel, dim3(8, (n + 63) / 64), dim3(128), 0, s, L, ldl, n, W, blk);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  for (int h = 64; h < blk; h *= 2) {
+    // T(c, i) = sum_k W11(k, c) L21(i, k), then W21(i, c) = -sum_k T(c, k) W22(i, k)
+    GemmProducts p1, p2;
+    for (int g0 = 0; g0 + h < n; g0 += 2 * h) {
+      const int n2 = n - g0 - h < h ? n - g0 - h : h, off = g0 % blk;
+      const long long w11 = (long long)g0 * blk + off, w22 = (long long)(g0 + h) * blk + off + h;
+      const long long w21 = (long long)(g0 + h) * blk + off, tt = (long long)g0 * ldt;
+      p1.b[p1.count++] = GemmProduct{w11, (long long)g0 * ldl + g0 + h, tt, h, n2, h, 0};
+      p2.b[p2.count++] = GemmProduct{tt, w22, w21, h, n2, n2, 0};
+      if (p1.count == kMaxGemmProducts || g0 + 3 * h >= n) {
+        if ((e = launch_gemm_f64_products(T, ldt, W, blk, L, ldl, false, p1, s)) != cudaSuccess) return e;
+        if ((e = launch_gemm_f64_products(W, blk, T, ldt, W, blk, true, p2, s)) != cudaSuccess) return e;
+        p1.count = p2.count = 0;
+      }
+    }
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_solve(const double* L, int ldl, double* B, int ldb, int n, int nrhs, void* work, cudaStream_t s) {
+  const int blk = solve_block(n);
+  const double* W = static_cast<const double*>(work);
+  double* Z = static_cast<double*>(work) + (size_t)n * (blk + solve_scratch(n));
+  for (int c0 = 0; c0 < nrhs; c0 += kPotrsMaxRhs) {
+    const int nc = nrhs - c0 < kPotrsMaxRhs ? nrhs - c0 : kPotrsMaxRhs;
+    double* Bc = B + (size_t)c0 * ldb;
+    const cudaError_t e = nc <= 8 ? solve_group<1>(L, ldl, Bc, ldb, n, nc, blk, W, Z, s)
+                                  : solve_group<2>(L, ldl, Bc, ldb, n, nc, blk, W, Z, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// Single solves gain at every size (figures above) but with one right-hand side on large factors, whose
+// sweeps read L once and whose links are short: 3000 323 us against 330, 4096 442 against 419, 8192 900
+// against 794.  In a batch, whose systems overlap on streams and whose launches the host issues one after
+// another (3.7 us each), the block solve's n / 64 launches cost more than the sweeps' three from a few
+// hundred rows on; up to 8 right-hand sides and 1024 rows single solves do as batched ones, so that both
+// agree to the bit there.
+bool solve_blocked(int n, int nrhs) { return n <= kSolveSmall || nrhs > 8 || (n > 1024 && (nrhs > 1 || n <= 3072)); }
+
+int solve_launches(int n, int nrhs, bool inverses) {
+  const int blk = solve_block(n), nb = (n + blk - 1) / blk;
+  int l = (nrhs + kPotrsMaxRhs - 1) / kPotrsMaxRhs * (4 * nb - 2);
+  if (inverses) {
+    l += 1;
+    for (int h = 64; h < blk && h < n; h *= 2) l += 2 * ((n + 2 * h * kMaxGemmProducts - 1) / (2 * h * kMaxGemmProducts));
+  }
+  return l;
+}
+
+}  // namespace hrp

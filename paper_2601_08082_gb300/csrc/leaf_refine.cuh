@@ -60,22 +60,6 @@ struct Smem {
   unsigned rmax[2], emax[2];           // largest |R| and scaled |E| here (bits), by step parity
 };
 
-// Digits of 8 bits: byte s of a fixed-point value with kByteBias (128 at every byte) added is d + 128,
-// weight 2^(8 (7 - s)); a pair of digits takes a byte permutation, a mask and a subtraction, less
-// than half of digits.cuh's 9-bit ones, which matters here where every value is split once per use.
-// Eight digits, weights s + t <= 7 kept; a product of 128 terms sums to at most 8 x 128 x 2^14 =
-// 2^24 per weight, exact in binary32 without intermediate moves.
-constexpr unsigned long long kByteBias = 0x8080808080808080ull;
-// digits s of M0 and M1 as a pair of halves
-__device__ __forceinline__ uint32_t byte_pair(unsigned long long M0, unsigned long long M1, int s) {
-  const int byte = 7 - s;                // from the low end
-  const uint32_t w0 = byte >= 4 ? (uint32_t)(M0 >> 32) : (uint32_t)M0, w1 = byte >= 4 ? (uint32_t)(M1 >> 32) : (uint32_t)M1;
-  const uint32_t b = byte & 3;
-  const uint32_t x = (__byte_perm(w0, w1, b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12)) & 0x00ff00ffu) | 0x64006400u;
-  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&x), __half2half2(__ushort_as_half(0x6480)));   // 1152
-  return *reinterpret_cast<const uint32_t*>(&d);
-}
-
 __device__ __forceinline__ int tix(int I, int J) { return I * (I + 1) / 2 + J; }
 // element (i, j) of a binary32 tile: 16-byte groups swizzled so that 8 rows read without conflicts
 __device__ __forceinline__ int ft(int i, int j) { return i * 16 + ((((j >> 2) ^ (i >> 1)) & 3) << 2) + (j & 3); }
