@@ -344,8 +344,9 @@ hrp_status hrp_autotune(hrp_handle* h, const hrp_tree* tree, int n, int reps, in
 hrp_status hrp_potrf_batched(hrp_handle* h, const hrp_tree* const* trees, int batch, const int* n,
                              double* const* dA, const int* lda, int* d_info, void* stream);
 /*
- * Batched POTRS (FP64; by block inverses up to n[i] = 256, else double-float): for each i, dB[i] (n[i] x nrhs, ldb[i]) <- A_i^{-1} dB[i] with the
- * factor in the lower triangle of dL[i].  Same stream pool and capture rules as above.
+ * Batched POTRS (FP64; by block inverses up to n[i] = 256, above that the double-float sweeps):
+ * for each i, dB[i] (n[i] x nrhs, ldb[i]) <- A_i^{-1} dB[i] with the factor in the lower
+ * triangle of dL[i].  Same stream pool and capture rules as above.
  */
 hrp_status hrp_potrs_batched(hrp_handle* h, int batch, const int* n, double* const* dL, const int* ldl,
                              int nrhs, double* const* dB, const int* ldb, void* stream);

@@ -420,7 +420,8 @@ cudaError_t launch_step(const double* P, int ldp, int rows, int K, const double*
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if constexpr (ADD) {
-    // rows enough for the wide kernel: more than the clusters' CTAs fit the chip
+    // the wide kernel where the clusters would be more than two CTAs per SM (n = 3000 .. 8192 with 16
+    // right-hand sides: 2 to 4 % above lines at one half, one and four CTAs)
     if (tiles * ky > 2 * device_sm_count()) {
       static unsigned long long attr_mask = 0;
       const unsigned long long attr_bit = dev_bit();
@@ -511,8 +512,8 @@ cudaError_t launch_solve(const double* L, int ldl, double* B, int ldb, int n, in
 }
 
 // Single solves gain at every size (figures above) but with one right-hand side on large factors, whose
-// sweeps read L once and whose links are short: 3000 323 us against 330, 4096 442 against 419, 8192 900
-// against 794.  In a batch, whose systems overlap on streams and whose launches the host issues one after
+// sweeps read L once and whose links are short: n = 2048 233 us against 248, 4096 about equal (418),
+// 8192 870 against 794.  In a batch, whose systems overlap on streams and whose launches the host issues one after
 // another (3.7 us each), the block solve's n / 64 launches cost more than the sweeps' three from a few
 // hundred rows on; up to 8 right-hand sides and 1024 rows single solves do as batched ones, so that both
 // agree to the bit there.
