@@ -284,6 +284,7 @@ struct Fact {
   int side_ctas = 0;
   // record mode (persistent batched launch): operations are appended here, nothing is launched
   std::vector<BatchOp>* rec = nullptr;
+  bool rec_nodes = false;                // FP32-level TRSM nodes as one operation, for replay()
   // host input (hrp_potrf_host): event of the copy of each 128-column block (rows from the
   // block's diagonal down), and the last block each stream has waited for
   const std::vector<cudaEvent_t>* col_ev = nullptr;
@@ -343,6 +344,7 @@ struct Fact {
   void replay(const BatchOp& o) {
     if (o.type == BOP_POTRF) leaf_potrf(o.a, o.b, o.p);
     else if (o.type == BOP_TRSM) leaf_trsm(o.a, o.b, o.c, o.d, o.p);
+    else if (o.type == BOP_NODE) trsm(o.a, o.b, o.c, o.d, o.p, o.e);
     else gemm(o.p, o.a, o.b, o.c, o.d, o.e, o.f, o.g != 0);
   }
   int tleaf() const { return t->trsm_leaf ? t->trsm_leaf : t->leaf; }
@@ -479,10 +481,55 @@ struct Fact {
       leaf_trsm(r0, m, c0, nc, p);
       return;
     }
+    if (rec && rec_nodes && p == HRP_F32 && nc <= 128 * kPanelLeaves) {
+      rec->push_back(BatchOp{BOP_NODE, p, r0, m, c0, nc, mdec, 0, 0});
+      return;
+    }
+    if (!rec && trsm_node(r0, m, c0, nc, p, mdec)) return;
     int n1 = split(nc);
     trsm(r0, m, c0, n1, p, mdec);
     gemm(p, r0, m, c0 + n1, nc - n1, c0, n1, false);   // B2 -= B1 L21^T
     trsm(r0, m, c0 + n1, nc - n1, p, mdec);
+  }
+
+  // The node in one launch (k_panel.cu), or false: FP32 level on CUDA cores, an inverse for every leaf, and
+  // rows for one pass of its CTAs over the chip (more rows run faster on the separate kernels, whose
+  // larger tiles read less shared memory).
+  bool trsm_node(int r0, int m, int c0, int nc, int p, int mdec) {
+    if (p != HRP_F32 || t->trsm_compute == 1 || !w32 || h32 || nc > 128 * kPanelLeaves) return false;
+    PanelPlan plan;
+    if (!node_units(plan, c0, c0, nc, mdec) || m > panel_max_rows(nc, plan.nleaf, shadow32 != nullptr)) return false;
+    double fl = 0.0;
+    for (int u = 0; u < plan.nunit; ++u) fl += (plan.k[u] == plan.t[u] ? 1.0 : 2.0) * m * plan.sz[plan.k[u]] * plan.sz[plan.t[u]];
+    begin(CLS_TRSM, fl);
+    chk(launch_trsm_panel32(A, lda, r0, m, c0, nc, w32, shadow, lds, shadow32, ld32, info, h->d_err, plan, s));
+    return true;
+  }
+  // the recursion of trsm() over columns c .. c + nc - 1 of the node at c0
+  bool node_units(PanelPlan& plan, int c0, int c, int nc, int mdec) const {
+    if (std::min(mdec, nc) <= tleaf()) {
+      const auto lf = leaves.find(c);
+      if (plan.nleaf == kPanelLeaves || nc > 128 || lf == leaves.end() || lf->second != nc) return false;
+      const int l = plan.nleaf++;
+      plan.off[l] = (short)(c - c0);
+      plan.sz[l] = (short)nc;
+      plan.t[plan.nunit] = plan.k[plan.nunit] = (signed char)l;
+      plan.flag[plan.nunit++] = 3;
+      return true;
+    }
+    const int n1 = split(nc), l0 = plan.nleaf;
+    if (!node_units(plan, c0, c, n1, mdec)) return false;
+    // the update of the right part: its leaves are numbered first, on a copy of the plan
+    const int l1 = plan.nleaf;
+    PanelPlan right = plan;
+    if (!node_units(right, c0, c + n1, nc - n1, mdec)) return false;
+    for (int a = l1; a < right.nleaf; ++a)
+      for (int b = l0; b < l1; ++b) {
+        plan.t[plan.nunit] = (signed char)a;
+        plan.k[plan.nunit] = (signed char)b;
+        plan.flag[plan.nunit++] = (signed char)((b == l0 ? 1 : 0) | (b == l1 - 1 ? 2 : 0));
+      }
+    return node_units(plan, c0, c + n1, nc - n1, mdec);
   }
 
   // Alg. 3 flattened: C = A[c0:c0+nc, c0:c0+nc] (lower) -= X X^T, X = A[c0:c0+nc, a0:a0+k]
@@ -1659,6 +1706,7 @@ cudaError_t issue_factors(int batch, const std::vector<int>& order, const Setup&
     r.i = i;
     if (!setup(i, r.f)) continue;
     r.f.rec = &r.ops;
+    r.f.rec_nodes = true;
     r.f.potrf(0, r.f.n, 0);
     r.f.rec = nullptr;
     ++live;

@@ -113,6 +113,22 @@ cudaError_t launch_trsm_leaf32_subst(double* A, int ld, int r0, int m, int c0, i
 cudaError_t launch_trsm_refine64(double* A, int ld, int r0, int m, int c0, int nc, const float* W, int ldw,
                                  __half* shadow16, int lds, float* shadow32, int ld32, const int* info, unsigned* err,
                                  cudaStream_t s, const double* Lm = nullptr, int ldl = 0);
+// A TRSM node of up to kPanelLeaves diagonal leaves with their FP32 inverses, in one launch (k_panel.cu):
+// B = A[r0.., c0..] (m x nc), leaf l at columns off[l] .. + sz[l] - 1 (sz <= 128), its inverse at W32 +
+// 128 (c0 + off[l]) (ld 128).  Units in order: k == t, solve leaf t; else update leaf t's columns with
+// the solution of leaf k (flag 1: the first of an update's leaves, 2: the last).  Rounding and outputs
+// as launch_trsm_leaf32; updates as launch_gemm_simt at FP32 with operands from S32, or from A if null.
+constexpr int kPanelLeaves = 8;
+constexpr int kPanelUnits = kPanelLeaves * (kPanelLeaves + 1) / 2;
+struct PanelPlan {
+  int nleaf = 0, nunit = 0;
+  short off[kPanelLeaves], sz[kPanelLeaves];
+  signed char t[kPanelUnits], k[kPanelUnits], flag[kPanelUnits];
+};
+// rows at which its CTAs fill the chip once
+int panel_max_rows(int nc, int nleaf, bool shadow32);
+cudaError_t launch_trsm_panel32(double* A, int ld, int r0, int m, int c0, int nc, const float* W32, __half* S, int lds,
+                                float* S32, int ld32, const int* info, unsigned* err, const PanelPlan& plan, cudaStream_t s);
 // FP32 inverses of diagonal blocks of a given lower triangle (a standalone TRSM)
 struct LeafList {
   int count = 0;
@@ -337,7 +353,7 @@ cudaError_t launch_diag_check(const double* A, int lda, int n, double limit, int
 //   BOP_POTRF: leaf POTRF of the diagonal block at offset a, order b, precision p;
 //   BOP_TRSM:  leaf TRSM of rows [a, a+b), columns [c, c+d), FP64 if e else FP32;
 //   BOP_GEMM:  A[a:a+b, c:c+d] -= A[a:a+b, e:e+f] A[c:c+d, e:e+f]^T at precision p, lower if g.
-enum { BOP_POTRF = 1, BOP_TRSM = 2, BOP_GEMM = 3 };
+enum { BOP_POTRF = 1, BOP_TRSM = 2, BOP_GEMM = 3, BOP_NODE = 4 };
 struct BatchOp {
   int type, p, a, b, c, d, e, f, g;
 };
