@@ -49,14 +49,13 @@ struct Smem {
     __half h[kTiles][2][256];          // L0 as binary16 pairs hi + lo 2^-11, row-major with ht()
   } L0;
   __half W0[kTiles][2][256];           // L0^{-1}, pairs
-  __half R[kTiles][2][256];            // R (lower tiles), scaled, pairs
+  __half R[kTiles][2][256];            // R (lower tiles, the diagonal ones whole), scaled, pairs
   __half Tt[2][16][kTtLd];             // T = R W0_J^T, then F, transposed: [column][row]; rows of H
   float Wrow[16][132];                 // rows 16 rank .. of the inverse, binary32
   __half Sbuf[12][2][256];             // phase 1: sums for the off-diagonal blocks of W0, pairs
   float4 xy[16][16];                   // phase 1: the diagonal block's column pairs, rows 2 j, 2 j + 1
   float4 rr[16];                       // phase 1: 1 / l_kk, 1 / l_{k+1,k+1}, l_{k+1,k} of a pair
   int e[128];                          // scales
-  unsigned char tI[kTiles], tJ[kTiles];   // row and column of each lower tile
   unsigned rmax[2], emax[2];           // largest |R| and scaled |E| here (bits), by step parity
 };
 
@@ -164,8 +163,9 @@ __device__ __forceinline__ void tile_pair_mm(float (&c0)[2][4], float (&c1)[2][4
 // Warp 0's lane i holds row i; columns two at a time: every lane forms the pair's pivots (both
 // reciprocal square roots at once, 1 / l_11 = l_00 (a_00 a_11 - a_10^2)^{-1/2}), the lanes' entries of
 // the two columns go through shared memory (16-byte broadcast reads; a shuffle costs four issue slots of the
-// sub-partition) and update the rest.  The next pair's 2 x 2 block is fetched before it is needed,
-// so the chain of a pair is one reciprocal square root and one exchange.  Warp 1's lane c holds column
+// sub-partition) and update the rest, columns 16 .. 31 once for the first sixteen.  The entries that
+// the next pair's pivots need are shuffled instead, and its reciprocal square roots started before
+// the exchange and the update: the chain of a pair is one reciprocal square root and one shuffle.  Warp 1's lane c holds column
 // c of W and applies the same column pairs to it one step behind, told by named barriers 1 .. 15
 // (one per pair: the producer only arrives).  False (warp 0) when a pivot is not positive and finite;
 // both warps pass every barrier in any case.
@@ -187,61 +187,76 @@ __device__ __forceinline__ bool potrf32(Smem& sm, int p, int lane) {
   }
   bool ok = true;
   float d0 = __shfl_sync(full, a[0], 0), q = __shfl_sync(full, a[0], 1), s = __shfl_sync(full, a[1], 1);
+  float det = fmaf(s, d0, -q * q);
+  float r0 = rsqrt_fast(d0), rd = rsqrt_fast(det);
 #pragma unroll
   for (int k = 0; k < 32; k += 2) {
+    const int end = k < 16 ? 16 : 32;            // columns 16 .. 31 get columns 0 .. 15 all at once
     float nd0 = 0.f, nq = 0.f, ns = 0.f;         // the next pair's block before this pair's update
-    if (k + 2 < 32) {
+    if (k + 2 < end) {
       nd0 = __shfl_sync(full, a[k + 2], k + 2);
       nq = __shfl_sync(full, a[k + 2], k + 3);
       ns = __shfl_sync(full, a[k + 3], k + 3);
     }
-    const float det = fmaf(s, d0, -q * q);
-    const float r0 = rsqrt_fast(d0), rd = rsqrt_fast(det);
     ok = ok && d0 > 1e-12f && det > 1e-12f * d0;   // scaled pivots: false for NaN too
     const float m = q * r0, r1 = d0 * r0 * rd;
+    const float4 rr = make_float4(r0, r1, m, 0.f);
     const float x = a[k] * r0;                   // column k of L (rows >= k)
     const float y = fmaf(-x, m, a[k + 1]) * r1;  // column k + 1 (rows > k)
     a[k] = x;
     a[k + 1] = y;
+    if (k + 2 < end) {
+      // the next pair, as far as its reciprocal square roots: the chain
+      const float vx = __shfl_sync(full, x, k + 2), vy = __shfl_sync(full, y, k + 2);
+      const float vz = __shfl_sync(full, x, k + 3), vw = __shfl_sync(full, y, k + 3);
+      d0 = fmaf(-vy, vy, fmaf(-vx, vx, nd0));
+      q = fmaf(-vw, vy, fmaf(-vz, vx, nq));
+      s = fmaf(-vw, vw, fmaf(-vz, vz, ns));
+      det = fmaf(s, d0, -q * q);
+      r0 = rsqrt_fast(d0);
+      rd = rsqrt_fast(det);
+      a[k + 2] = fmaf(-y, vy, fmaf(-x, vx, a[k + 2]));
+      a[k + 3] = fmaf(-y, vw, fmaf(-x, vz, a[k + 3]));
+    }
     reinterpret_cast<float2*>(sm.xy[k >> 1])[lane] = make_float2(x, y);
-    if (lane == 0) sm.rr[k >> 1] = make_float4(r0, r1, m, 0.f);
+    if (lane == 0) sm.rr[k >> 1] = rr;
     __syncwarp();
     if (k < 28) pair_arrive((k >> 1) + 1);       // 15 is the caller's, after the last two pairs
-    if (k + 2 < 32) {
-#pragma unroll
-      for (int j = k + 2; j < 32; j += 2) {
-        const float4 v = sm.xy[k >> 1][j >> 1];  // rows j and j + 1 of the two columns
-        if (j == k + 2) {
-          d0 = fmaf(-v.y, v.y, fmaf(-v.x, v.x, nd0));
-          q = fmaf(-v.w, v.y, fmaf(-v.z, v.x, nq));
-          s = fmaf(-v.w, v.w, fmaf(-v.z, v.z, ns));
-        }
-        a[j] = fmaf(-y, v.y, fmaf(-x, v.x, a[j]));
-        a[j + 1] = fmaf(-y, v.w, fmaf(-x, v.z, a[j + 1]));
-      }
+    if ((k >> 4) <= ti) {                        // the columns as pairs (zero above the diagonal), over the binary32 tile
+      __half2 hi, lo;
+      half_pair2(make_float2(k <= lane ? x : 0.f, k + 1 <= lane ? y : 0.f), hi, lo);
+      __half (*t)[256] = sm.L0.h[tix(2 * p + ti, 2 * p + (k >> 4))];
+      *reinterpret_cast<__half2*>(t[0] + ht(ri, k & 15)) = hi;
+      *reinterpret_cast<__half2*>(t[1] + ht(ri, k & 15)) = lo;
     }
-  }
-  // L as pairs (zero above the diagonal), in place of the binary32 tiles
 #pragma unroll
-  for (int tj = 0; tj < 2; ++tj) {
-    if (tj > ti) continue;
-    __half (*t)[256] = sm.L0.h[tix(2 * p + ti, 2 * p + tj)];
+    for (int j = k + 4; j < end; j += 2) {
+      const float4 v = sm.xy[k >> 1][j >> 1];    // rows j and j + 1 of the two columns
+      a[j] = fmaf(-y, v.y, fmaf(-x, v.x, a[j]));
+      a[j + 1] = fmaf(-y, v.w, fmaf(-x, v.z, a[j + 1]));
+    }
+    if (k == 14) {
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      __half2 hi[4], lo[4];
+      for (int j = 16; j < 32; j += 2)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = 16 * tj + 8 * c + 2 * u;
-        half_pair2(make_float2(j <= lane ? a[j] : 0.f, j + 1 <= lane ? a[j + 1] : 0.f), hi[u], lo[u]);
-      }
-      *reinterpret_cast<uint4*>(t[0] + ht(ri, 8 * c)) = *reinterpret_cast<const uint4*>(hi);
-      *reinterpret_cast<uint4*>(t[1] + ht(ri, 8 * c)) = *reinterpret_cast<const uint4*>(lo);
+        for (int c = 0; c < 16; c += 2) {
+          const float4 v = sm.xy[c >> 1][j >> 1];
+          a[j] = fmaf(-a[c + 1], v.y, fmaf(-a[c], v.x, a[j]));
+          a[j + 1] = fmaf(-a[c + 1], v.w, fmaf(-a[c], v.z, a[j + 1]));
+        }
+      d0 = __shfl_sync(full, a[16], 16);
+      q = __shfl_sync(full, a[16], 17);
+      s = __shfl_sync(full, a[17], 17);
+      det = fmaf(s, d0, -q * q);
+      r0 = rsqrt_fast(d0);
+      rd = rsqrt_fast(det);
     }
   }
   return ok;
 }
 // warp 1: W = L^{-1} of the block as pairs
 __device__ __forceinline__ void inverse32(Smem& sm, int p, int lane) {
+  const int ti = lane >> 4, ri = lane & 15;
   float w[32];
 #pragma unroll
   for (int r = 0; r < 32; ++r) w[r] = r == lane ? 1.f : 0.f;
@@ -251,23 +266,21 @@ __device__ __forceinline__ void inverse32(Smem& sm, int p, int lane) {
     const float4 rr = sm.rr[k >> 1];
     w[k] *= rr.x;
     w[k + 1] = fmaf(-rr.z, w[k], w[k + 1]) * rr.y;
+    if (ti <= (k >> 4)) {                        // rows k and k + 1 are final
+      __half (*t)[256] = sm.W0[tix(2 * p + (k >> 4), 2 * p + ti)];
+      __half2 hi, lo;
+      half_pair2(make_float2(w[k], w[k + 1]), hi, lo);
+      t[0][ht(k & 15, ri)] = __low2half(hi);
+      t[0][ht((k & 15) + 1, ri)] = __high2half(hi);
+      t[1][ht(k & 15, ri)] = __low2half(lo);
+      t[1][ht((k & 15) + 1, ri)] = __high2half(lo);
+    }
 #pragma unroll
     for (int j = k + 2; j < 32; j += 2) {
       const float4 v = sm.xy[k >> 1][j >> 1];
       w[j] = fmaf(-v.y, w[k + 1], fmaf(-v.x, w[k], w[j]));
       w[j + 1] = fmaf(-v.w, w[k + 1], fmaf(-v.z, w[k], w[j + 1]));
     }
-  }
-  const int ti = lane >> 4, ri = lane & 15;
-#pragma unroll
-  for (int r = 0; r < 32; ++r) {
-    const int I = r >> 4;
-    if (ti > I) continue;
-    __half (*t)[256] = sm.W0[tix(2 * p + I, 2 * p + ti)];
-    __half hi, lo;
-    half_pair(w[r], hi, lo);
-    t[0][ht(r & 15, ri)] = hi;
-    t[1][ht(r & 15, ri)] = lo;
   }
 }
 
@@ -510,15 +523,11 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int gi = 16 * uI[x] + (lane >> 2) + 8 * (q >> 1), gj = 16 * uJ[x] + 8 * uH[x] + 2 * (lane & 3) + (q & 1);
-        araw[x][q] = (uI[x] >= 0 && gi < n && gj <= gi) ? A[(size_t)gj * ld + gi] : 0.0;
+        // a diagonal tile's residual is formed whole, from A's lower triangle
+        const int gr = max(gi, gj), gc = min(gi, gj);
+        araw[x][q] = (uI[x] >= 0 && gr < n) ? A[(size_t)gc * ld + gr] : 0.0;
       }
     if (tid < 2) sm.rmax[tid] = sm.emax[tid] = 0;
-    if (tid < kTiles) {
-      int I = 0;
-      while ((I + 1) * (I + 2) / 2 <= tid) ++I;
-      sm.tI[tid] = (unsigned char)I;
-      sm.tJ[tid] = (unsigned char)(tid - I * (I + 1) / 2);
-    }
     if (tid < 128) {
       int e = 0;
       if (tid < n) {
@@ -556,7 +565,7 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
     for (int q = 0; q < 4; ++q) {
       const int gi = 16 * uI[x] + (lane >> 2) + 8 * (q >> 1), gj = 16 * uJ[x] + 8 * uH[x] + 2 * (lane & 3) + (q & 1);
       afix[x][q] = 0;
-      if (gi < n && gj <= gi) afix[x][q] = dig_fix(araw[x][q], sm.e[gi] + sm.e[gj] + 2 + 1022) >> 2;
+      if (gi < n && gj < n) afix[x][q] = dig_fix(araw[x][q], sm.e[gi] + sm.e[gj] + 2 + 1022) >> 2;
       if (gi >= n && gi == gj) afix[x][q] = 1ll << 57;         // 0.5
     }
   }
@@ -592,11 +601,9 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
       float res[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int i = (lane >> 2) + 8 * (q >> 1), j = j0 + 2 * (lane & 3) + (q & 1);
         const long long d = afix[x][q] - sum[q];
         const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
         res[q] = fmaf((float)(unsigned)(a >> 32), 0x1p32f, (float)(unsigned)a) * (d < 0 ? -0x1p-58f : 0x1p-58f);
-        if (I == J && j > i) res[q] = 0.f;                     // above the diagonal (mirrored below)
         mx = fmaxf(mx, fabsf(res[q]));
       }
       float* o = xR + tix(I, J) * 256 + (lane >> 2) * 16 + j0 + 2 * (lane & 3);
@@ -629,25 +636,12 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
         __half2 h0, l0, h1, l1;
         half_pair2(make_float2(g[u].x * fs, g[u].y * fs), h0, l0);
         half_pair2(make_float2(g[u].z * fs, g[u].w * fs), h1, l1);
-        if (sm.tI[t] != sm.tJ[t]) {
-          __half2* p = reinterpret_cast<__half2*>(&sm.R[t][0][ht(i, j)]);
-          p[0] = h0;
-          p[1] = h1;
-          p = reinterpret_cast<__half2*>(&sm.R[t][1][ht(i, j)]);
-          p[0] = l0;
-          p[1] = l1;
-        } else {
-          const __half hi[4] = {__low2half(h0), __high2half(h0), __low2half(h1), __high2half(h1)};
-          const __half lo[4] = {__low2half(l0), __high2half(l0), __low2half(l1), __high2half(l1)};
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (j + q <= i) {
-              sm.R[t][0][ht(i, j + q)] = hi[q];
-              sm.R[t][1][ht(i, j + q)] = lo[q];
-              sm.R[t][0][ht(j + q, i)] = hi[q];
-              sm.R[t][1][ht(j + q, i)] = lo[q];
-            }
-        }
+        __half2* p = reinterpret_cast<__half2*>(&sm.R[t][0][ht(i, j)]);
+        p[0] = h0;
+        p[1] = h1;
+        p = reinterpret_cast<__half2*>(&sm.R[t][1][ht(i, j)]);
+        p[0] = l0;
+        p[1] = l1;
       }
     }
     __syncthreads();
