@@ -35,6 +35,8 @@ namespace {
 // (up to 2^7 units); their difference is below 2^-2 or the rows go to the substitution.
 constexpr int kRFrac = 60;
 constexpr int kMaxPass = 8;
+// the scale of a column whose first X is zero in every row: it must weigh nothing in the rows of L
+constexpr int kNoScale = -4096;
 
 struct T64Layout {                            // byte offsets into dynamic shared memory
   int lx, w, xd, b, r, total, xd_ld, xd_plane;
@@ -255,7 +257,7 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
       // the 16 lanes of this column
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
-      if (rr == 0) s_c[8 * g + cq + q] = ex == INT_MIN ? 0 : ex;
+      if (rr == 0) s_c[8 * g + cq + q] = ex == INT_MIN ? kNoScale : ex;
     }
   }
   bad = __syncthreads_or(bad);
@@ -325,8 +327,10 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
       const int el = s_el[ku];
       float4 w0 = *reinterpret_cast<float4*>(Ws + 8 * u), w1 = *reinterpret_cast<float4*>(Ws + 8 * u + 4);
       const int* cc = s_c + 8 * gu;
-      w0 = make_float4(w0.x * pow2f(el - cc[0]), w0.y * pow2f(el - cc[1]), w0.z * pow2f(el - cc[2]), w0.w * pow2f(el - cc[3]));
-      w1 = make_float4(w1.x * pow2f(el - cc[4]), w1.y * pow2f(el - cc[5]), w1.z * pow2f(el - cc[6]), w1.w * pow2f(el - cc[7]));
+      // columns without a scale take no correction (a residual there goes to the substitution)
+      auto f = [&](int q) { return cc[q] == kNoScale ? 0.f : pow2f(el - cc[q]); };
+      w0 = make_float4(w0.x * f(0), w0.y * f(1), w0.z * f(2), w0.w * f(3));
+      w1 = make_float4(w1.x * f(4), w1.y * f(5), w1.z * f(6), w1.w * f(7));
       *reinterpret_cast<float4*>(Ws + 8 * u) = w0;
       *reinterpret_cast<float4*>(Ws + 8 * u + 4) = w1;
     }
@@ -414,14 +418,14 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
             long long mb = (long long)(((unsigned long long)__double_as_longlong(x) & 0xfffffffffffffull) |
                                        (F ? 0x10000000000000ull : 0ull));
             if (mb != 0 && (sh > 18 || F == 0x7ff)) bad = 1;            // B outside the scales
-            else if (sh >= 0) mb <<= sh;
+            else if (sh >= 0) mb <<= min(sh, 63);
             else mb = (mb + (1ll << (min(-sh, 62) - 1))) >> min(-sh, 62);
             if (__double_as_longlong(x) < 0) mb = -mb;
             // |d| to binary32 by halves (of d itself the halves would cancel)
             const long long d = mb - sum[h][q];
             const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
             res = fmaf((float)(unsigned)(a >> 32), 0x1p32f, (float)(unsigned)a) * (d < 0 ? -0x1p-60f : 0x1p-60f);
-            if (!(fabsf(res) < 0.25f)) bad = 1;
+            if (!(fabsf(res) < 0.25f) || (s_c[j] == kNoScale && res != 0.f)) bad = 1;
           }
           Rs[j * ROWS + r] = res;
         }
