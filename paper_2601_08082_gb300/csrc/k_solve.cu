@@ -13,20 +13,21 @@
 // Both products take 16 rows at a time and up to 512 inner terms, a warp 16 (few rows,
 // solve_step_kernel) or 64 of them (many, solve_wide_kernel).  The entries go from memory to registers
 // in the order the mma fragments want them, are cut into 8-bit digits there and multiplied exactly by
-// 28 mma per 16 terms (digits.cuh); the warps' sums are added in FP64 in a fixed order.  Scales: term k
-// by its largest right-hand side, then a row of P and a column of Y by the largest entry among the
-// warp's terms, so 7 digits keep 55 bits below the largest term of a sum (with several right-hand
-// sides, below the row's times the column's), whatever powers of two scale the unknowns.
+// 28 mma per 16 terms (digits.cuh).  Scales: term k by its largest right-hand side, then a row of P and
+// a column of Y by the largest entry among the terms (of the warp, whose sums are then added in FP64 in
+// a fixed order; in the wide kernel of all, whose sums stay integers until the end), so 7 digits keep
+// 55 bits below the largest term of a sum (with several right-hand sides, below the row's times the
+// column's), whatever powers of two scale the unknowns.
 // What bounds it: latency, 5 us a step with few rows and 8 to 11 us with many (at n = 4096 and one
 // right-hand side 170 us of inverses, most of it the last doubling, then 30 steps); from n = 8192 on the
-// integer work of the wide kernel (~2000 instructions per warp and 16 x 64 entries at two warps per
-// scheduler: 5 us a row tile, issue slots 30 % used).  Solves against the sweeps', us with 1, 4 and 16
-// right-hand sides:
-//   n = 64 18 18 23 (56 60 84), 128 41 41 47 (105 113 140), 2048 233 237 286 (248 365 994),
-//   4 and 16: 4096 427 560 (637 1914), 8192 907 1246 (1204 3794).
+// wide kernel's tiles, 3 to 5 us each of load latency and integer work at two warps per scheduler (with
+// the warps' sums converted and added in FP64, ~2000 instead of ~1600 instructions a tile: n = 4096 560
+// -> 542 us, 8192 1246 -> 1186, 16384 3232 -> 2995 with 16 right-hand sides).  Solves against the
+// sweeps', us with 1, 4 and 16 right-hand sides:
+//   n = 64 18 18 23 (56 60 84), 128 41 41 47 (105 113 140), 2048 231 236 282 (248 365 994),
+//   4 and 16: 4096 421 542 (637 1914), 8192 896 1186 (1204 3794).
 // Backward errors are 3 to 30 times below the sweeps' (whose double-float products keep 44 bits), also
-// for kernel matrices of condition 1e15.  A warp that meets a NaN or an infinity uses FP64 FMAs for its
-// terms.
+// for kernel matrices of condition 1e15.  Tiles that meet a NaN or an infinity use FP64 FMAs.
 #include <cooperative_groups.h>
 
 #include <climits>
@@ -310,7 +311,8 @@ static_assert(kRows * 16 == kThreads, "one output per thread at 16 right-hand si
 
 // O -= P Y for many rows: a warp keeps 64 terms, whose right-hand sides' digits it cuts once and holds in
 // shared memory as mma fragments, and the CTA runs over row tiles, the next tile's entries in flight
-// during the products.
+// during the products.  The warps share the tile's scales (a row's largest entry over all terms, found
+// a tile ahead), so that their sums are added as 64-bit integers and converted once.
 constexpr int kWide = 4;                         // k steps per warp
 template <int NH>
 constexpr int wide_smem() {
@@ -323,86 +325,146 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // by tile modulo 3: a tile's rows are scaled while the one before is multiplied and the words of the one
+  // after it are cleared
+  __shared__ int s_ea[3][kRows], s_special[3];
+  __shared__ int s_ey[8 * NH], s_yspecial;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2;
   uint2 (*bfs)[kDig][NH][32] = reinterpret_cast<uint2 (*)[kDig][NH][32]>(smem) + warp * kWide;     // [s][digit][half][lane]
-  double (*parts)[8][kRows][8 * NH] =
-      reinterpret_cast<double (*)[8][kRows][8 * NH]>(smem + 8 * kWide * kDig * NH * 32 * 8);        // [parity]
+  long long (*parts)[8][kRows][8 * NH] =
+      reinterpret_cast<long long (*)[8][kRows][8 * NH]>(smem + 8 * kWide * kDig * NH * 32 * 8);     // [parity]
   const int k0 = 16 * kWide * warp;
   const bool act = k0 < K;
   const int step = (int)gridDim.x * kRows;
   int r0 = (int)blockIdx.x * kRows;
+  if (tid < 3 * kRows) (&s_ea[0][0])[tid] = INT_MIN;
+  if (tid < 3) s_special[tid] = 0;
+  if (tid < 8 * NH) s_ey[tid] = kNone;
+  if (tid == 0) s_yspecial = 0;
   double a[2][kWide][4];
   if (act) load_rows<TRANS, kWide>(a, P, ldp, r0, rows, k0, K);
   unsigned ek[kWide][2];
   int ey[NH];
-  bool yspecial = false;
+  double y[NH][kWide][4];
+  __syncthreads();
   if (act) {
-    double y[NH][kWide][4];
+    bool special = false;
     load_rhs<NH, kWide>(y, Y, ldy, nrhs, k0, K);
-    rhs_scales<NH, kWide>(y, ek, ey, yspecial);
-    if (!__any_sync(0xffffffffu, yspecial)) {
+    rhs_scales<NH, kWide>(y, ek, ey, special);
+    if ((lane & 3) == 0) {
 #pragma unroll
-      for (int s = 0; s < kWide; ++s) {
-        uint32_t bf[kDig][NH][2];
-        rhs_digits<NH, kWide>(y, ek, ey, s, bf);
+      for (int h = 0; h < NH; ++h) atomicMax(&s_ey[8 * h + g], ey[h]);
+    }
+    if (special) s_yspecial = 1;
+  }
+  auto scale_rows = [&](int buf) {
+    int ea[2];
+    bool special = false;
+    row_scales<kWide>(a, ek, ea, special);
+    if ((lane & 3) == 0) {
+      atomicMax(&s_ea[buf][g], ea[0]);
+      atomicMax(&s_ea[buf][g + 8], ea[1]);
+    }
+    if (special) s_special[buf] = 1;
+  };
+  if (act) scale_rows(0);
+  __syncthreads();
+  if (act && !s_yspecial) {
 #pragma unroll
-        for (int d = 0; d < kDig; ++d)
+    for (int h = 0; h < NH; ++h) ey[h] = s_ey[8 * h + g];
 #pragma unroll
-          for (int h = 0; h < NH; ++h) bfs[s][d][h][lane] = make_uint2(bf[d][h][0], bf[d][h][1]);
-      }
+    for (int s = 0; s < kWide; ++s) {
+      uint32_t bf[kDig][NH][2];
+      rhs_digits<NH, kWide>(y, ek, ey, s, bf);
+#pragma unroll
+      for (int d = 0; d < kDig; ++d)
+#pragma unroll
+        for (int h = 0; h < NH; ++h) bfs[s][d][h][lane] = make_uint2(bf[d][h][0], bf[d][h][1]);
     }
     __syncwarp();
   }
   const int i = tid % kRows, c = tid / kRows;
-  for (int par = 0; r0 < rows; r0 += step, par ^= 1) {
+  for (int t = 0, par = 0, buf = 0; r0 < rows; r0 += step, ++t, par ^= 1) {
     const bool out = c < 8 * NH && r0 + i < rows && c < nrhs;
     double* o = O + (size_t)c * ldo + r0 + i;
     const double o0 = out ? *o : 0.0;
-    double (*part)[8 * NH] = parts[par][warp];
-    if (act) {
-      int ea[2];
-      bool special = yspecial;
-      row_scales<kWide>(a, ek, ea, special);
-      if (__any_sync(0xffffffffu, special)) {
-        plain_sums<NH, TRANS>(P, ldp, r0, rows, Y, ldy, nrhs, [&](int) { return k0; },
-                              [&](int) { return min(K, k0 + 16 * kWide); }, part);
-        if (r0 + step < rows) load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
-      } else {
-        unsigned long long m[kWide][2][4];
-#pragma unroll
-        for (int s = 0; s < kWide; ++s)
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-              m[s][h][j] = (unsigned long long)dig_fix(a[h][s][j], ea[h] - term<kWide>(ek, s, j)) + kByteBias;
-        if (r0 + step < rows) load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
-        float acc[kDig][NH][4] = {};
-#pragma unroll
-        for (int s = 0; s < kWide; ++s) {
-          uint2 bf[kDig][NH];
-#pragma unroll
-          for (int d = 0; d < kDig; ++d)
-#pragma unroll
-            for (int h = 0; h < NH; ++h) bf[d][h] = bfs[s][d][h][lane];
-#pragma unroll
-          for (int d = 0; d < kDig; ++d) {
-            uint32_t af[4];
-            row_fragment(m[s][0], m[s][1], d, af);
-#pragma unroll
-            for (int e = 0; e < kDig - d; ++e)
-#pragma unroll
-              for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h].x, bf[e][h].y);
-          }
-        }
-        store_sums<NH>(acc, ea, ey, part);
+    const int next = buf == 2 ? 0 : buf + 1, after = 3 - buf - next;
+    const bool plain = s_yspecial || s_special[buf];             // the same in every warp
+    const bool more = r0 + step < rows;
+    if (tid < kRows) s_ea[after][tid] = INT_MIN;
+    if (tid == 0) s_special[after] = 0;
+    if (plain) {
+      double (*part)[8 * NH] = reinterpret_cast<double (*)[8 * NH]>(parts[par][warp]);
+      plain_sums<NH, TRANS>(P, ldp, r0, rows, Y, ldy, nrhs, [&](int) { return k0; },
+                            [&](int) { return min(K, k0 + 16 * kWide); }, part);
+      if (act && more) {
+        load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
+        scale_rows(next);
       }
+    } else if (act) {
+      const int ea[2] = {s_ea[buf][g], s_ea[buf][g + 8]};
+      unsigned long long m[kWide][2][4];
+#pragma unroll
+      for (int s = 0; s < kWide; ++s)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            m[s][h][j] = (unsigned long long)dig_fix(a[h][s][j], ea[h] - term<kWide>(ek, s, j)) + kByteBias;
+      if (more) load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
+      float acc[kDig][NH][4] = {};
+#pragma unroll
+      for (int s = 0; s < kWide; ++s) {
+        uint2 bf[kDig][NH];
+#pragma unroll
+        for (int d = 0; d < kDig; ++d)
+#pragma unroll
+          for (int h = 0; h < NH; ++h) bf[d][h] = bfs[s][d][h][lane];
+#pragma unroll
+        for (int d = 0; d < kDig; ++d) {
+          uint32_t af[4];
+          row_fragment(m[s][0], m[s][1], d, af);
+#pragma unroll
+          for (int e = 0; e < kDig - d; ++e)
+#pragma unroll
+            for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h].x, bf[e][h].y);
+        }
+      }
+      // weights 2^(-12 - 8 w) joined in units of 2^-54 (512 terms below 1)
+#pragma unroll
+      for (int h = 0; h < NH; ++h)
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+          long long v[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            long long hi = 0, lo = 0;
+#pragma unroll
+            for (int w = 0; w < 3; ++w) hi = (hi << 8) + __float2int_rn(acc[w][h][q + u]);
+#pragma unroll
+            for (int w = 3; w < kDig; ++w) lo = (lo << 8) + __float2int_rn(acc[w][h][q + u]);
+            v[u] = (hi << 26) + (lo >> 6);
+          }
+          *reinterpret_cast<longlong2*>(&parts[par][warp][g + 4 * q][8 * h + 2 * (lane & 3)]) = make_longlong2(v[0], v[1]);
+        }
+      if (more) scale_rows(next);
     } else {
-      for (int e = lane; e < kRows * 8 * NH; e += 32) part[e / (8 * NH)][e % (8 * NH)] = 0.0;
+      for (int e = lane; e < kRows * 8 * NH; e += 32) parts[par][warp][e / (8 * NH)][e % (8 * NH)] = 0;
     }
     // one barrier per tile: the sums of the next go to the other half
+    const int er = s_ea[buf][i];
     __syncthreads();
-    if (out) *o = o0 - sum_parts<NH>(parts[par], i, c);
+    if (out) {
+      if (plain) {
+        *o = o0 - sum_parts<NH>(reinterpret_cast<const double (*)[kRows][8 * NH]>(parts[par]), i, c);
+      } else {
+        long long v = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += parts[par][w][i][c];
+        *o = o0 - dig_to_double(v, er + s_ey[c] - 2 * 1022 - 54);
+      }
+    }
+    buf = next;
   }
 }
 
