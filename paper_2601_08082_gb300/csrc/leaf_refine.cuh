@@ -776,6 +776,7 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
       // W = W0 + H W0, H = I - W0 L (a Newton step on the inverse), rows 16 rank ..: L = L0 plus the
       // first correction; every product down to 2^-32, the sums of magnitude 1 start from -I
       const int C = warp;
+      const bool delta = mx > 0.f && !good;                    // else the correction is below 2^-33 and R still the residual
       if (C <= rank) {
         float c0[2][4] = {}, c1[2][4] = {}, c2[2][4] = {};
         uint32_t ah[4], al[4], bh[4], bl[4], bd[4];
@@ -792,11 +793,11 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
           frag<Op::Bt>(bh, sm.L0.h[tix(K, C)][0], lane);
           frag<Op::Bt>(bl, sm.L0.h[tix(K, C)][1], lane);
           pair_mm(c0, c1, ah, al, bh, bl);
-          if (mx > 0.f) frag<Op::Bt>(bd, sm.R[tix(K, C)][0], lane);
+          if (delta) frag<Op::Bt>(bd, sm.R[tix(K, C)][0], lane);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             dig_mma(c2[h], al, bl[2 * h], bl[2 * h + 1]);
-            if (mx > 0.f) dig_mma(c2[h], ah, bd[2 * h], bd[2 * h + 1]);
+            if (delta) dig_mma(c2[h], ah, bd[2 * h], bd[2 * h + 1]);
           }
         }
         // -H times 2^16 as one binary16 plane, rows of H
