@@ -40,12 +40,17 @@ METRIC = "POTRF TFLOP/s (n^3/3 per s) mixed vs FP64 tree on GB300 at stated back
 FP64_MEASURED_TFLOPS = 1.20
 FP32_MEASURED_TFLOPS = 75.2
 # DRAM bytes (read + write) per launch of the leaf POTRF kernel from one ncu capture, reported
-# while the kernel's device code is the code captured: the source up to its launcher, hashed.
-LEAF_TRAFFIC = {"bytes": 162176, "source": "paper_2601_08082_gb300/csrc/k_leaf_cluster.cu",
-                "until": "cudaError_t launch_potrf_leaf_cluster(", "sha1": "c1833c238d6246960dce60c58aa7a6d40dfe023a"}
-# The leaves of trees with a level below FP64 run in double-float arithmetic on the FP32 pipe:
-# one double-float multiply-add (the Dot2 accumulation step of the tile updates) is 12 FP32
-# instructions, so FP64-class work done that way peaks at the FP32 rate / 12.
+# while the kernel's device code is the code captured: its sources (the first up to the launcher),
+# hashed.
+LEAF_TRAFFIC = {"bytes": 246144, "sources": [
+    ("paper_2601_08082_gb300/csrc/k_leaf_cluster.cu", "cudaError_t launch_potrf_leaf_cluster(",
+     "05eebf399f6f05f6004264c9a307ba2179178c67"),
+    ("paper_2601_08082_gb300/csrc/leaf_refine.cuh", "}  // namespace leafref",
+     "7ae23e0bb92880bce7ba12789ae2eb5046d57841")]}
+# The leaves' yardstick in trees with a level below FP64 is double-float arithmetic on the FP32 pipe
+# (their direct schedule; the refinement that runs first does the work as digit products): one
+# double-float multiply-add (the Dot2 accumulation step of the tile updates) is 12 FP32 instructions,
+# so FP64-class work done that way peaks at the FP32 rate / 12.
 DF_OPS_PER_FMA = 12
 
 
@@ -62,7 +67,8 @@ def leaf_traffic():
     if LEAF_TRAFFIC["bytes"] is None:
         return None
     try:
-        ok = device_code_sha1(os.path.join(ROOT, LEAF_TRAFFIC["source"]), LEAF_TRAFFIC["until"]) == LEAF_TRAFFIC["sha1"]
+        ok = all(device_code_sha1(os.path.join(ROOT, path), until) == sha1
+                 for path, until, sha1 in LEAF_TRAFFIC["sources"])
     except OSError:
         ok = False
     return LEAF_TRAFFIC["bytes"] if ok else None
