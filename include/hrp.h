@@ -135,7 +135,7 @@ hrp_status hrp_potrf_async(hrp_handle* h, const hrp_tree* tree, int n, double* d
  * Solve A X = B given the factor from hrp_potrf (L in the lower triangle of dL):
  * forward substitution L Y = B, then backward L^T X = Y, with FP64 storage and sums.  Two
  * ways, both off GB300's slow FP64 pipe:
- *   - n <= 256, more than 8 right-hand sides, or n > 1024 (one right-hand side: up to 3072):
+ *   - n <= 512, more than 8 right-hand sides, or n > 1024 (one right-hand side: up to 3072):
  *     with FP64 inverses of the diagonal blocks of up to 512 rows, products exact to 2^-55 of
  *     the largest term (with several right-hand sides, of the row's times the column's largest);
  *   - otherwise, and where the device's memory does not hold those inverses (6.3 KB per row):
@@ -344,7 +344,7 @@ hrp_status hrp_autotune(hrp_handle* h, const hrp_tree* tree, int n, int reps, in
 hrp_status hrp_potrf_batched(hrp_handle* h, const hrp_tree* const* trees, int batch, const int* n,
                              double* const* dA, const int* lda, int* d_info, void* stream);
 /*
- * Batched POTRS (FP64; by block inverses up to n[i] = 256, above that the double-float sweeps):
+ * Batched POTRS (FP64; by block inverses up to n[i] = 512, above that the double-float sweeps):
  * for each i, dB[i] (n[i] x nrhs, ldb[i]) <- A_i^{-1} dB[i] with the factor in the lower
  * triangle of dL[i].  Same stream pool and capture rules as above.
  */

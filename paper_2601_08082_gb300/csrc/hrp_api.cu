@@ -1956,21 +1956,26 @@ hrp_status hrp_potrs_batched(hrp_handle* h, int batch, const int* n, double* con
   if ((st = fork(h, s)) != HRP_OK) return st;
   cudaError_t err = cudaSuccess;
   long long launches = 0;
-  for (int i = 0; i < batch; ++i) {
-    if (n[i] == 0) continue;
-    cudaStream_t si = h->bstreams[which[i]];
-    cudaError_t e;
-    if (n[i] <= kSolveSmall) {
-      e = launch_solve_inverses(dL[i], ldl[i], n[i], h->bwork + ws[i].swork, si);
-      if (e == cudaSuccess) e = launch_solve(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, h->bwork + ws[i].swork, si);
-      launches += solve_launches(n[i], nrhs, true);
-    } else {
-      e = launch_potrs(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, false, h->bwork + ws[i].pinv,
-                       reinterpret_cast<int*>(h->bwork + ws[i].ticket), h->d_err, si, h->wait_ns);
-      launches += 1 + potrs_sweeps(nrhs);
+  // longest first; the sweeps and the block inverses of all systems, then the solves with the inverses
+  const std::vector<int> order = longest_first(batch, n);
+  for (int part = 0; part < 2; ++part)
+    for (int i : order) {
+      if (n[i] == 0) continue;
+      cudaStream_t si = h->bstreams[which[i]];
+      cudaError_t e = cudaSuccess;
+      if (n[i] > kSolveSmall) {
+        if (part == 1) continue;
+        e = launch_potrs(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, false, h->bwork + ws[i].pinv,
+                         reinterpret_cast<int*>(h->bwork + ws[i].ticket), h->d_err, si, h->wait_ns);
+        launches += 1 + potrs_sweeps(nrhs);
+      } else if (part == 0) {
+        e = launch_solve_inverses(dL[i], ldl[i], n[i], h->bwork + ws[i].swork, si);
+      } else {
+        e = launch_solve(dL[i], ldl[i], dB[i], ldb[i], n[i], nrhs, h->bwork + ws[i].swork, si);
+        launches += solve_launches(n[i], nrhs, true);
+      }
+      if (e != cudaSuccess && err == cudaSuccess) err = e;
     }
-    if (e != cudaSuccess && err == cudaSuccess) err = e;
-  }
   if ((st = join(h, s)) != HRP_OK) return st;
   h->launches = launches;
   return cuda_status(h, err, "hrp_potrs_batched");

@@ -263,7 +263,7 @@ cudaError_t launch_solve(const double* L, int ldl, double* B, int ldb, int n, in
 // whether a single solve takes the block inverses rather than the sweeps; a batched one does up to
 // kSolveSmall
 bool solve_blocked(int n, int nrhs);
-constexpr int kSolveSmall = 256;
+constexpr int kSolveSmall = 512;
 // their launches (nrhs = 0: of the inverses alone)
 int solve_launches(int n, int nrhs, bool inverses);
 

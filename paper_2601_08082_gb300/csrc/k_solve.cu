@@ -574,11 +574,12 @@ cudaError_t launch_solve(const double* L, int ldl, double* B, int ldb, int n, in
 }
 
 // Single solves gain at every size (figures above) but with one right-hand side on large factors, whose
-// sweeps read L once and whose links are short: n = 2048 233 us against 248, 4096 about equal (418),
-// 8192 870 against 794.  In a batch, whose systems overlap on streams and whose launches the host issues one after
-// another (3.7 us each), the block solve's n / 64 launches cost more than the sweeps' three from a few
-// hundred rows on; up to 8 right-hand sides and 1024 rows single solves do as batched ones, so that both
-// agree to the bit there.
+// sweeps read L once and whose links are short: n = 2048 231 us against 248, 4096 about equal (418),
+// 8192 870 against 794.  In a batch, whose systems overlap on streams, the launches count: 24 FP64
+// systems of 64 .. 1024, factored and solved with 4 right-hand sides, take 3.01 ms with the block solve up
+// to 256 rows, 2.91 up to 512, 3.31 up to 1024.  Up to 8 right-hand sides and 1024 rows single solves do as
+// batched ones, so that both agree to the bit there (at 1024 rows that costs a single solve 45 us of
+// 175, at 512 the blocks take 88 us against 133).
 bool solve_blocked(int n, int nrhs) { return n <= kSolveSmall || nrhs > 8 || (n > 1024 && (nrhs > 1 || n <= 3072)); }
 
 int solve_launches(int n, int nrhs, bool inverses) {

@@ -1,4 +1,4 @@
-"""POTRS by block inverses (orders up to 256 or above 1024, or more than 8 right-hand sides): edges of the
+"""POTRS by block inverses (orders up to 512 or above 1024, or more than 8 right-hand sides): edges of the
 64-, 128-, 256- and 512-row blocks and of the groups of 8 and 16 right-hand sides, ragged leading
 dimensions, rows scaled by powers of two from 2^-60 to 2^60, and a NaN in one right-hand side.
 
@@ -10,7 +10,7 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-CASES = [(n, r) for n in (1, 63, 64, 65, 127, 128) for r in (1, 8)]
+CASES = [(n, r) for n in (1, 63, 64, 65, 127, 128, 256, 257, 512) for r in (1, 8)]
 CASES += [(n, r) for n in (129, 255, 257, 512, 513, 1024) for r in (9, 17)]
 CASES += [(n, r) for n in (1025, 1537) for r in (1, 3, 16)] + [(4096, 3), (4096, 16)]
 
