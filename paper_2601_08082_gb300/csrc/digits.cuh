@@ -10,9 +10,14 @@
 // it).  The digit products d_s d_t are integers of at most 2^16; those of one weight s + t = g
 // <= 6 are summed by the tensor cores in FP32, exactly: at most 7 pairs x 32 terms x 2^16 < 2^24
 // per chunk of 32 inner terms (checked against 64-bit integers on the device for the largest
-// magnitudes).  Chunk sums are then carried in 32-bit integers.  The dropped pairs (g > 6) and
-// the digits' tails are below 2^-62 of the two scales' product per term, so the only rounding
-// that shows is the final one to FP64.
+// magnitudes).  Chunk sums are then carried in 32-bit integers.  Per term, the dropped pairs (six of
+// weight 7: 2^-60.4) and the digits' tails (2^-62 each) are below 2^-59.7 of the two scales' product.
+//
+// A scale is shared by the terms of a row, and the error is relative to it: FP64 sums give every term its
+// own exponent, a digit product does not.  An output whose terms are all far below its row's scale times
+// its column's (rows or columns in different units) would lose the digits that matter, so the kernels
+// also sum bfloat16 magnitudes (dig_abs), an estimate of sum |x| |y| against the same scales, and
+// compute by FP64 FMAs the outputs where it is too small.
 #pragma once
 #include <stdint.h>
 
@@ -23,7 +28,7 @@ namespace hrp {
 constexpr int kDig = 7;        // digits per operand, and weights s + t = 0 .. 6 kept
 constexpr int kDigK = 32;      // inner terms per chunk (exactness bound above)
 constexpr int kDigLd = 40;     // halves per staged row of 32: 80 bytes, conflict-free for ldmatrix
-constexpr int kDigHead = 2;    // bits of headroom of a row's scale over its largest entry so far
+constexpr int kDigHead = 1;    // bits of headroom of a row's scale over its largest entry so far
 
 __device__ __forceinline__ int dig_field(double x) {         // biased exponent field
   return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff;
@@ -81,6 +86,22 @@ __device__ __forceinline__ void dig_split8(const double (&v)[8], int eb, __half*
   dig_split8(v, e, dst, plane);
 }
 
+// |x| against the same scale as a bfloat16, truncated, not below 2^-60 unless x is zero: the operands
+// of the estimate of sum |x| |y| that tells which outputs the digits cover.  A sum of such products
+// is zero only where every product is.
+constexpr int kAbsMin = (127 - 60) << 7;
+__device__ __forceinline__ uint32_t dig_abs(double x, int eb) {
+  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  const int b = max((int)(h >> 13) + ((126 - eb) << 7), kAbsMin);
+  return (h | (uint32_t)__double2loint(x)) ? (uint32_t)b : 0u;
+}
+__device__ __forceinline__ void dig_abs8(const double (&v)[8], const int (&eb)[8], __half* dst) {
+  uint32_t w[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) w[p] = dig_abs(v[2 * p], eb[2 * p]) | (dig_abs(v[2 * p + 1], eb[2 * p + 1]) << 16);
+  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 __device__ __forceinline__ void dig_ldmatrix(uint32_t (&r)[4], const __half* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -100,11 +121,20 @@ __device__ __forceinline__ void dig_mma(float (&d)[4], const uint32_t (&a)[4], u
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void dig_mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 // One chunk of a warp's 16 x 16 output: rows a0 .. a0 + 15 of the staged digits A ([s][row][k],
 // `aplane` halves per digit), columns = rows b0 .. b0 + 15 of B.  The weights' sums over the
-// chunk are added to iacc[g][j], j = 4 (column half) + the mma accumulator's register.
+// chunk are added to iacc[g][j], j = 4 (column half) + the mma accumulator's register, and those of
+// the bfloat16 magnitudes (EST: plane kDig of both operands) to est.
+template <bool EST>
 __device__ __forceinline__ void dig_chunk(const __half* A, int aplane, int a0, const __half* B, int bplane, int b0,
-                                          int (&iacc)[kDig][8]) {
+                                          int (&iacc)[kDig][8], float (&est)[2][4]) {
   const int lane = threadIdx.x & 31;
   float acc[kDig][2][4];
 #pragma unroll
@@ -119,6 +149,13 @@ __device__ __forceinline__ void dig_chunk(const __half* A, int aplane, int a0, c
   const __half* bp = B + (size_t)(b0 + (lane & 7) + ((lane >> 4) << 3)) * kDigLd + ((lane >> 3) & 1) * 8;
 #pragma unroll
   for (int ks = 0; ks < kDigK; ks += 16) {
+    if (EST) {
+      uint32_t a[4], e[4];
+      dig_ldmatrix(a, ap + (size_t)kDig * aplane + ks);
+      dig_ldmatrix(e, bp + (size_t)kDig * bplane + ks);
+      dig_mma_bf16(est[0], a, e[0], e[1]);
+      dig_mma_bf16(est[1], a, e[2], e[3]);
+    }
     uint32_t b[kDig][4];
 #pragma unroll
     for (int t = 0; t < kDig; ++t) dig_ldmatrix(b[t], bp + (size_t)t * bplane + ks);

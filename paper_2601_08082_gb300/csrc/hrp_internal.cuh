@@ -190,7 +190,7 @@ inline int gemm_block_offsets(GemmBlocks& bl, int t) {
   }
   return tiles;
 }
-// FP64 products of a list of blocks (k_gemm_f64.cu), with the accuracy of FP64 or better
+// FP64 products of a list of blocks (k_gemm_f64.cu); every entry is accurate against its own sum |x| |y|
 cudaError_t launch_gemm_f64_blocks(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, int k,
                                    GemmBlocks& bl, cudaStream_t s);
 // Independent products C[co ..] = X[xo ..] Y[yo ..]^T (m x n, inner dimension k; offsets in elements), or

@@ -4,7 +4,7 @@
 //
 // One CTA of 4 warps computes one 32 x 32 tile (a warp 16 x 16).  Per chunk of 32 inner terms the
 // CTA loads its 64 operand rows from the master (coalesced along rows), takes the rows' largest
-// exponents, writes the digits to shared memory (36 KB) and multiplies them; the next chunk's
+// exponents, writes the digits and magnitudes to shared memory (41 KB) and multiplies them; the next chunk's
 // loads are in flight during the products.  What bounds it: 56 mma per warp and 16 terms (8 clocks
 // each per sub-partition) against ~45 integer instructions per entry of splitting; two or three
 // CTAs per SM overlap the two.  The small tile is for the small products this library runs in
@@ -16,10 +16,18 @@
 // 2.58 -> 1.96 ms.  Relative error against extended precision 5e-17 .. 7e-17, where the FMA
 // chains had 1.2e-16 (k = 16) .. 8.5e-16 (k = 1000).
 //
-// A row's scale carries 2 bits of headroom over its largest entry so far.  When a later chunk
+// A row's scale carries a bit of headroom over its largest entry so far.  When a later chunk
 // holds a larger entry still, the CTA moves its integer sums to FP64 first (at the old scales)
 // and goes on with the new ones.  A tile whose operand rows hold a NaN or an infinity is computed
 // by plain FP64 FMAs instead, so that those propagate as they would there.
+//
+// Outputs that the digits do not cover.  A term is held to 2^-59.7 of the product of the two rows'
+// scales; where sum |x| |y| (estimated beside the digit products, two mma per warp and 16 terms)
+// is below 2^-8 of that product, the output is computed by FP64 FMAs, by the warp's lanes together for up to
+// four lanes' outputs, else for the warp's whole part.  The rest is then within k 2^-51.7 sum |x| |y| at
+// worst, and a few 2^-53 sum |x| |y| for ordinary digits.  The line: factors of dominant matrices stay
+// 2^4 above it and those of kernel matrices 2^0 to 2^3; one bit of headroom instead of two (and 2^-10)
+// costs no time.  The estimate costs 2 to 2.5 % (the SYRK 424 -> 435 us, n = 1024 1434 -> 1463).
 #include "digits.cuh"
 #include "hrp_internal.cuh"
 
@@ -30,6 +38,8 @@ constexpr int kT = 32;                         // tile edge
 constexpr int kThreads = 128;
 constexpr int kPlane = kT * kDigLd;            // halves per digit plane of one operand
 constexpr int kSpecial = 1 << 20;              // OPs 1 and 2: the exponent of a NaN or an infinity
+constexpr float kCovered = 0x1p-8f;            // smallest sum |x| |y| against the scales that the digits cover
+constexpr int kManyLow = 4;                    // lanes with uncovered outputs above which the warp computes all by FMAs
 constexpr int kFlush = 64;                     // chunks the 32-bit sums hold (2^24 each) before a move to FP64
 
 // OP 0: C -= X Y^T.  OP 1: C = X Y^T with term kk of X's row r zero for kk < r.  OP 2: C = -X Y^T with Y
@@ -44,7 +54,9 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
                        const double* __restrict__ Y, int ldy, int k, const __grid_constant__ List bl) {
   pdl_wait();
   pdl_trigger();
-  extern __shared__ __align__(16) __half dig[];                  // [2 operands][7][32][kDigLd]
+  constexpr bool EST = OP == 0;
+  constexpr int kOperand = (kDig + EST) * kPlane;                // halves of one operand
+  extern __shared__ __align__(16) __half dig[];                  // [2 operands][7 digits, magnitude][32][kDigLd]
   __shared__ int rowmax[2][2 * kT];                              // largest exponent field of the chunk, by parity
   __shared__ int scale[2 * kT];                                  // the rows' scales (biased exponent)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -93,6 +105,7 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
     }
   };
   int iacc[kDig][8];
+  float est[2][4] = {};                                          // sum |x| |y| against the scales
   double vacc[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -156,53 +169,103 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
         flushed = true;
         held = 0;
       }
+      int old[2][2][2];                                          // [row half][column half][column]
+      if (EST) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) old[(j >> 1) & 1][j >> 2][j & 1] = scale[gr + 8 * ((j >> 1) & 1)] + scale[kT + gc + 8 * (j >> 2) + (j & 1)];
+      }
       __syncthreads();
       if (need) scale[tid] = max(mx, 1) + kDigHead;
       __syncthreads();
+      if (EST) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int d = old[(j >> 1) & 1][j >> 2][j & 1] - scale[gr + 8 * ((j >> 1) & 1)] - scale[kT + gc + 8 * (j >> 2) + (j & 1)];
+          float& t = est[j >> 2][j & 3];
+          if (t > 0.f) t = fmaxf(t * __int_as_float((max(d, -126) + 127) << 23), 0x1p-126f);      // zero means none
+        }
+      }
     }
-    if constexpr (OP != 0) {
+    {
       int ex[8], ey[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        ex[q] = scale[lane] - tk[q];
-        ey[q] = scale[kT + lane] + tk[q];
+        ex[q] = scale[lane] - (OP == 0 ? 0 : tk[q]);
+        ey[q] = scale[kT + lane] + (OP == 0 ? 0 : tk[q]);
       }
-      dig_split8(px, ex, dig + lane * kDigLd + 8 * warp, kPlane);
-      dig_split8(py, ey, dig + kDig * kPlane + lane * kDigLd + 8 * warp, kPlane);
-    } else {
-      dig_split8(px, scale[lane], dig + lane * kDigLd + 8 * warp, kPlane);
-      dig_split8(py, scale[kT + lane], dig + kDig * kPlane + lane * kDigLd + 8 * warp, kPlane);
+      __half* dx = dig + lane * kDigLd + 8 * warp;
+      dig_split8(px, ex, dx, kPlane);
+      dig_split8(py, ey, dx + kOperand, kPlane);
+      if (EST) {
+        dig_abs8(px, ex, dx + kDig * kPlane);
+        dig_abs8(py, ey, dx + kOperand + kDig * kPlane);
+      }
     }
     if (c + 1 < nchunk) fetch((c + 1) * kDigK);
     __syncthreads();
-    dig_chunk(dig, kPlane, a0, dig + kDig * kPlane, kPlane, b0, iacc);
+    dig_chunk<EST>(dig, kPlane, a0, dig + kOperand, kPlane, b0, iacc, est);
     ++held;
   }
-  if (special) {
+  // outputs whose terms are all too far below the scales of their row and column
+  unsigned low = 0;
+  if (EST && !special) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
-      if (r >= m || cl >= n || (lower && r < cl)) continue;
-      double s = 0.0;
-      for (int kk = 0; kk < k; ++kk)
-        s = fma(Xb[(size_t)kk * ldx + r], OP == 2 ? Yb[(size_t)cl * ldy + kk] : Yb[(size_t)kk * ldy + cl], s);
-      double* p = Cb + (size_t)cl * ldc + r;
-      if (OP == 0) *p -= s;
-      else *p = OP == 1 ? s : -s;
+      const float t = est[j >> 2][j & 3];
+      if (r < m && cl < n && !(lower && r < cl) && t > 0.f && t < kCovered) low |= 1u << j;
+    }
+    special = __popc(__ballot_sync(0xffffffffu, low != 0)) > kManyLow;       // this warp's part
+  }
+  auto yv = [&](int cl, int kk) { return OP == 2 ? Yb[(size_t)cl * ldy + kk] : Yb[(size_t)kk * ldy + cl]; };
+  auto store = [&](int r, int cl, double s) {
+    double* p = Cb + (size_t)cl * ldc + r;
+    if (OP == 0) *p -= s;
+    else *p = OP == 1 ? s : -s;
+  };
+  if (special) {
+    double s[8] = {};
+    for (int kk = 0; kk < k; ++kk) {
+      double x[2], y[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) x[h] = Xb[(size_t)kk * ldx + min(m0 + gr + 8 * h, m - 1)];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) y[h] = yv(min(n0 + gc + 8 * (h >> 1) + (h & 1), n - 1), kk);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) s[j] = fma(x[(j >> 1) & 1], y[2 * (j >> 2) + (j & 1)], s[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
+      if (r < m && cl < n && !(lower && r < cl)) store(r, cl, s[j]);
     }
     return;
+  }
+  if (EST && __any_sync(0xffffffffu, low != 0)) {
+    // a few: FP64 FMAs by the whole warp, the terms over its lanes
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j)
+      for (unsigned who = __ballot_sync(0xffffffffu, (low >> j) & 1); who; who &= who - 1) {
+        const int src = __ffs(who) - 1;
+        const int r = m0 + a0 + (src >> 2) + 8 * ((j >> 1) & 1), cl = n0 + b0 + 2 * (src & 3) + 8 * (j >> 2) + (j & 1);
+        double s = 0.0;
+        for (int kk = lane; kk < k; kk += 32) s = fma(Xb[(size_t)kk * ldx + r], yv(cl, kk), s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) store(r, cl, s);
+      }
   }
   double cv[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
-    cv[j] = (OP == 0 && r < m && cl < n && !(lower && r < cl)) ? Cb[(size_t)cl * ldc + r] : 0.0;
+    cv[j] = (OP == 0 && r < m && cl < n && !(lower && r < cl) && !((low >> j) & 1)) ? Cb[(size_t)cl * ldc + r] : 0.0;
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int rr = gr + 8 * ((j >> 1) & 1), cc = gc + 8 * (j >> 2) + (j & 1);
     const int r = m0 + rr, cl = n0 + cc;
-    if (r >= m || cl >= n || (lower && r < cl)) continue;
+    if (r >= m || cl >= n || (lower && r < cl) || ((low >> j) & 1)) continue;
     double f0, f1;
     dig_scale(scale[rr], scale[kT + cc], f0, f1);
     double v = dig_value(iacc, j);
@@ -220,7 +283,7 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
 
 }  // namespace
 
-constexpr int kSmem = 2 * kDig * kPlane * (int)sizeof(__half);
+constexpr int kSmem = 2 * (kDig + 1) * kPlane * (int)sizeof(__half);
 
 cudaError_t launch_gemm_f64_blocks(double* C, int ldc, const double* X, int ldx, const double* Y, int ldy, int k,
                                    GemmBlocks& bl, cudaStream_t s) {
