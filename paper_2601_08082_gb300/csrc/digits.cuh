@@ -131,8 +131,7 @@ __device__ __forceinline__ void dig_mma_bf16(float (&d)[4], const uint32_t (&a)[
 // One chunk of a warp's 16 x 16 output: rows a0 .. a0 + 15 of the staged digits A ([s][row][k],
 // `aplane` halves per digit), columns = rows b0 .. b0 + 15 of B.  The weights' sums over the
 // chunk are added to iacc[g][j], j = 4 (column half) + the mma accumulator's register, and those of
-// the bfloat16 magnitudes (EST: plane kDig of both operands) to est.
-template <bool EST>
+// the bfloat16 magnitudes (plane kDig of both operands) to est.
 __device__ __forceinline__ void dig_chunk(const __half* A, int aplane, int a0, const __half* B, int bplane, int b0,
                                           int (&iacc)[kDig][8], float (&est)[2][4]) {
   const int lane = threadIdx.x & 31;
@@ -149,7 +148,7 @@ __device__ __forceinline__ void dig_chunk(const __half* A, int aplane, int a0, c
   const __half* bp = B + (size_t)(b0 + (lane & 7) + ((lane >> 4) << 3)) * kDigLd + ((lane >> 3) & 1) * 8;
 #pragma unroll
   for (int ks = 0; ks < kDigK; ks += 16) {
-    if (EST) {
+    {
       uint32_t a[4], e[4];
       dig_ldmatrix(a, ap + (size_t)kDig * aplane + ks);
       dig_ldmatrix(e, bp + (size_t)kDig * bplane + ks);

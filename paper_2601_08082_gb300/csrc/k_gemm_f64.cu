@@ -27,7 +27,9 @@
 // four lanes' outputs, else for the warp's whole part.  The rest is then within k 2^-51.7 sum |x| |y| at
 // worst, and a few 2^-53 sum |x| |y| for ordinary digits.  The line: factors of dominant matrices stay
 // 2^4 above it and those of kernel matrices 2^0 to 2^3; one bit of headroom instead of two (and 2^-10)
-// costs no time.  The estimate costs 2 to 2.5 % (the SYRK 424 -> 435 us, n = 1024 1434 -> 1463).
+// costs no time.  OPs 1 and 2 take 2^-14: their triangle's rows are mostly their diagonal entry, and one
+// output in 100 of an ordinary factor is below 2^-10, one in 10^4 below 2^-14, where ordinary digits
+// still leave 2^-46 (the sweeps' double-float products 2^-44).  The estimate costs 2 to 2.5 % (the SYRK 424 -> 435 us, n = 1024 1434 -> 1463).
 #include "digits.cuh"
 #include "hrp_internal.cuh"
 
@@ -39,6 +41,7 @@ constexpr int kThreads = 128;
 constexpr int kPlane = kT * kDigLd;            // halves per digit plane of one operand
 constexpr int kSpecial = 1 << 20;              // OPs 1 and 2: the exponent of a NaN or an infinity
 constexpr float kCovered = 0x1p-8f;            // smallest sum |x| |y| against the scales that the digits cover
+constexpr float kCoveredInv = 0x1p-14f;        // the same in OPs 1 and 2
 constexpr int kManyLow = 4;                    // lanes with uncovered outputs above which the warp computes all by FMAs
 constexpr int kFlush = 64;                     // chunks the 32-bit sums hold (2^24 each) before a move to FP64
 
@@ -54,8 +57,7 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
                        const double* __restrict__ Y, int ldy, int k, const __grid_constant__ List bl) {
   pdl_wait();
   pdl_trigger();
-  constexpr bool EST = OP == 0;
-  constexpr int kOperand = (kDig + EST) * kPlane;                // halves of one operand
+  constexpr int kOperand = (kDig + 1) * kPlane;                  // halves of one operand
   extern __shared__ __align__(16) __half dig[];                  // [2 operands][7 digits, magnitude][32][kDigLd]
   __shared__ int rowmax[2][2 * kT];                              // largest exponent field of the chunk, by parity
   __shared__ int scale[2 * kT];                                  // the rows' scales (biased exponent)
@@ -170,20 +172,16 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
         held = 0;
       }
       int old[2][2][2];                                          // [row half][column half][column]
-      if (EST) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) old[(j >> 1) & 1][j >> 2][j & 1] = scale[gr + 8 * ((j >> 1) & 1)] + scale[kT + gc + 8 * (j >> 2) + (j & 1)];
-      }
+      for (int j = 0; j < 8; ++j) old[(j >> 1) & 1][j >> 2][j & 1] = scale[gr + 8 * ((j >> 1) & 1)] + scale[kT + gc + 8 * (j >> 2) + (j & 1)];
       __syncthreads();
       if (need) scale[tid] = max(mx, 1) + kDigHead;
       __syncthreads();
-      if (EST) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int d = old[(j >> 1) & 1][j >> 2][j & 1] - scale[gr + 8 * ((j >> 1) & 1)] - scale[kT + gc + 8 * (j >> 2) + (j & 1)];
-          float& t = est[j >> 2][j & 3];
-          if (t > 0.f) t = fmaxf(t * __int_as_float((max(d, -126) + 127) << 23), 0x1p-126f);      // zero means none
-        }
+      for (int j = 0; j < 8; ++j) {
+        const int d = old[(j >> 1) & 1][j >> 2][j & 1] - scale[gr + 8 * ((j >> 1) & 1)] - scale[kT + gc + 8 * (j >> 2) + (j & 1)];
+        float& t = est[j >> 2][j & 3];
+        if (t > 0.f) t = fmaxf(t * __int_as_float((max(d, -126) + 127) << 23), 0x1p-126f);        // zero means none
       }
     }
     {
@@ -196,24 +194,22 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
       __half* dx = dig + lane * kDigLd + 8 * warp;
       dig_split8(px, ex, dx, kPlane);
       dig_split8(py, ey, dx + kOperand, kPlane);
-      if (EST) {
-        dig_abs8(px, ex, dx + kDig * kPlane);
-        dig_abs8(py, ey, dx + kOperand + kDig * kPlane);
-      }
+      dig_abs8(px, ex, dx + kDig * kPlane);
+      dig_abs8(py, ey, dx + kOperand + kDig * kPlane);
     }
     if (c + 1 < nchunk) fetch((c + 1) * kDigK);
     __syncthreads();
-    dig_chunk<EST>(dig, kPlane, a0, dig + kOperand, kPlane, b0, iacc, est);
+    dig_chunk(dig, kPlane, a0, dig + kOperand, kPlane, b0, iacc, est);
     ++held;
   }
   // outputs whose terms are all too far below the scales of their row and column
   unsigned low = 0;
-  if (EST && !special) {
+  if (!special) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int r = m0 + gr + 8 * ((j >> 1) & 1), cl = n0 + gc + 8 * (j >> 2) + (j & 1);
       const float t = est[j >> 2][j & 3];
-      if (r < m && cl < n && !(lower && r < cl) && t > 0.f && t < kCovered) low |= 1u << j;
+      if (r < m && cl < n && !(lower && r < cl) && t > 0.f && t < (OP == 0 ? kCovered : kCoveredInv)) low |= 1u << j;
     }
     special = __popc(__ballot_sync(0xffffffffu, low != 0)) > kManyLow;       // this warp's part
   }
@@ -241,7 +237,7 @@ gemm_f64_digits_kernel(double* __restrict__ C, int ldc, const double* __restrict
     }
     return;
   }
-  if (EST && __any_sync(0xffffffffu, low != 0)) {
+  if (__any_sync(0xffffffffu, low != 0)) {
     // a few: FP64 FMAs by the whole warp, the terms over its lanes
 #pragma unroll 1
     for (int j = 0; j < 8; ++j)
