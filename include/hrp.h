@@ -136,8 +136,10 @@ hrp_status hrp_potrf_async(hrp_handle* h, const hrp_tree* tree, int n, double* d
  * forward substitution L Y = B, then backward L^T X = Y, with FP64 storage and sums.  Two
  * ways, both off GB300's slow FP64 pipe:
  *   - n <= 512, more than 8 right-hand sides, or n > 1024 (one right-hand side: up to 3072):
- *     with FP64 inverses of the diagonal blocks of up to 512 rows, products exact to 2^-55 of
- *     the largest term (with several right-hand sides, of the row's times the column's largest);
+ *     with FP64 inverses of the diagonal blocks of up to 512 rows; every product is accurate
+ *     against the sum of its own terms' magnitudes, whatever the units of rows, columns and
+ *     right-hand sides (about 2^-53 of it, 2^-46 where the terms lie far below their row's and
+ *     column's largest, 2^-38 if in addition all digits of all entries were at their extremes);
  *   - otherwise, and where the device's memory does not hold those inverses (6.3 KB per row):
  *     in 64-row blocks whose 16-term partial products are formed in double-float (a pair of
  *     binary32 values, about 2^-44 relative to the sum of |terms| at worst).

@@ -13,11 +13,21 @@
 // Both products take 16 rows at a time and up to 512 inner terms, a warp 16 (few rows,
 // solve_step_kernel) or 64 of them (many, solve_wide_kernel).  The entries go from memory to registers
 // in the order the mma fragments want them, are cut into 8-bit digits there and multiplied exactly by
-// 28 mma per 16 terms (digits.cuh).  Scales: term k by its largest right-hand side, then a row of P and
-// a column of Y by the largest entry among the terms (of the warp, whose sums are then added in FP64 in
-// a fixed order; in the wide kernel of all, whose sums stay integers until the end), so 7 digits keep
-// 55 bits below the largest term of a sum (with several right-hand sides, below the row's times the
-// column's), whatever powers of two scale the unknowns.
+// 36 (few rows) or 28 mma per 16 terms (digits.cuh).  Scales: term k by its largest right-hand side, then a
+// row of P and a column of Y by the largest entry among the terms (of the warp, whose sums are then
+// added in FP64 in a fixed order; in the wide kernel of all, whose sums stay integers until the end),
+// so that powers of two that scale the unknowns change nothing.
+//
+// Several right-hand sides share the terms' scales, and where one is large in a term that the others
+// hardly see, the others' digits are too few.  One more mma per 16 terms, of the digits' magnitudes, therefore
+// estimates every output's sum |a| |y| against its scales, and outputs below a line are computed by
+// FP64 FMAs (a term per lane; by all lanes for the warp's outputs where there are many).  Per term the
+// scales' product is held to 2^-61.5 with eight digits and 2^-54.3 with seven, ordinary digits taken
+// (2^-58.9 and 2^-51.4 at worst), so that the lines at 2^-13 of a warp's 16 terms and 2^-4 of a wide
+// tile's 512 both leave 2^-46 of sum |a| |y| (2^-42 and 2^-38 at worst); the sweeps' double-float products
+// keep 2^-44 at worst.  Ordinary columns stay above the lines but for one output in 1000 of the diagonal
+// blocks (seven digits there: one in 40, hence the eight); n = 4096, 16 right-hand sides: 562 -> 601 us
+// with the estimate (1926 by the sweeps).
 // What bounds it: latency, 5 us a step with few rows and 8 to 11 us with many (at n = 4096 and one
 // right-hand side 170 us of inverses, most of it the last doubling, then 30 steps); from n = 8192 on the
 // wide kernel's tiles, 3 to 5 us each of load latency and integer work at two warps per scheduler (with
@@ -42,7 +52,13 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kRows = 16;
+constexpr int kSd = kByteDig, kWd = kDig;        // digits per operand (few rows, many), weights s + t below kept
+// smallest sum |a| |y| against the scales that the digits cover, of a warp's 16 terms and of a wide tile's, in
+// units of the first digits' product
+constexpr float kCoveredStep = 0x1p-13f * 4096.f, kCoveredWide = 0x1p-4f * 4096.f;
+constexpr int kManyLow = 4;                      // lanes with outputs to recompute above which a warp recomputes all
 constexpr int kNone = -4096;                     // below every exponent of a right-hand side against its term's
+constexpr int kNoRow = -(1 << 20);               // the scale of a row of zeros
 
 // The inverse of a 64 x 64 diagonal block of L (block blockIdx.y), 8 of its columns per CTA: columns
 // blockIdx.x + 8 u, two to a warp, so that every CTA has as much to do.  16 lanes hold a column, rows
@@ -157,8 +173,8 @@ __device__ __forceinline__ void rhs_scales(const double (&y)[NH][KS][4], unsigne
     for (int s = 0; s < KS; ++s)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int f = dig_field(y[h][s][j]);
-        if (f != 0) ey[h] = max(ey[h], f - term<KS>(ek, s, j));
+        const double v = y[h][s][j];             // (words: a 64-bit test becomes a comparison on the FP64 pipe)
+        if (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) ey[h] = max(ey[h], max(dig_field(v), 1) - term<KS>(ek, s, j));
       }
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) ey[h] = max(ey[h], __shfl_xor_sync(0xffffffffu, ey[h], o));
@@ -169,33 +185,44 @@ __device__ __forceinline__ void row_scales(const double (&a)[2][KS][4], const un
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     ea[h] = INT_MIN;
+    unsigned any = 0;
 #pragma unroll
     for (int s = 0; s < KS; ++s)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int f = dig_field(a[h][s][j]);
         special |= f == 0x7ff;
+        any |= (unsigned)__double2hiint(a[h][s][j]) | (unsigned)__double2loint(a[h][s][j]);
         ea[h] = max(ea[h], max(f, 1) + term<KS>(ek, s, j));
       }
+    if (any == 0) ea[h] = kNoRow;
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) ea[h] = max(ea[h], __shfl_xor_sync(0xffffffffu, ea[h], o));
   }
 }
-// the digits of a k step of the right-hand sides, and its products
-template <int NH, int KS>
+// the digits of a k step of the right-hand sides
+template <int ND, int NH, int KS>
 __device__ __forceinline__ void rhs_digits(const double (&y)[NH][KS][4], const unsigned (&ek)[KS][2], const int (&ey)[NH], int s,
-                                           uint32_t (&bf)[kDig][NH][2]) {
+                                           uint32_t (&bf)[ND][NH][2]) {
 #pragma unroll
   for (int h = 0; h < NH; ++h) {
     unsigned long long m[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) m[j] = (unsigned long long)dig_fix(y[h][s][j], ey[h] + term<KS>(ek, s, j)) + kByteBias;
 #pragma unroll
-    for (int d = 0; d < kDig; ++d) {
+    for (int d = 0; d < ND; ++d) {
       bf[d][h][0] = byte_pair(m[0], m[1], d);
       bf[d][h][1] = byte_pair(m[2], m[3], d);
     }
   }
+}
+// |first digit| + 2^-8 |second| of a pair: the magnitudes behind the estimate of sum |a| |y|
+__device__ __forceinline__ uint32_t pair_abs(uint32_t d0, uint32_t d1) {
+  d0 &= 0x7fff7fffu;
+  d1 &= 0x7fff7fffu;
+  const __half2 v = __hfma2(*reinterpret_cast<const __half2*>(&d1), __half2half2(__ushort_as_half(0x1c00)),      // 2^-8
+                            *reinterpret_cast<const __half2*>(&d0));
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 __device__ __forceinline__ void row_fragment(const unsigned long long (&m0)[4], const unsigned long long (&m1)[4], int d,
                                              uint32_t (&af)[4]) {
@@ -204,12 +231,44 @@ __device__ __forceinline__ void row_fragment(const unsigned long long (&m0)[4], 
   af[2] = byte_pair(m0[2], m0[3], d);
   af[3] = byte_pair(m1[2], m1[3], d);
 }
-// the warp's sums to part[row][right-hand side]: weights 2^(-12 - 8 w) joined in units of 2^-57 (at most 64
-// terms below 1)
+// the products of a k step: rows(d) gives digit d of the rows, bf[d] the right-hand sides'; est: the estimate, from
+// the first digits or (FINE) the first two
+template <int ND, bool FINE, int NH, class Rows>
+__device__ __forceinline__ void step_products(float (&acc)[ND][NH][4], float (&est)[NH][4], const Rows& rows,
+                                              const uint32_t (&bf)[ND][NH][2]) {
+  uint32_t first[4];
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    uint32_t af[4];
+    rows(d, af);
+#pragma unroll
+    for (int e = 0; e < ND - d; ++e)
+#pragma unroll
+      for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h][0], bf[e][h][1]);
+    if (d == 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) first[q] = FINE ? af[q] : af[q] & 0x7fff7fffu;
+    }
+    if (FINE && d == 1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) first[q] = pair_abs(first[q], af[q]);
+    }
+    if (d == (FINE ? 1 : 0)) {
+#pragma unroll
+      for (int h = 0; h < NH; ++h)
+        dig_mma(est[h], first, FINE ? pair_abs(bf[0][h][0], bf[1][h][0]) : bf[0][h][0] & 0x7fff7fffu,
+                FINE ? pair_abs(bf[0][h][1], bf[1][h][1]) : bf[0][h][1] & 0x7fff7fffu);
+    }
+  }
+}
+// the warp's sums to part[row][right-hand side]: weights 2^(-12 - 8 w) joined in units of 2^-28 (w < 3) and
+// 2^-68, and these in units of 2^-58 (16 terms below 1).  Returns the outputs that the digits do not
+// cover: bit 4 h + register.
 template <int NH>
-__device__ __forceinline__ void store_sums(const float (&acc)[kDig][NH][4], const int (&ea)[2], const int (&ey)[NH],
-                                           double (*part)[8 * NH]) {
+__device__ __forceinline__ unsigned store_sums(const float (&acc)[kSd][NH][4], const float (&est)[NH][4], const int (&ea)[2],
+                                               const int (&ey)[NH], bool estimate, double (*part)[8 * NH]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
+  unsigned low = 0;
 #pragma unroll
   for (int h = 0; h < NH; ++h)
 #pragma unroll
@@ -218,11 +277,12 @@ __device__ __forceinline__ void store_sums(const float (&acc)[kDig][NH][4], cons
 #pragma unroll
       for (int w = 0; w < 3; ++w) hi = (hi << 8) + __float2int_rn(acc[w][h][q]);
 #pragma unroll
-      for (int w = 3; w < kDig; ++w) lo = (lo << 8) + __float2int_rn(acc[w][h][q]);
-      const int c = t2 + (q & 1);
-      const int e = ea[q >> 1] + __shfl_sync(0xffffffffu, ey[h], 4 * c) - 2 * 1022;
-      part[g + 8 * (q >> 1)][8 * h + c] = dig_to_double((hi << 29) + (lo >> 3), e - 57);
+      for (int w = 3; w < kSd; ++w) lo = (lo << 8) + __float2int_rn(acc[w][h][q]);
+      const int c = t2 + (q & 1), ec = __shfl_sync(0xffffffffu, ey[h], 4 * c);
+      part[g + 8 * (q >> 1)][8 * h + c] = dig_to_double((hi << 30) + ((lo + 512) >> 10), ea[q >> 1] + ec - 2 * 1022 - 58);
+      if (estimate && est[h][q] < kCoveredStep && ea[q >> 1] != kNoRow && ec != kNone) low |= 1u << (4 * h + q);
     }
+  return low;
 }
 // the same sums by FP64 FMAs over the terms kb .. ke - 1 (row i: from lo(i), below hi(i))
 template <int NH, bool TRANS, class Lo, class Hi>
@@ -271,24 +331,39 @@ solve_step_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
       plain_sums<NH, TRANS>(P, ldp, r0, rows, Y, ldy, nrhs, [&](int i) { return TRI == 2 ? max(k0, i) : k0; },
                             [&](int i) { return min(min(K, k0 + 16), TRI == 1 ? i + 1 : K); }, part[warp]);
     } else {
-      float acc[kDig][NH][4] = {};
-      uint32_t bf[kDig][NH][2];
-      rhs_digits<NH, 1>(y, ek, ey, 0, bf);
+      float acc[kSd][NH][4] = {}, est[NH][4] = {};
+      uint32_t bf[kSd][NH][2];
+      rhs_digits<kSd, NH, 1>(y, ek, ey, 0, bf);
       unsigned long long m[2][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int h = 0; h < 2; ++h) m[h][j] = (unsigned long long)dig_fix(a[h][0][j], ea[h] - term<1>(ek, 0, j)) + kByteBias;
+      const bool estimate = nrhs > 1;                            // alone, a column sets its own terms' scales
+      step_products<kSd, true, NH>(acc, est, [&](int d, uint32_t (&af)[4]) { row_fragment(m[0], m[1], d, af); }, bf);
+      const unsigned low = store_sums<NH>(acc, est, ea, ey, estimate, part[warp]);
+      const unsigned lanes = __ballot_sync(0xffffffffu, low != 0);
+      if (lanes) {
+        auto lo = [&](int i) { return TRI == 2 ? max(k0, i) : k0; };
+        auto hi = [&](int i) { return min(min(K, k0 + 16), TRI == 1 ? i + 1 : K); };
+        __syncwarp();
+        if (__popc(lanes) > kManyLow) {
+          plain_sums<NH, TRANS>(P, ldp, r0, rows, Y, ldy, nrhs, lo, hi, part[warp]);
+        } else {
+          // a term per lane
+#pragma unroll 1
+          for (int q = 0; q < 4 * NH; ++q)
+            for (unsigned who = __ballot_sync(0xffffffffu, (low >> q) & 1); who; who &= who - 1) {
+              const int src = __ffs(who) - 1, i = (src >> 2) + 8 * ((q >> 1) & 1), c = 8 * (q >> 2) + 2 * (src & 3) + (q & 1);
+              const int k = lo(r0 + i) + (lane & 15);
+              double v = 0.0;
+              if (k < hi(r0 + i)) v = (TRANS ? P[(size_t)(r0 + i) * ldp + k] : P[(size_t)k * ldp + r0 + i]) * Y[(size_t)c * ldy + k];
 #pragma unroll
-      for (int d = 0; d < kDig; ++d) {
-        uint32_t af[4];
-        row_fragment(m[0], m[1], d, af);
-#pragma unroll
-        for (int e = 0; e < kDig - d; ++e)
-#pragma unroll
-          for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h][0], bf[e][h][1]);
+              for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+              if (lane == 0) part[warp][i][c] = v;
+            }
+        }
       }
-      store_sums<NH>(acc, ea, ey, part[warp]);
     }
   } else {
     for (int e = lane; e < kRows * 8 * NH; e += 32) part[warp][e / (8 * NH)][e % (8 * NH)] = 0.0;
@@ -316,7 +391,7 @@ static_assert(kRows * 16 == kThreads, "one output per thread at 16 right-hand si
 constexpr int kWide = 4;                         // k steps per warp
 template <int NH>
 constexpr int wide_smem() {
-  return 8 * kWide * kDig * NH * 32 * 8 + 2 * 8 * kRows * 8 * NH * 8;
+  return 8 * kWide * kWd * NH * 32 * 8 + 2 * 8 * kRows * 8 * NH * (8 + 4);
 }
 template <int NH, bool TRANS>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -330,14 +405,17 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
   __shared__ int s_ea[3][kRows], s_special[3];
   __shared__ int s_ey[8 * NH], s_yspecial;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2;
-  uint2 (*bfs)[kDig][NH][32] = reinterpret_cast<uint2 (*)[kDig][NH][32]>(smem) + warp * kWide;     // [s][digit][half][lane]
+  uint2 (*bfs)[kWd][NH][32] = reinterpret_cast<uint2 (*)[kWd][NH][32]>(smem) + warp * kWide;       // [s][digit][half][lane]
+  // [parity]: the warps' sums, and their estimates of sum |a| |y|
   long long (*parts)[8][kRows][8 * NH] =
-      reinterpret_cast<long long (*)[8][kRows][8 * NH]>(smem + 8 * kWide * kDig * NH * 32 * 8);     // [parity]
+      reinterpret_cast<long long (*)[8][kRows][8 * NH]>(smem + 8 * kWide * kWd * NH * 32 * 8);
+  float (*ests)[8][kRows][8 * NH] = reinterpret_cast<float (*)[8][kRows][8 * NH]>(parts + 2);
+  const bool estimate = nrhs > 1;
   const int k0 = 16 * kWide * warp;
   const bool act = k0 < K;
   const int step = (int)gridDim.x * kRows;
   int r0 = (int)blockIdx.x * kRows;
-  if (tid < 3 * kRows) (&s_ea[0][0])[tid] = INT_MIN;
+  if (tid < 3 * kRows) (&s_ea[0][0])[tid] = kNoRow;
   if (tid < 3) s_special[tid] = 0;
   if (tid < 8 * NH) s_ey[tid] = kNone;
   if (tid == 0) s_yspecial = 0;
@@ -374,10 +452,10 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
     for (int h = 0; h < NH; ++h) ey[h] = s_ey[8 * h + g];
 #pragma unroll
     for (int s = 0; s < kWide; ++s) {
-      uint32_t bf[kDig][NH][2];
-      rhs_digits<NH, kWide>(y, ek, ey, s, bf);
+      uint32_t bf[kWd][NH][2];
+      rhs_digits<kWd, NH, kWide>(y, ek, ey, s, bf);
 #pragma unroll
-      for (int d = 0; d < kDig; ++d)
+      for (int d = 0; d < kWd; ++d)
 #pragma unroll
         for (int h = 0; h < NH; ++h) bfs[s][d][h][lane] = make_uint2(bf[d][h][0], bf[d][h][1]);
     }
@@ -391,7 +469,7 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
     const int next = buf == 2 ? 0 : buf + 1, after = 3 - buf - next;
     const bool plain = s_yspecial || s_special[buf];             // the same in every warp
     const bool more = r0 + step < rows;
-    if (tid < kRows) s_ea[after][tid] = INT_MIN;
+    if (tid < kRows) s_ea[after][tid] = kNoRow;
     if (tid == 0) s_special[after] = 0;
     if (plain) {
       double (*part)[8 * NH] = reinterpret_cast<double (*)[8 * NH]>(parts[par][warp]);
@@ -412,23 +490,19 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
           for (int h = 0; h < 2; ++h)
             m[s][h][j] = (unsigned long long)dig_fix(a[h][s][j], ea[h] - term<kWide>(ek, s, j)) + kByteBias;
       if (more) load_rows<TRANS, kWide>(a, P, ldp, r0 + step, rows, k0, K);
-      float acc[kDig][NH][4] = {};
+      float acc[kWd][NH][4] = {}, est[NH][4] = {};
 #pragma unroll
       for (int s = 0; s < kWide; ++s) {
-        uint2 bf[kDig][NH];
+        uint32_t bf[kWd][NH][2];
 #pragma unroll
-        for (int d = 0; d < kDig; ++d)
+        for (int d = 0; d < kWd; ++d)
 #pragma unroll
-          for (int h = 0; h < NH; ++h) bf[d][h] = bfs[s][d][h][lane];
-#pragma unroll
-        for (int d = 0; d < kDig; ++d) {
-          uint32_t af[4];
-          row_fragment(m[s][0], m[s][1], d, af);
-#pragma unroll
-          for (int e = 0; e < kDig - d; ++e)
-#pragma unroll
-            for (int h = 0; h < NH; ++h) dig_mma(acc[d + e][h], af, bf[e][h].x, bf[e][h].y);
-        }
+          for (int h = 0; h < NH; ++h) {
+            const uint2 v = bfs[s][d][h][lane];
+            bf[d][h][0] = v.x;
+            bf[d][h][1] = v.y;
+          }
+        step_products<kWd, false, NH>(acc, est, [&](int d, uint32_t (&af)[4]) { row_fragment(m[s][0], m[s][1], d, af); }, bf);
       }
       // weights 2^(-12 - 8 w) joined in units of 2^-54 (512 terms below 1)
 #pragma unroll
@@ -442,17 +516,23 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
 #pragma unroll
             for (int w = 0; w < 3; ++w) hi = (hi << 8) + __float2int_rn(acc[w][h][q + u]);
 #pragma unroll
-            for (int w = 3; w < kDig; ++w) lo = (lo << 8) + __float2int_rn(acc[w][h][q + u]);
+            for (int w = 3; w < kWd; ++w) lo = (lo << 8) + __float2int_rn(acc[w][h][q + u]);
             v[u] = (hi << 26) + (lo >> 6);
           }
-          *reinterpret_cast<longlong2*>(&parts[par][warp][g + 4 * q][8 * h + 2 * (lane & 3)]) = make_longlong2(v[0], v[1]);
+          const int i = g + 4 * q, c = 8 * h + 2 * (lane & 3);
+          *reinterpret_cast<longlong2*>(&parts[par][warp][i][c]) = make_longlong2(v[0], v[1]);
+          *reinterpret_cast<float2*>(&ests[par][warp][i][c]) = make_float2(est[h][q], est[h][q + 1]);
         }
       if (more) scale_rows(next);
     } else {
-      for (int e = lane; e < kRows * 8 * NH; e += 32) parts[par][warp][e / (8 * NH)][e % (8 * NH)] = 0;
+      for (int e = lane; e < kRows * 8 * NH; e += 32) {
+        parts[par][warp][e / (8 * NH)][e % (8 * NH)] = 0;
+        ests[par][warp][e / (8 * NH)][e % (8 * NH)] = 0.f;
+      }
     }
     // one barrier per tile: the sums of the next go to the other half
     const int er = s_ea[buf][i];
+    bool low = false;
     __syncthreads();
     if (out) {
       if (plain) {
@@ -461,8 +541,21 @@ solve_wide_kernel(const double* __restrict__ P, int ldp, int rows, int K, const 
         long long v = 0;
 #pragma unroll
         for (int w = 0; w < 8; ++w) v += parts[par][w][i][c];
-        *o = o0 - dig_to_double(v, er + s_ey[c] - 2 * 1022 - 54);
+        float est = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) est += ests[par][w][i][c];
+        low = estimate && est < kCoveredWide && er != kNoRow && s_ey[c] != kNone;
+        if (!low) *o = o0 - dig_to_double(v, er + s_ey[c] - 2 * 1022 - 54);
       }
+    }
+    // outputs the digits do not cover: FP64 FMAs, the terms over the warp's lanes
+    for (unsigned who = __ballot_sync(0xffffffffu, low); who; who &= who - 1) {
+      const int src = __ffs(who) - 1, si = r0 + src % kRows, sc = (tid - lane + src) / kRows;
+      double f = 0.0;
+      for (int k = lane; k < K; k += 32) f = fma(TRANS ? P[(size_t)si * ldp + k] : P[(size_t)k * ldp + si], Y[(size_t)sc * ldy + k], f);
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) f += __shfl_xor_sync(0xffffffffu, f, d);
+      if (lane == src) *o = o0 - f;
     }
     buf = next;
   }
