@@ -109,7 +109,7 @@ cudaError_t launch_trsm_leaf32_subst(double* A, int ld, int r0, int m, int c0, i
                                      unsigned* err, cudaStream_t s, const double* Lm = nullptr, int ldl = 0);
 
 // FP64 leaf TRSM by refinement on the tensor pipe (k_trsm64.cu), nc <= 128, with the FP32 inverse
-// W of the leaf (ldw): the accuracy of FP64 substitution or better; outputs as launch_trsm_leaf64.
+// W of the leaf (ldw): every entry within the bound of FP64 substitution; outputs as launch_trsm_leaf64.
 cudaError_t launch_trsm_refine64(double* A, int ld, int r0, int m, int c0, int nc, const float* W, int ldw,
                                  __half* shadow16, int lds, float* shadow32, int ld32, const int* info, unsigned* err,
                                  cudaStream_t s, const double* Lm = nullptr, int ldl = 0);

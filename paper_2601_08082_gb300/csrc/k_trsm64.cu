@@ -13,16 +13,26 @@
 // bounds it is latency of the staged phases at few rows, and the mma and splitting work (28
 // products per entry and pass) at many.  Against the right-looking FP64 substitution
 // (trsm_rl64_kernel, FP64 pipe and a 63-step chain), 128 columns: 1000 rows 66 -> ~28 us, 3000
-// rows 188 -> ~45 us; a standalone TRSM of 3000 x 2048 (three levels, 16 leaves of 128) 3.51 ->
-// 1.13 ms, the n = 1024 FP64 factor and solve with leaf 64 1.96 -> 1.84 ms.  Its error against
+// rows 188 -> ~49 us; a standalone TRSM of 3000 x 2048 (three levels, 16 leaves of 128) 3.51 ->
+// 1.20 ms, the n = 1024 FP64 factor and solve with leaf 64 1.96 -> 1.84 ms.  Its error against
 // extended precision is 2 to 10 times smaller than the substitution's.
 //
 // Scales are powers of two, applied exactly: 2^beta_r from the largest entry of row r of B, c_j
 // from the largest entry of column j of the first X over the CTA's rows, rho_r of row r of that X
 // after the columns' scales, and El_j of row j of L with the columns' scales.  X is held to
-// 2^-62 of its row's and column's scale, so its error does not grow with the rows' or columns'
-// ranges.  Rows whose first X is not finite, whose B does not fit the scales, or that do not
-// converge (an ill-conditioned or singular leaf) are solved by FP64 substitution in the same CTA.
+// 2^-62 of its row's and column's scale.  Rows whose first X is not finite, whose B does not fit the
+// scales, or that do not converge (an ill-conditioned or singular leaf) are solved by FP64
+// substitution in the same CTA.
+//
+// A column's scale comes from all rows of the CTA, and an entry whose own terms are far below its row's and
+// column's scales (rows or columns in different units) would be left with their error.  So sum |x| |l|
+// is estimated for every entry beside the first residual (one mma per 16 terms on bfloat16 magnitudes),
+// and the entries below 2^-12 of the scales are computed again, x_j = (b_j - sum_{k<j} x_k l_jk) / l_jj in FP64,
+// once the others are done; a row with more than kMaxLow of them sends its CTA to the substitution.  The line:
+// a residual is good to 2^-59.8 of its scales (128 terms, ordinary digits; nc 2^-59.7 at worst), so 2^-47.8 of
+// sum |x| |l| at it, under the substitution's bound of nc 2^-53; of 2000 entries of an ordinary panel one is
+// below it (16 at 2^-10).  It costs 3 % of the n = 1024 FP64 factorization (1468 -> 1515 us) and 6 % of the
+// TRSM of 3000 x 2048 (1126 -> 1198).
 #include <climits>
 
 #include "digits.cuh"
@@ -35,6 +45,9 @@ namespace {
 // (up to 2^7 units); their difference is below 2^-2 or the rows go to the substitution.
 constexpr int kRFrac = 60;
 constexpr int kMaxPass = 8;
+// Entries below 2^-12 of their scales (kCovered) are computed again by FP64 FMAs, up to kMaxLow in a row
+constexpr float kCovered = 0x1p-12f;
+constexpr int kMaxLow = 6;
 // the scale of a column whose first X is zero in every row: it must weigh nothing in the rows of L
 constexpr int kNoScale = -4096;
 
@@ -47,9 +60,9 @@ __host__ __device__ inline T64Layout t64_layout(int nc, int rows) {
   l.lx = 0;                                   // L: lower 16 x 16 tiles of 64-bit values
   l.w = l.lx + T * (T + 1) / 2 * 256 * 8;     // W: groups of 8 rows j, [k][8] for k < 8 (g + 1)
   l.xd = l.w + 32 * (2 * T) * (2 * T + 1) * 4;
-  l.xd_ld = ncp + 8;                          // X's digits [7][rows][ncp + 8]
+  l.xd_ld = ncp + 8;                          // X's digits [7][rows][ncp + 8], and its magnitudes
   l.xd_plane = rows * l.xd_ld;
-  l.b = l.xd + kDig * l.xd_plane * 2;         // B: [k][rows] doubles
+  l.b = l.xd + (kDig + 1) * l.xd_plane * 2;         // B: [k][rows] doubles
   l.r = l.b + ncp * rows * 8;                 // R (and fl32(B)): [k][rows] floats
   l.total = l.r + ncp * rows * 4;
   return l;
@@ -85,6 +98,15 @@ __device__ __forceinline__ long long fix_float(float x, int E) {
   return (int)b < 0 ? -v : v;
 }
 
+// |v| of a fixed-point entry (unit 2^-62, plus kDigBias) as a bfloat16, truncated, at least 2^-60 unless zero
+__device__ __forceinline__ uint32_t fix_abs(unsigned long long v) {
+  const long long d = (long long)(v - kDigBias);
+  const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
+  const unsigned hi = (unsigned)(a >> 32);                    // units 2^-30
+  const int b = (int)(__float_as_uint((float)hi * 0x1p-30f) >> 16);
+  return a == 0 ? 0u : (uint32_t)max(b, kAbsMin);
+}
+
 // unit u of the packed W -> its group and column: 4 g (g + 1) units come before group g
 __device__ __forceinline__ void w_unit(int u, int& g, int& k) {
   g = (int)((sqrtf((float)(u + 1)) - 1.0f) * 0.5f);
@@ -116,7 +138,8 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_beta[ROWS], s_rho[ROWS], s_c[16 * TM], s_el[16 * TM];
-  __shared__ unsigned s_max;
+  __shared__ unsigned s_max, s_low[ROWS][TM / 2];            // entries to compute again, a bit per column
+  __shared__ int s_nlow[ROWS];
   if (*(volatile const int*)info != INT_MAX) return;
   const T64Layout lay = t64_layout(nc, ROWS);
   const int T = (nc + 15) / 16, ncp = 16 * T, G = 2 * T, nt = T * (T + 1) / 2;
@@ -183,6 +206,8 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
     }
   }
   if (tid < ROWS) s_beta[tid] = s_rho[tid] = INT_MIN;
+  if (tid < ROWS) s_nlow[tid] = 0;
+  if (tid < ROWS * (TM / 2)) s_low[tid / (TM / 2)][tid % (TM / 2)] = 0;
   if (tid < 16 * TM) s_c[tid] = INT_MIN;
   if (tid == 0) s_max = 0;
   __syncthreads();
@@ -341,9 +366,54 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
 #pragma unroll
         for (int q = 0; q < 4; ++q) X[h][q] = fix_float(x0[h][q], s_rho[rr + 16 * h] + s_c[8 * g + cq + q] + 1);
       put_digits();
+      // the magnitudes of the first X against the same scales, as bfloat16 (dig_abs)
+#pragma unroll
+      for (int h = 0; h < MR; ++h) {
+        uint32_t b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int e = s_rho[rr + 16 * h] + s_c[8 * g + cq + q] + 1, v = (int)(__float_as_uint(fabsf(x0[h][q])) >> 16);
+          b[q] = x0[h][q] == 0.f ? 0u : (uint32_t)max(v - e * 128, kAbsMin);
+        }
+        *reinterpret_cast<uint2*>(Xd + kDig * lay.xd_plane + (size_t)(rr + 16 * h) * lay.xd_ld + 8 * g + cq) =
+            make_uint2(b[0] | (b[1] << 16), b[2] | (b[3] << 16));
+      }
     }
   }
   __syncthreads();
+
+  // sum |x| |l| of every entry of X L^T against the scales (a fifth of a pass): where an entry's own terms are
+  // far below them, the residual's digits do not cover it
+  int many = 0;                               // too many of them in a row: joins `bad` with the first pass
+  if (!bad && act) {
+    const int I = g >> 1, jrow = 8 * (g & 1) + (lane >> 2);
+    float est[MR][4] = {};
+    const __half* xa = Xd + kDig * lay.xd_plane + (size_t)(lane & 15) * lay.xd_ld + (lane >> 4) * 8;
+#pragma unroll 2
+    for (int kt = 0; kt <= I; ++kt) {
+      const long long* lt = Lx + (I * (I + 1) / 2 + kt) * 256;
+      const ulonglong2 p0 = *reinterpret_cast<const ulonglong2*>(lt + lx_at(jrow, 2 * (lane & 3)));
+      const ulonglong2 p1 = *reinterpret_cast<const ulonglong2*>(lt + lx_at(jrow, 2 * (lane & 3) + 8));
+      const uint32_t b0 = fix_abs(p0.x) | (fix_abs(p0.y) << 16), b1 = fix_abs(p1.x) | (fix_abs(p1.y) << 16);
+#pragma unroll
+      for (int h = 0; h < MR; ++h) {
+        uint32_t a[4];
+        dig_ldmatrix(a, xa + (size_t)(16 * h) * lay.xd_ld + 16 * kt);
+        dig_mma_bf16(est[h], a, b0, b1);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < MR; ++h)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = 16 * h + (lane >> 2) + 8 * (q >> 1), j = 8 * g + 2 * (lane & 3) + (q & 1);
+        // (all terms and the right-hand side zero: so is the entry)
+        if (j < nc && r < live && est[h][q] < kCovered && (est[h][q] > 0.f || !is_zero(Bs[j * ROWS + r]))) {
+          atomicOr(&s_low[r][j >> 5], 1u << (j & 31));
+          if (atomicAdd(&s_nlow[r], 1) >= kMaxLow) many = 1;
+        }
+      }
+  }
 
   float first = 1.f, last = 1.f;
   bool done = false;
@@ -451,7 +521,7 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
       const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
       if (lane == 0) atomicMax(&s_max, mb);
     }
-    bad = __syncthreads_or(bad);
+    bad = __syncthreads_or(bad | many);
     const float delta = __uint_as_float(s_max);
     if (pass == 0) first = fmaxf(delta, 0x1p-24f);
     else if (delta > 0.25f * last && delta > 0x1p-50f) bad = 1;        // does not converge
@@ -479,6 +549,41 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
             over16 |= fabs(x) > (double)kF16Max;
             S[(size_t)(r0 + row0 + r) * lds + c0 + j] = __double2half(x);
           }
+        }
+    }
+    // the entries that the digits do not cover, from the others of their row: x_j = (b_j - sum_{k<j} x_k l_jk) / l_jj,
+    // a row per warp, the terms over its lanes
+    __syncthreads();
+    for (int r = warp; r < live; r += NT / 32) {
+      if (s_nlow[r] == 0) continue;
+      double* xr = A + (size_t)c0 * ld + r0 + row0 + r;
+      for (int w = 0; w < TM / 2; ++w)
+        for (unsigned m = s_low[r][w]; m; m &= m - 1) {
+          const int j = 32 * w + __ffs(m) - 1;
+          const double* lj = Lm + (size_t)c0 * ldl + c0 + j;
+          const double b = Bs[j * ROWS + r], d = lj[(size_t)j * ldl];
+          double xk[TM / 2], lk[TM / 2], t = 0.0;             // a row's terms, 32 apart, all in flight at once
+#pragma unroll
+          for (int u = 0; u < TM / 2; ++u) {
+            const int k = lane + 32 * u;
+            xk[u] = k < j ? __ldcg(xr + (size_t)k * ld) : 0.0;
+            lk[u] = k < j ? lj[(size_t)k * ldl] : 0.0;
+          }
+          const double rd = 1.0 / d;                          // off the chain
+#pragma unroll
+          for (int u = 0; u < TM / 2; ++u) t = fma(xk[u], lk[u], t);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+          if (lane == 0) {
+            const double x = (b - t) * rd;
+            xr[(size_t)j * ld] = x;
+            if (S32 != nullptr) S32[(size_t)(c0 + j) * ld32 + r0 + row0 + r] = (float)x;
+            if (S != nullptr) {
+              over16 |= fabs(x) > (double)kF16Max;
+              S[(size_t)(r0 + row0 + r) * lds + c0 + j] = __double2half(x);
+            }
+          }
+          __syncwarp();
         }
     }
   } else {
