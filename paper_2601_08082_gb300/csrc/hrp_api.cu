@@ -1920,6 +1920,7 @@ hrp_status hrp_potrf_batched(hrp_handle* h, const hrp_tree* const* trees_in, int
     f.tile_exp = nullptr;
     f.w32 = reinterpret_cast<float*>(h->bwork + ws[i].w32);
     f.scratch = f.w32 + (size_t)f.n * 128;
+    f.waited[f.s] = true;                  // by fork()
     f.begin(CLS_OTHER, 0.0);
     f.chk(launch_fill_int(f.info, INT_MAX, 1, f.s));
     return true;
@@ -1956,6 +1957,7 @@ hrp_status hrp_potrs_batched(hrp_handle* h, int batch, const int* n, double* con
   if ((st = fork(h, s)) != HRP_OK) return st;
   cudaError_t err = cudaSuccess;
   long long launches = 0;
+  launch_ctx() = LaunchCtx{};
   // longest first; the sweeps and the block inverses of all systems, then the solves with the inverses
   const std::vector<int> order = longest_first(batch, n);
   for (int part = 0; part < 2; ++part)
@@ -2370,6 +2372,7 @@ extern "C" hrp_status hrp_posv_batched(hrp_handle* h, const hrp_tree* const* tre
       f.shadow = tree_has(f.t, HRP_F16) ? reinterpret_cast<__half*>(h->bwork + ws[i].shadow) : nullptr;
       f.w32 = reinterpret_cast<float*>(h->bwork + ws[i].w32);
       f.scratch = f.w32 + (size_t)n[i] * 128;
+      f.waited[si] = true;                 // by fork()
       f.begin(CLS_OTHER, 0.0);
       f.chk(launch_copy_lower(fact_of(i), n[i], dA[i], lda[i], n[i], si));
       f.begin(CLS_OTHER, 0.0);
@@ -2410,7 +2413,9 @@ extern "C" hrp_status hrp_posv_batched(hrp_handle* h, const hrp_tree* const* tre
         cudaStream_t si = h->bstreams[which[i]];
         double* R = res_of(i);
         if (part == 0) {
+          launch_ctx().pdl = false;        // the stream has waited for another
           if (fresh[i]) note(launch_copy_matrix(dX[i], ldx[i], dB[i], ldb[i], n[i], nrhs, si));
+          launch_ctx().pdl = true;
           note(launch_potrs(fact_of(i), n[i], fresh[i] ? dX[i] : R, fresh[i] ? ldx[i] : n[i], n[i], nrhs, true,
                             h->bwork + ws[i].pinv, reinterpret_cast<int*>(h->bwork + ws[i].ticket), h->d_err, si,
                             h->wait_ns));

@@ -570,10 +570,11 @@ cudaError_t launch_step(const double* P, int ldp, int rows, int K, const double*
   cfg.blockDim = dim3(kThreads);
   cfg.stream = s;
   cudaLaunchAttribute at[2];
+  const int np = launch_ctx().pdl ? 1 : 0;
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = np;
   if constexpr (ADD) {
     // the wide kernel where the clusters would be more than two CTAs per SM (n = 3000 .. 8192 with 16
     // right-hand sides: 2 to 4 % above lines at one half, one and four CTAs)
@@ -593,11 +594,11 @@ cudaError_t launch_step(const double* P, int ldp, int rows, int K, const double*
     }
   }
   cfg.gridDim = dim3(tiles, ky);
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = 1;
-  at[1].val.clusterDim.y = ky;
-  at[1].val.clusterDim.z = 1;
-  cfg.numAttrs = 2;
+  at[np].id = cudaLaunchAttributeClusterDimension;
+  at[np].val.clusterDim.x = 1;
+  at[np].val.clusterDim.y = ky;
+  at[np].val.clusterDim.z = 1;
+  cfg.numAttrs = np + 1;
   return cudaLaunchKernelEx(&cfg, solve_step_kernel<NH, TRANS, ADD, TRI>, P, ldp, rows, K, Y, ldy, O, ldo, nrhs);
 }
 
@@ -630,7 +631,12 @@ cudaError_t launch_solve_inverses(const double* L, int ldl, int n, void* work, c
   const int blk = solve_block(n), ldt = solve_scratch(n);
   double* W = static_cast<double*>(work);
   double* T = W + (size_t)n * blk;
+  // the first kernel may follow a join with another stream (see LaunchCtx): launched plainly
+  LaunchCtx& lc = launch_ctx();
+  const bool pdl = lc.pdl;
+  lc.pdl = false;
   (void)launch_pdl(inverse64_kernel, dim3(8, (n + 63) / 64), dim3(128), 0, s, L, ldl, n, W, blk);
+  lc.pdl = pdl;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   for (int h = 64; h < blk; h *= 2) {
