@@ -126,7 +126,7 @@ hrp_status hrp_potrf(hrp_handle* h, const hrp_tree* tree, int n, double* dA, int
 /*
  * As hrp_potrf, but never synchronizes: d_info is a DEVICE int that receives 0 or the
  * failing column when the enqueued work completes. Capturable in a CUDA graph once the
- * workspace for n exists.
+ * workspace for n exists (an all-FP64 tree also before, its leaves then unrefined).
  */
 hrp_status hrp_potrf_async(hrp_handle* h, const hrp_tree* tree, int n, double* dA, int lda,
                            int* d_info, void* stream);
@@ -140,10 +140,12 @@ hrp_status hrp_potrf_async(hrp_handle* h, const hrp_tree* tree, int n, double* d
  *     against the sum of its own terms' magnitudes, whatever the units of rows, columns and
  *     right-hand sides (about 2^-53 of it, 2^-46 where the terms lie far below their row's and
  *     column's largest, 2^-38 if in addition all digits of all entries were at their extremes);
- *   - otherwise, and where the device's memory does not hold those inverses (6.3 KB per row):
+ *   - otherwise, where the device's memory does not hold those inverses (6.3 KB per row; remembered, not
+ *     tried again), and in a capture that comes before the first such call of its order:
  *     in 64-row blocks whose 16-term partial products are formed in double-float (a pair of
  *     binary32 values, about 2^-44 relative to the sum of |terms| at worst).
- * Its workspaces for order n are allocated by the first call of that order (capturable after).
+ * Its workspaces for order n are allocated by the first call of that order (capturable after);
+ * that of the inverses by the first call that uses them.
  * dB (n x nrhs, ldb >= max(1,n)) is overwritten with X. Asynchronous.
  */
 hrp_status hrp_potrs(hrp_handle* h, int n, int nrhs, const double* dL, int ldl,
@@ -432,7 +434,8 @@ hrp_status hrp_posv_batched(hrp_handle* h, const hrp_tree* const* trees, int bat
  *   triangle of the n x n dL (ldl), which is not modified.  Base case: min(m, n) <= trsm_leaf
  *   (0 = leaf), trsm_leaf <= 128 unless m <= 128.
  * Workspace: an FP16 copy of A (n x k) or of [B; L] ((m + n) x n), and an FP32 copy when the
- * tree has F32 levels, in the handle.
+ * tree has F32 levels, in the handle; for hrp_trsm with FP64 base cases also n x 128 floats, without
+ * which (no memory, or a first call in a capture) they go by FP64 substitution.
  */
 hrp_status hrp_syrk(hrp_handle* h, const hrp_tree* tree, int n, int k, const double* dA, int lda, double* dC, int ldc,
                     void* stream);
@@ -458,10 +461,14 @@ long long hrp_last_launch_count(const hrp_handle* h);
  *   the kernel records the timeout and returns, and the call reports HRP_ERR_TIMEOUT with
  *   *waited_us (host, may be NULL) the time the device waited.  The context stays usable.
  *   Synchronous.
+ * hrp_alloc_selftest: the handle goes on as if no workspace of `bytes` or more could be allocated of those
+ *   that its calls can do without: the block inverses of the solves, the leaf inverses of all-FP64
+ *   factorizations and of hrp_trsm (0: as the device allows, trying again what it refused before).
  */
 hrp_status hrp_check(hrp_handle* h, void* stream);
 hrp_status hrp_set_wait_limit(hrp_handle* h, long long microseconds);
 hrp_status hrp_wait_selftest(hrp_handle* h, long long microseconds, double* waited_us, void* stream);
+hrp_status hrp_alloc_selftest(hrp_handle* h, size_t bytes);
 
 /*
  * hrp_potrs_noalloc: the same solve as hrp_potrs (B <- A^{-1} B from the factor in the

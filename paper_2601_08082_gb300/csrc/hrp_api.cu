@@ -61,6 +61,8 @@ struct hrp_handle_s {
   size_t pwork_cap = 0;
   unsigned char* swork = nullptr;  // block inverses of the solves (k_solve.cu)
   size_t swork_cap = 0;
+  size_t swork_refused = SIZE_MAX; // smallest size of it that the device did not hold
+  size_t alloc_limit = SIZE_MAX;   // of ensure_optional (hrp_alloc_selftest)
   unsigned char* rwork = nullptr;  // scales and digits of the residual's operands
   size_t rwork_cap = 0;
   double* d_norms = nullptr;   // 2 * 64 doubles
@@ -165,6 +167,32 @@ hrp_status ensure(hrp_handle* h, T** p, size_t* cap, size_t need) {
   }
   *cap = need;
   return HRP_OK;
+}
+
+// A workspace that its call can do without: false, and no error, where the device's memory does not hold it
+// (remembered in *refused, if given), or while the stream captures and it is not there yet.  The old buffer
+// is kept until the new one is there.
+template <typename T>
+bool ensure_optional(hrp_handle* h, T** p, size_t* cap, size_t need, cudaStream_t s, size_t* refused = nullptr) {
+  if (*cap >= need && *p) return true;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if ((refused && need >= *refused) || cudaStreamIsCapturing(s, &capturing) != cudaSuccess ||
+      capturing != cudaStreamCaptureStatusNone)
+    return false;
+  T* q = nullptr;
+  if (need * sizeof(T) >= h->alloc_limit || cudaMalloc(reinterpret_cast<void**>(&q), need * sizeof(T)) != cudaSuccess) {
+    cudaGetLastError();
+    if (refused) *refused = need;
+    return false;
+  }
+  cudaFree(*p);
+  *p = q;
+  *cap = need;
+  return true;
+}
+// h->swork for the block inverses of order n; without it the sweeps solve
+bool solve_workspace(hrp_handle* h, int n, cudaStream_t s) {
+  return ensure_optional(h, &h->swork, &h->swork_cap, solve_workspace_bytes(n), s, &h->swork_refused);
 }
 
 int split(int n) {
@@ -711,8 +739,11 @@ hrp_status potrf_enqueue(hrp_handle* h, const hrp_tree* t, int n, double* dA, in
     f.shadow8 = h->shadow8;
     f.tile_exp = h->tile_exp;
   }
-  if (n > 0) {
-    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128 + kLeafScratch)) != HRP_OK) return st;
+  const size_t w32_need = (size_t)n * 128 + kLeafScratch;
+  const bool lower = tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || has8;
+  if (n > 0 && lower && (st = ensure(h, &h->w32, &h->w32_cap, w32_need)) != HRP_OK) return st;
+  // an all-FP64 tree can do without: its leaves then run their direct schedules
+  if (n > 0 && (lower || ensure_optional(h, &h->w32, &h->w32_cap, w32_need, s))) {
     f.w32 = h->w32;
     f.scratch = h->w32 + (size_t)n * 128;
   }
@@ -1059,21 +1090,15 @@ hrp_status hrp_potrf(hrp_handle* h, const hrp_tree* tree, int n, double* dA, int
 }
 
 
-// h->swork for the block inverses of order n; false (the sweeps do without) where the device's memory
-// does not hold it
-static bool solve_workspace(hrp_handle* h, int n) {
-  return ensure(h, &h->swork, &h->swork_cap, solve_workspace_bytes(n)) == HRP_OK;
-}
-
 // A solve with the factor in dL.  prepared: h->swork already holds this factor's block inverses
 // (hrp_posv forms them once per factorization).
 static hrp_status potrs_impl(hrp_handle* h, int n, int nrhs, const double* dL, int ldl, double* dB, int ldb,
                              bool fp32, cudaStream_t s, bool prepared = false) {
   hrp_status st;
   if (n <= 0 || nrhs <= 0) return HRP_OK;
-  // both workspaces whatever the path: after one call of order n, none of that order allocates
+  // the sweeps' workspace whatever the path: after one call of order n, none of that order needs to allocate
   if ((st = ensure(h, &h->pwork, &h->pwork_cap, potrs_workspace_bytes(n))) != HRP_OK) return st;
-  if (prepared || (solve_workspace(h, n) && solve_blocked(n, nrhs))) {
+  if (prepared || (solve_blocked(n, nrhs) && solve_workspace(h, n, s))) {
     cudaError_t e = cudaSuccess;
     launch_ctx() = LaunchCtx{};
     if (!prepared) e = launch_solve_inverses(dL, ldl, n, h->swork, s);
@@ -1249,7 +1274,7 @@ hrp_status hrp_posv(hrp_handle* h, const hrp_tree* tree, int n, int nrhs, const 
     // 16 right-hand sides, one correction, no slower than FP32 sweeps anywhere (one right-hand side:
     // n = 200 330 -> 308 us a call, 1024 892 -> 851, 4096 4611 -> 4404; 16: 407 -> 328, 1011 -> 928,
     // 4921 -> 4757)
-    const bool prepared = solve_workspace(h, n);
+    const bool prepared = solve_workspace(h, n, s);
     if (prepared) {
       if ((e = launch_solve_inverses(h->fact, n, n, h->swork, s)) != cudaSuccess) return cuda_status(h, e, "hrp_posv");
       h->launches += solve_launches(n, 0, true);
@@ -1567,6 +1592,13 @@ hrp_status hrp_set_wait_limit(hrp_handle* h, long long microseconds) {
   return HRP_OK;
 }
 
+hrp_status hrp_alloc_selftest(hrp_handle* h, size_t bytes) {
+  if (!h) return HRP_ERR_INVALID_ARG;
+  h->alloc_limit = bytes ? bytes : SIZE_MAX;
+  h->swork_refused = SIZE_MAX;
+  return HRP_OK;
+}
+
 hrp_status hrp_wait_selftest(hrp_handle* h, long long microseconds, double* waited_us, void* stream) {
   if (!h) return HRP_ERR_INVALID_ARG;
   h->last_arg = 0;
@@ -1618,7 +1650,9 @@ hrp_status batch_prepare(hrp_handle* h, int batch, const int* n, std::vector<Sys
     w.shadow = need_factor_ws ? take((size_t)ni * w.lds * sizeof(__half)) : 0;
     w.w32 = need_factor_ws ? take(((size_t)ni * 128 + kLeafScratch) * sizeof(float)) : 0;
     w.pinv = take(potrs_workspace_bytes(ni));
-    w.swork = ni <= kSolveSmall ? take(solve_workspace_bytes(ni)) : 0;
+    // (for hrp_potrf_batched too, so that hrp_potrs_batched after it allocates nothing; refined solves
+    // use the sweeps)
+    w.swork = ni <= kSolveSmall && !nrhs_ir ? take(solve_workspace_bytes(ni)) : 0;
     w.ticket = take(sizeof(int));
     w.fact = nrhs_ir ? take(sizeof(double) * (size_t)ni * ni) : 0;
     w.res = nrhs_ir ? take(sizeof(double) * (size_t)ni * nrhs_ir + sizeof(double) * 2 * nrhs_ir) : 0;
@@ -2797,8 +2831,8 @@ hrp_status hrp_trsm(hrp_handle* h, const hrp_tree* tree, int m, int n, const dou
   }
   std::vector<std::pair<int, int>> lv;
   r.leaves(0, n, 0, lv);
-  if (!lv.empty()) {                             // all inverses at once, one CTA each
-    if ((st = ensure(h, &h->w32, &h->w32_cap, (size_t)n * 128)) != HRP_OK) return st;
+  // all inverses at once, one CTA each (without a workspace the leaves go by substitution)
+  if (!lv.empty() && ensure_optional(h, &h->w32, &h->w32_cap, (size_t)n * 128, r.s)) {
     r.w32 = h->w32;
     LeafList list;
     for (size_t i = 0; i < lv.size(); ++i) {

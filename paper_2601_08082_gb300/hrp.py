@@ -33,7 +33,7 @@ EXPORTED = [
     "hrp_policy_features", "hrp_mlp_forward", "hrp_mlp_grad", "hrp_mlp_adam", "hrp_mlp_param_count",
     "hrp_policy_set", "hrp_policy_predict", "hrp_policy_tree", "hrp_last_policy_choice",
     "hrp_autotune_candidates", "hrp_autotune", "hrp_policy_load", "hrp_check", "hrp_set_wait_limit",
-    "hrp_wait_selftest", "hrp_set_lookahead", "hrp_syrk", "hrp_trsm", "hrp_set_refinement",
+    "hrp_wait_selftest", "hrp_alloc_selftest", "hrp_set_lookahead", "hrp_syrk", "hrp_trsm", "hrp_set_refinement",
     "hrp_last_inner_iterations", "hrp_autotune_orders", "hrp_set_batched_mode", "hrp_set_scaling",
     "hrp_set_fp32_split", "hrp_set_f8_gemm", "hrp_set_leaf_chain", "hrp_get_timeline", "hrp_policy_set_min_order",
 ]
@@ -115,6 +115,7 @@ def load(path: str = LIB_PATH):
     L.hrp_check.argtypes = [vp, vp]
     L.hrp_set_wait_limit.argtypes = [vp, ctypes.c_longlong]
     L.hrp_wait_selftest.argtypes = [vp, ctypes.c_longlong, dp, vp]
+    L.hrp_alloc_selftest.argtypes = [vp, ctypes.c_size_t]
     L.hrp_policy_tree.argtypes = [c_int, tp]
     L.hrp_last_policy_choice.argtypes = [vp]
     L.hrp_autotune_candidates.argtypes = [tp, vp, c_int]
@@ -398,6 +399,10 @@ class Handle:
 
     def set_wait_limit(self, microseconds: int) -> None:
         self._check(self._lib.hrp_set_wait_limit(self._h, int(microseconds)))
+
+    def alloc_selftest(self, nbytes: int) -> None:
+        """hrp_alloc_selftest: solves as if no block-inverse workspace of nbytes or more could be had."""
+        self._check(self._lib.hrp_alloc_selftest(self._h, int(nbytes)))
 
     def wait_selftest(self, microseconds: int, stream=None) -> tuple[int, float]:
         """(status, microseconds the device waited) of a bounded wait on a flag nothing sets."""
