@@ -13,8 +13,8 @@
 // bounds it is latency of the staged phases at few rows, and the mma and splitting work (28
 // products per entry and pass) at many.  Against the right-looking FP64 substitution
 // (trsm_rl64_kernel, FP64 pipe and a 63-step chain), 128 columns: 1000 rows 66 -> ~28 us, 3000
-// rows 188 -> ~49 us; a standalone TRSM of 3000 x 2048 (three levels, 16 leaves of 128) 3.51 ->
-// 1.20 ms, the n = 1024 FP64 factor and solve with leaf 64 1.96 -> 1.84 ms.  Its error against
+// rows 188 -> ~50 us; a standalone TRSM of 3000 x 2048 (three levels, 16 leaves of 128) 3.51 ->
+// 1.22 ms, the n = 1024 FP64 factor and solve with leaf 64 1.96 -> 1.84 ms.  Its error against
 // extended precision is 2 to 10 times smaller than the substitution's.
 //
 // Scales are powers of two, applied exactly: 2^beta_r from the largest entry of row r of B, c_j
@@ -31,8 +31,8 @@
 // once the others are done; a row with more than kMaxLow of them sends its CTA to the substitution.  The line:
 // a residual is good to 2^-59.8 of its scales (128 terms, ordinary digits; nc 2^-59.7 at worst), so 2^-47.8 of
 // sum |x| |l| at it, under the substitution's bound of nc 2^-53; of 2000 entries of an ordinary panel one is
-// below it (16 at 2^-10).  It costs 3 % of the n = 1024 FP64 factorization (1468 -> 1515 us) and 6 % of the
-// TRSM of 3000 x 2048 (1126 -> 1198).
+// below it or fewer (up to 13 at 2^-10).  It costs 4 % of the n = 1024 FP64 factorization (1470 -> 1530 us) and 8 %
+// of the TRSM of 3000 x 2048 (1127 -> 1224).
 #include <climits>
 
 #include "digits.cuh"
@@ -124,6 +124,71 @@ __device__ __forceinline__ void cp_async_wait_all() {
 
 // float scale 2^e (saturating: values past binary32's range make the refinement give up)
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned)(max(-126, min(127, e)) + 127) << 23); }
+
+// The CTA's rows by FP64 substitution, 16 lanes per row: lane q holds columns q, q + 16, ..  L and its reciprocal
+// pivots are staged first (over L, W and X's digits, and over R); what bounds it is then the FP64 pipe, 4.5 FMAs
+// a column and pair of rows.  200 rows of 128 columns in units far apart take 120 us, refined ones 76 and
+// trsm_rl64_kernel 80; 3000 rows 178, 97 and 202.  (With L read from global memory, a division per
+// column in every lane and idle rows computed too: 437 and 363.)
+template <int TM, int ROWS, int NT>
+__device__ __noinline__ bool substitute(double* X, int ld, int r0, int m, int c0, int nc, const double* __restrict__ L, int ldl,
+                                        unsigned char* smem, __half* s16, int lds, float* s32, int ld32) {
+  const T64Layout lay = t64_layout(nc, ROWS);
+  double* Ls = reinterpret_cast<double*>(smem);
+  double* rinv = reinterpret_cast<double*>(smem + lay.r);
+  const double* Bs = reinterpret_cast<const double*>(smem + lay.b);
+  const int row0 = blockIdx.x * ROWS, live = min(ROWS, m - row0);
+  X += (size_t)c0 * ld + r0 + row0;
+  L += (size_t)c0 * ldl + c0;
+  if (s16 != nullptr) s16 += (size_t)(r0 + row0) * lds + c0;
+  if (s32 != nullptr) s32 += (size_t)c0 * ld32 + r0 + row0;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = tid & 15, ncp = (nc + 15) / 16 * 16;
+  bool over16 = false;
+  __syncthreads();
+#pragma unroll 4
+  for (int k = warp; k < nc; k += NT / 32)
+#pragma unroll
+    for (int u = 0; u < TM / 2; ++u) {
+      const int j = lane + 32 * u;
+      if (j < ncp) Ls[k * ncp + j] = (j >= k && j < nc) ? L[(size_t)k * ldl + j] : 0.0;
+    }
+  __syncthreads();
+  if (tid < nc) rinv[tid] = 1.0 / Ls[tid * ncp + tid];
+  __syncthreads();
+  for (int rb = 0; rb < ROWS; rb += NT / 16) {
+    if (rb + 2 * warp >= live) continue;                      // whole warps
+    const int r = rb + (tid >> 4);
+    double y[TM];
+#pragma unroll
+    for (int c = 0; c < TM; ++c) y[c] = q + 16 * c < nc ? Bs[(q + 16 * c) * ROWS + r] : 0.0;
+#pragma unroll
+    for (int p = 0; p < TM; ++p)
+      for (int kk = 0; kk < 16; ++kk) {
+        const int k = 16 * p + kk;
+        if (k >= nc) break;
+        const double* lk = Ls + k * ncp + q;
+        const double v = __shfl_sync(0xffffffffu, y[p], (lane & 16) | kk) * rinv[k];
+        if (q == kk) y[p] = v;
+        else if (q > kk) y[p] = fma(-v, lk[16 * p], y[p]);
+#pragma unroll
+        for (int c = p + 1; c < TM; ++c)
+          if (16 * c < nc) y[c] = fma(-v, lk[16 * c], y[c]);
+      }
+    if (r >= live) continue;
+#pragma unroll
+    for (int c = 0; c < TM; ++c) {
+      const int j = q + 16 * c;
+      if (j >= nc) continue;
+      X[(size_t)j * ld + r] = y[c];
+      if (s32 != nullptr) s32[(size_t)j * ld32 + r] = (float)y[c];
+      if (s16 != nullptr) {
+        over16 |= fabs(y[c]) > (double)kF16Max;
+        s16[(size_t)r * lds + j] = __double2half(y[c]);
+      }
+    }
+  }
+  return over16;
+}
 
 // MR: 16-row tiles per CTA.  NT: threads, one warp per group of 8 columns (nc <= NT / 4).
 template <int MR, int NT>
@@ -587,39 +652,7 @@ trsm_refine64_kernel(double* __restrict__ A, int ld, int r0, int m, int c0, int 
         }
     }
   } else {
-    // FP64 substitution, 16 lanes per row: lane q holds columns q, q + 16, ..
-    for (int rb = 0; rb < ROWS; rb += NT / 16) {
-      const int r = rb + (tid >> 4), q = tid & 15;
-      const bool in = r < live;
-      double y[TM];
-#pragma unroll
-      for (int c = 0; c < TM; ++c) y[c] = (q + 16 * c < nc && in) ? Bg[(size_t)(q + 16 * c) * ld + r] : 0.0;
-#pragma unroll
-      for (int p = 0; p < TM; ++p)
-        for (int kk = 0; kk < 16; ++kk) {
-          const int k = 16 * p + kk;
-          if (k >= nc) break;
-          const double* Lk = Lm + (size_t)(c0 + k) * ldl + c0;
-          const double v = __shfl_sync(0xffffffffu, y[p], (lane & 16) | kk) / Lk[k];
-          if (q == kk) y[p] = v;
-#pragma unroll
-          for (int c = p; c < TM; ++c) {
-            const int j = q + 16 * c;
-            if (j > k && j < nc) y[c] = fma(-v, Lk[j], y[c]);
-          }
-        }
-#pragma unroll
-      for (int c = 0; c < TM; ++c) {
-        const int j = q + 16 * c;
-        if (j >= nc || !in) continue;
-        A[(size_t)(c0 + j) * ld + r0 + row0 + r] = y[c];
-        if (S32 != nullptr) S32[(size_t)(c0 + j) * ld32 + r0 + row0 + r] = (float)y[c];
-        if (S != nullptr) {
-          over16 |= fabs(y[c]) > (double)kF16Max;
-          S[(size_t)(r0 + row0 + r) * lds + c0 + j] = __double2half(y[c]);
-        }
-      }
-    }
+    over16 = substitute<TM, ROWS, NT>(A, ld, r0, m, c0, nc, Lm, ldl, smem, S, lds, S32, ld32);
   }
   if (S != nullptr && __any_sync(0xffffffffu, over16) && lane == 0) atomicOr(err, DEV_ERR_RANGE16);
 }
