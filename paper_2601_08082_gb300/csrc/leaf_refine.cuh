@@ -22,7 +22,7 @@
 // nothing else waits.
 //
 // A leaf whose diagonal is not positive, with |a_ij| > sqrt(a_ii a_jj), a binary32 pivot that is not
-// positive, or that does not converge (condition number above ~10^5) is left untouched and
+// positive, or that would not converge soon (a kernel matrix with nugget below ~10^-3) is left untouched and
 // factored by the direct schedules in the same launch.
 #pragma once
 #include <cooperative_groups.h>
@@ -41,6 +41,12 @@ constexpr int kTiles = 36;
 constexpr int kTtLd = 136;             // halves per row of the staged column block
 constexpr int kMaxStep = 6;
 constexpr float kTol = 0x1p-57f;
+// A leaf gives up where the loop would take longer than the direct schedules: with a scaled pivot of binary32
+// below kMinPivot, or a first correction above kMaxFirst (each step gains that factor: five steps of
+// ~12 us).  Kernel matrices of order 128, nugget 1e-2, 1e-3 and 1e-4, us: refined 74, given up 133 and 112
+// (186 and 186 when every leaf ran to its sixth step); FP64 schedule alone 106, double-float 70, where
+// giving up costs 97 and 78.
+constexpr float kMinPivot = 0x1p-12f, kMaxFirst = 0x1p-12f;
 
 struct Smem {
   unsigned long long Lx[kTiles][256];  // L in units of 2^(e_i - 62) plus kByteBias, rows swizzled
@@ -198,7 +204,7 @@ __device__ __forceinline__ bool potrf32(Smem& sm, int p, int lane) {
       nq = __shfl_sync(full, a[k + 2], k + 3);
       ns = __shfl_sync(full, a[k + 3], k + 3);
     }
-    ok = ok && d0 > 1e-12f && det > 1e-12f * d0;   // scaled pivots: false for NaN too
+    ok = ok && d0 > kMinPivot && det > kMinPivot * d0;   // scaled pivots: false for NaN too
     const float m = q * r0, r1 = d0 * r0 * rd;
     const float4 rr = make_float4(r0, r1, m, 0.f);
     const float x = a[k] * r0;                   // column k of L (rows >= k)
@@ -730,7 +736,7 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
     }
     cluster.sync();                                            // B2: the corrections are written
     em = cluster_max(cluster, &sm.emax[par]) * fsi;          // the scale is the same in every CTA
-    if (!(em < 0.25f)) break;
+    if (!(em < (step == 0 ? kMaxFirst : 0.25f))) break;
     if (step == 0) first = fmaxf(em, 0x1p-24f);
     else if (em > 0.25f * last && em > 0x1p-50f) break;
     last = em;
