@@ -1270,10 +1270,10 @@ hrp_status hrp_posv(hrp_handle* h, const hrp_tree* tree, int n, int nrhs, const 
     if ((st = check_dev_err(h, s)) == HRP_ERR_RANGE && attempt == 0) continue;
     if (st != HRP_OK) return st;
     if (hinfo) continue;
-    // the inverses of the diagonal blocks serve all solves with this factor: from n = 128 to 8192, 1 to
-    // 16 right-hand sides, one correction, no slower than FP32 sweeps anywhere (one right-hand side:
-    // n = 200 330 -> 308 us a call, 1024 892 -> 851, 4096 4611 -> 4404; 16: 407 -> 328, 1011 -> 928,
-    // 4921 -> 4757)
+    // the inverses of the diagonal blocks serve all solves with this factor.  A call with one correction, ms,
+    // with them and with FP32 sweeps instead: one right-hand side, n = 128 0.182 / 0.252, 1024 0.819 /
+    // 0.868, 4096 3.48 / 3.66, 32768 71.5 / 71.9; 16: 0.182 / 0.278, 0.924 / 0.986, 3.88 / 4.16, 12000
+    // 18.8 / 19.4, 16384 26.8 / 26.8, 32768 82.6 / 83.9
     const bool prepared = solve_workspace(h, n, s);
     if (prepared) {
       if ((e = launch_solve_inverses(h->fact, n, n, h->swork, s)) != cudaSuccess) return cuda_status(h, e, "hrp_posv");
