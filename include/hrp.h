@@ -186,11 +186,12 @@ hrp_status hrp_potrf_host(hrp_handle* h, const hrp_tree* tree, int n, const doub
 
 /*
  * Arithmetic of the FP64 leaves (Alg. 1 base case, the 128 x 128 leaf on an 8-CTA cluster).
- * A leaf is first factored in binary32 and refined with exact residuals to |A - L L^T|_ij <= 2^-56
- * sqrt(a_ii a_jj) (the bound of an FP64 Cholesky factorization is (n + 1) 2^-53 of it; entries of L far
- * below sqrt(a_ii) are accurate to 2^-56 of that, not of themselves).  A leaf that cannot be refined (a
- * pivot in binary32 below about 2^-12 of its diagonal entry, an entry that is not finite or above
- * sqrt(a_ii a_jj)) is factored directly, in the same launch:
+ * A leaf is first factored in binary32 and refined with exact residuals: |A - L L^T|_ij <= 2^-52
+ * sqrt(a_ii a_jj), the rounding of L to FP64 included (an FP64 Cholesky factorization: (n + 1) 2^-53).
+ * Entries below 2^-26 of their scale (2^-30 where the tree has a level below FP64) are computed again
+ * in FP64, and exact zeros stay zeros.  A leaf that cannot be refined (a pivot in binary32 below about
+ * 2^-12 of its diagonal entry, an entry that is not finite or above sqrt(a_ii a_jj), more than 16
+ * entries that small) is factored directly, in the same launch:
  *   mode 1: in double-float arithmetic (pairs of binary32, Dekker 1971; about 48 significant bits,
  *     relative error of each operation a few units of 2^-48) on the FP32 pipe, and again in FP64
  *     where an entry that is not finite, or a diagonal entry or pivot that is not positive or falls

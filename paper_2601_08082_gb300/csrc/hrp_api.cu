@@ -342,8 +342,8 @@ struct Fact {
     lc.pdl = !(w != waited.end() && w->second);
     if (w != waited.end()) w->second = false;
     lc.max_ctas = (la && s != main_s) ? side_ctas : 0;
-    lc.leaf_df = h->leaf_chain == 1 ||
-                 (h->leaf_chain < 0 && (tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || tree_has(t, HRP_F8E4M3)));
+    lc.lower = tree_has(t, HRP_F32) || tree_has(t, HRP_F16) || tree_has(t, HRP_F8E4M3);
+    lc.leaf_df = h->leaf_chain == 1 || (h->leaf_chain < 0 && lc.lower);
     if (h->timing) {
       cudaEvent_t e = event(ev_next);
       began = e && cudaEventRecord(e, s) == cudaSuccess;

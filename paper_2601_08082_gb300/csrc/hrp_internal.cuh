@@ -46,6 +46,7 @@ struct LaunchCtx {
   bool pdl = true;
   int max_ctas = 0;
   bool leaf_df = false;   // FP64 leaves: 16 x 16 pivot chains in double-float (k_leaf_cluster.cu)
+  bool lower = false;     // the tree has a level below FP64
 };
 inline LaunchCtx& launch_ctx() {
   thread_local LaunchCtx c;
@@ -78,7 +79,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // DEV_ERR_RANGE16.
 // scratch: kLeafScratch floats of device memory, 16-byte aligned, for the FP64 leaves' refinement (no
 // initial contents needed; calls that may overlap need one each), or nullptr to do without it.
-constexpr int kLeafScratch = 2 * 36 * 256;
+constexpr int kLeafScratch = 2 * 36 * 256 + 2 * 36 * 8;
 cudaError_t launch_potrf_leaf(double* A, int ld, int n, int col0, bool compute64, bool round16,
                               float* W32, int ldw, int* info, unsigned* err, float* scratch, cudaStream_t s);
 

@@ -908,14 +908,14 @@ __device__ int leaf_body(double* __restrict__ A, int ld, int n, int col0, float*
 
 __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCThreads, 1)
 potrf_leaf_cluster_kernel(double* __restrict__ A, int ld, int n, int col0, float* __restrict__ W32, int ldw,
-                          int* __restrict__ info, int df, float* scratch) {
+                          int* __restrict__ info, int df, float* scratch, float thr) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // an earlier block failed: stop like LAPACK (every CTA reads the same value: nothing in this
   // kernel writes info before a cluster barrier)
   if (*(volatile int*)info != INT_MAX) return;
-  if (scratch != nullptr && leafref::leaf_refine(A, ld, n, W32, ldw, scratch, smem_raw)) return;
+  if (scratch != nullptr && leafref::leaf_refine(A, ld, n, W32, ldw, scratch, thr, smem_raw)) return;
   if (df) {
     if (leaf_body<dfloat>(A, ld, n, col0, W32, ldw, info, smem_raw) != kFallback) return;
     cg::this_cluster().sync();          // every CTA has left the double-float attempt
@@ -944,7 +944,8 @@ cudaError_t launch_potrf_leaf_cluster(double* A, int ld, int n, int col0, float*
     attr_mask |= attr_bit;
   }
   (void)launch_pdl(potrf_leaf_cluster_kernel, dim3(kCL), dim3(kCThreads), kLeafSmem, s, A, ld, n, col0,
-                   W32, ldw, info, launch_ctx().leaf_df ? 1 : 0, scratch);
+                   W32, ldw, info, launch_ctx().leaf_df ? 1 : 0, scratch,
+                   ldexpf(1.f, -(launch_ctx().lower ? leafref::kCoarseBits : leafref::kFineBits)));
   return cudaGetLastError();
 }
 

@@ -21,6 +21,14 @@
 // measured at ~9 bytes per clock and SM for this all-to-all pattern), two cluster barriers a step;
 // nothing else waits.
 //
+// The error is relative to the scales, and an entry of L far below its own (weakly coupled unknowns) keeps
+// fewer digits than in an FP64 factorization.  So sum |l_ik| |l_jk| + |a_ij| is estimated for every entry from L0
+// (one mma a 16 x 8 tile and 16 terms); where it is zero, so is l_ij; entries below 2^-kFineBits or
+// 2^-kCoarseBits are computed again in FP64 at the end, l_ij = (a_ij - sum_{k<j} l_ik l_jk) / l_jj, up to kMaxRepair
+// of them (~1 us each; a leaf with more is factored directly).  The others are accurate to 2^-57 of the scale, so
+// to 2^-31 of themselves at the line.  Factors of dominant matrices of order n have entries of 2^-16 at n = 8192,
+// and one in 10^4 of those below 2^-30; all-FP64 trees are for the smaller orders.
+//
 // A leaf whose diagonal is not positive, with |a_ij| > sqrt(a_ii a_jj), a binary32 pivot that is not
 // positive, or that would not converge soon (a kernel matrix with nugget below ~10^-3) is left untouched and
 // factored by the direct schedules in the same launch.
@@ -48,6 +56,10 @@ constexpr float kTol = 0x1p-57f;
 // giving up costs 97 and 78.
 constexpr float kMinPivot = 0x1p-12f, kMaxFirst = 0x1p-12f;
 
+// Entries of L below their scale by kFineBits (all-FP64 trees) or kCoarseBits (others, whose off-diagonal blocks carry
+// binary32's 2^-24) are computed again in FP64; a leaf with more than kMaxRepair is factored directly
+constexpr int kMaxRepair = 16, kFineBits = 26, kCoarseBits = 30;
+
 struct Smem {
   unsigned long long Lx[kTiles][256];  // L in units of 2^(e_i - 62) plus kByteBias, rows swizzled
   union {
@@ -62,6 +74,10 @@ struct Smem {
   float4 xy[16][16];                   // phase 1: the diagonal block's column pairs, rows 2 j, 2 j + 1
   float4 rr[16];                       // phase 1: 1 / l_kk, 1 / l_{k+1,k+1}, l_{k+1,k} of a pair
   int e[128];                          // scales
+  unsigned zero[8][2][4];              // this column block's entries of L that are zero (half tiles, as the words of xC)
+  double rep_a[kMaxRepair];            // CTA 0: the entries to compute again, by column, and their values in A
+  int rep[kMaxRepair], nrep;
+  int nlow;                            // such entries found here, half tiles with zeros times 2^16, with lost ones times 2^24
   unsigned rmax[2], emax[2];           // largest |R| and scaled |E| here (bits), by step parity
 };
 
@@ -469,14 +485,44 @@ __device__ __forceinline__ float cluster_max(cg::cluster_group& cluster, unsigne
   return __uint_as_float(m);
 }
 
-// floats of global scratch the refinement exchanges through: residual tiles, then corrections
-constexpr int kScratch = 2 * kTiles * 256;
+// floats of global scratch the refinement exchanges through: residual tiles, corrections, and 8 words per half tile
+constexpr int kScratch = 2 * kTiles * 256 + 2 * kTiles * 8;
+
+// Entry classes of a half tile (rows 16 I .., columns 16 J + 8 h ..), from est = |a_ij| + sum_k |l_ik| |l_jk| with the
+// binary32 factor's upper halves (a: A's entries in units of 2^-58 of their scales, bit q of nz: a_ij is not zero): bits (lane, q) of low[q] where est is below thr, of zero[q] where it is zero
+// (then so is l_ij); any entry that its upper half cannot hold sets `lost`.
+__device__ __forceinline__ void entry_classes(const Smem& sm, int I, int J, int h, const long long (&a)[4], int nz, int n, float thr, int lane,
+                                              unsigned (&low)[4], unsigned (&zero)[4], bool& lost) {
+  float c[4] = {};
+#pragma unroll 2
+  for (int k = 0; k <= J; ++k) {
+    uint32_t ah[4], bh[4];
+    frag<Op::A>(ah, sm.L0.h[tix(I, k)][0], lane);
+    frag<Op::B>(bh, sm.L0.h[tix(J, k)][0], lane);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ah[q] &= 0x7fff7fffu;
+    dig_mma(c, ah, (h ? bh[2] : bh[0]) & 0x7fff7fffu, (h ? bh[3] : bh[1]) & 0x7fff7fffu);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int gi = 16 * I + (lane >> 2) + 8 * (q >> 1), gj = 16 * J + 8 * h + 2 * (lane & 3) + (q & 1);
+    const bool in = gi < n && gi > gj;
+    float est = c[q];
+    if (in && ((nz >> q) & 1)) {
+      const unsigned long long v = (unsigned long long)(a[q] < 0 ? -a[q] : a[q]);
+      est += fmaxf(fmaf((float)(unsigned)(v >> 32), 0x1p-26f, (float)(unsigned)v * 0x1p-58f), 0x1p-120f);
+    }
+    low[q] = __ballot_sync(0xffffffffu, in && est > 0.f && est < thr);
+    zero[q] = __ballot_sync(0xffffffffu, in && est == 0.f);
+    lost |= in && est > 0.f && est < 0x1p-24f;
+  }
+}
 
 // The leaf.  Returns true when A holds L (and W32 its FP32 inverse); false, the same in every CTA,
 // with nothing written, when the direct schedules must factor it.  Every thread of the cluster
 // takes the same path through the cluster barriers.
 __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __restrict__ W32, int ldw,
-                            float* scratch, unsigned char* smem_raw) {
+                            float* scratch, float thr, unsigned char* smem_raw) {
   Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -484,6 +530,8 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
   const int NB = (n + 31) / 32, T = 2 * NB, NTL = T * (T + 1) / 2;
   float* xR = scratch;                        // residual tiles
   float* xD = scratch + kTiles * 256;         // corrections of L
+  unsigned* xC = reinterpret_cast<unsigned*>(scratch + 2 * kTiles * 256);   // entry classes
+  int total = 0;                              // entries to compute again
 
   // this warp's residual units: half tiles (16 rows, 8 columns) of the CTA's tiles, longest products
   // first; the tile's entries in fixed point (unit 2^(e_i + e_j - 58)) stay in registers
@@ -534,6 +582,7 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
         araw[x][q] = (uI[x] >= 0 && gr < n) ? A[(size_t)gc * ld + gr] : 0.0;
       }
     if (tid < 2) sm.rmax[tid] = sm.emax[tid] = 0;
+    if (tid == 0) sm.nlow = sm.nrep = 0;
     if (tid < 128) {
       int e = 0;
       if (tid < n) {
@@ -564,6 +613,7 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
   }
   if (__syncthreads_or(bad)) return false;
   long long afix[2][4];
+  int nz = 0;
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
     if (uI[x] < 0) continue;
@@ -572,6 +622,7 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
       const int gi = 16 * uI[x] + (lane >> 2) + 8 * (q >> 1), gj = 16 * uJ[x] + 8 * uH[x] + 2 * (lane & 3) + (q & 1);
       afix[x][q] = 0;
       if (gi < n && gj < n) afix[x][q] = dig_fix(araw[x][q], sm.e[gi] + sm.e[gj] + 2 + 1022) >> 2;
+      if (((unsigned)__double2hiint(araw[x][q]) << 1) | (unsigned)__double2loint(araw[x][q])) nz |= 1 << (4 * x + q);
       if (gi >= n && gi == gj) afix[x][q] = 1ll << 57;         // 0.5
     }
   }
@@ -597,6 +648,24 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
     // ---- R = A - L L^T: this CTA's tiles, to the scratch ----
     const int par = step & 1;
     float mx = 0.f;
+    if (step == 0) {
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (uI[x] < 0) continue;
+        unsigned low[4], zero[4], w = 0;
+        bool lost = false;
+        entry_classes(sm, uI[x], uJ[x], uH[x], afix[x], nz >> (4 * x), n, thr, lane, low, zero, lost);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (lane == q) w = low[q];
+          if (lane == 4 + q) w = zero[q];
+        }
+        if (lane < 8) __stcg(xC + (tix(uI[x], uJ[x]) * 2 + uH[x]) * 8 + lane, w);
+        const int c = __popc(low[0]) + __popc(low[1]) + __popc(low[2]) + __popc(low[3]) +
+                      (zero[0] | zero[1] | zero[2] | zero[3] ? 1 << 16 : 0) + (__any_sync(0xffffffffu, lost) ? 1 << 24 : 0);
+        if (lane == 0 && c) atomicAdd(&sm.nlow, c);
+      }
+    }
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
       if (uI[x] < 0) continue;
@@ -630,6 +699,49 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
       g[u] = (idx >> 6) < NTL ? __ldcg(reinterpret_cast<const float4*>(xR) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     mx = cluster_max(cluster, &sm.rmax[par]);
+    if (step == 0) {
+      int w[kCtas];
+      bool zeros = false, lost = false;
+#pragma unroll
+      for (int u = 0; u < kCtas; ++u) w[u] = *(volatile int*)cluster.map_shared_rank(&sm.nlow, u);
+#pragma unroll
+      for (int u = 0; u < kCtas; ++u) {
+        total += w[u] & 0xffff;
+        zeros |= ((w[u] >> 16) & 0xff) != 0;
+        lost |= (w[u] >> 24) != 0;
+      }
+      // the same in every CTA.  (Fill from an entry that its upper half cannot hold would pass for a zero.)
+      if (total > kMaxRepair || (zeros && (lost || total > 0))) break;
+      if (mine && tid < 64) {
+        const int I = tid >> 3;
+        (&sm.zero[0][0][0])[tid] = I >= rank && I < T ? __ldcg(xC + (tix(I, rank) * 2 + ((tid >> 2) & 1)) * 8 + 4 + (tid & 3)) : 0u;
+      }
+      if (rank == 0 && total > 0) {
+        // half tile u / 4, word u % 4
+        for (int u = tid; u < 2 * NTL * 4; u += kThreads) {
+          const int t = u >> 3, h = (u >> 2) & 1, q = u & 3;
+          int I = 0;
+          while ((I + 1) * (I + 2) / 2 <= t) ++I;
+          const int J = t - I * (I + 1) / 2;
+          for (unsigned m = __ldcg(xC + (t * 2 + h) * 8 + q); m; m &= m - 1) {
+            const int l = __ffs(m) - 1, i = 16 * I + (l >> 2) + 8 * (q >> 1), j = 16 * J + 8 * h + 2 * (l & 3) + (q & 1);
+            const int at = atomicAdd(&sm.nrep, 1);
+            sm.rep[at] = (j << 8) | i;
+          }
+        }
+        __syncthreads();
+        if (warp == 0) {                                       // by column, then row
+          const int v = lane < total ? sm.rep[lane] : INT_MAX;
+          int at = 0;
+          for (int u = 0; u < total; ++u) at += __shfl_sync(0xffffffffu, v, u) < v;
+          __syncwarp();
+          if (lane < total) {
+            sm.rep[at] = v;
+            sm.rep_a[at] = A[(size_t)(v >> 8) * ld + (v & 255)];
+          }
+        }
+      }
+    }
     // scale 2^s with max |R| 2^s in [0.5, 1)
     const int xe = max((int)(__float_as_uint(mx) >> 23) & 0xff, 1) - 126;
     const int s = min(-xe, 100);
@@ -846,8 +958,11 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
 #pragma unroll
     for (int I = 0; I < 8; ++I) {
       const int gi = 16 * I + li;
-      if (I >= J && I < T && gi < n && gj <= gi)
-        A[(size_t)gj * ld + gi] = dig_to_double((long long)(sm.Lx[tix(I, J)][lx(li, lk)] - kByteBias), sm.e[gi] - 62);
+      if (I >= J && I < T && gi < n && gj <= gi) {
+        // bit of entry (li, lk) in its half tile's words: lane 4 (li mod 8) + (lk mod 8) / 2, register 2 (li / 8) + lk mod 2
+        const bool z = (sm.zero[I][lk >> 3][2 * (li >> 3) + (lk & 1)] >> (4 * (li & 7) + ((lk & 7) >> 1))) & 1;
+        A[(size_t)gj * ld + gi] = z ? 0.0 : dig_to_double((long long)(sm.Lx[tix(I, J)][lx(li, lk)] - kByteBias), sm.e[gi] - 62);
+      }
     }
     if (W32 != nullptr) {
       const int gi = 16 * rank + li;
@@ -857,6 +972,19 @@ __device__ bool leaf_refine(double* __restrict__ A, int ld, int n, float* __rest
     }
   }
   cluster.sync();                       // no CTA leaves (or reuses its memory) while others may read it
+  if (good && total > 0 && rank == 0 && warp == 0) {
+    // l_ij = (a_ij - sum_{k<j} l_ik l_jk) / l_jj from the finished entries, column by column
+    for (int u = 0; u < total; ++u) {
+      const int i = sm.rep[u] & 255, j = sm.rep[u] >> 8;
+      double t = 0.0;
+      for (int k = lane; k < j; k += 32) t = fma(__ldcg(A + (size_t)k * ld + i), __ldcg(A + (size_t)k * ld + j), t);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) A[(size_t)j * ld + i] = (sm.rep_a[u] - t) / __ldcg(A + (size_t)j * ld + j);
+      __threadfence_block();
+      __syncwarp();
+    }
+  }
   return good;
 }
 
