@@ -42,11 +42,11 @@ FP32_MEASURED_TFLOPS = 75.2
 # DRAM bytes (read + write) per launch of the leaf POTRF kernel from one ncu capture, reported
 # while the kernel's device code is the code captured: its sources (the first up to the launcher),
 # hashed.
-LEAF_TRAFFIC = {"bytes": 246144, "sources": [
+LEAF_TRAFFIC = {"bytes": 262144, "sources": [
     ("paper_2601_08082_gb300/csrc/k_leaf_cluster.cu", "cudaError_t launch_potrf_leaf_cluster(",
-     "05eebf399f6f05f6004264c9a307ba2179178c67"),
+     "205b8d72970f354b2e14e73813333bcddeacabf9"),
     ("paper_2601_08082_gb300/csrc/leaf_refine.cuh", "}  // namespace leafref",
-     "7ae23e0bb92880bce7ba12789ae2eb5046d57841")]}
+     "83eaff2e3b5a8af4d20ec53b9a67ad838859c1a2")]}
 # The leaves' yardstick in trees with a level below FP64 is double-float arithmetic on the FP32 pipe
 # (their direct schedule; the refinement that runs first does the work as digit products): one
 # double-float multiply-add (the Dot2 accumulation step of the tile updates) is 12 FP32 instructions,

@@ -84,7 +84,7 @@ cudaError_t launch_potrf_leaf(double* A, int ld, int n, int col0, bool compute64
                               float* W32, int ldw, int* info, unsigned* err, float* scratch, cudaStream_t s);
 
 // The same FP64 leaf POTRF (no FP16 rounding) on a cluster of 8 CTAs holding 16 x 16
-// tiles in shared memory (k_leaf_cluster.cu); launch_potrf_leaf uses it for n > 32.
+// tiles in shared memory (k_leaf_cluster.cu); launch_potrf_leaf uses it for n > 8.
 cudaError_t launch_potrf_leaf_cluster(double* A, int ld, int n, int col0, float* W32, int ldw, int* info,
                                       float* scratch, cudaStream_t s);
 

@@ -2,8 +2,8 @@
 // factor (leaf_refine.cuh), and, for the leaves that cannot be refined, by the direct schedules
 // below in FP64 or in double-float arithmetic on the FP32 pipe.
 //
-// Order 128, one leaf alone in a call with copy and info kernels: 95 us (FP64 schedule) and 60 us
-// (double-float) -> 47 us refined, 68 us for kernel matrices that take a third and fourth step.
+// Order 128, one leaf alone in a call with copy and info kernels: 106 us (FP64 schedule) and 70 us
+// (double-float) -> 64 us refined, 74 us for kernel matrices that take a third step.
 //
 // FP64 on this GPU: each SM sub-partition issues one FP64 warp instruction per ~64
 // cycles (also the dependent latency), the SM as a whole about one per 19 cycles

@@ -34,10 +34,11 @@
 // the warps' sums converted and added in FP64, ~2000 instead of ~1600 instructions a tile: n = 4096 560
 // -> 542 us, 8192 1246 -> 1186, 16384 3232 -> 2995 with 16 right-hand sides).  Solves against the
 // sweeps', us with 1, 4 and 16 right-hand sides:
-//   n = 64 18 18 23 (56 60 84), 128 41 41 47 (105 113 140), 2048 231 236 282 (248 365 994),
-//   4 and 16: 4096 421 542 (637 1914), 8192 896 1186 (1204 3794).
-// Backward errors are 3 to 30 times below the sweeps' (whose double-float products keep 44 bits), also
-// for kernel matrices of condition 1e15.  Tiles that meet a NaN or an infinity use FP64 FMAs.
+//   n = 64 21 21 29 (56 61 85), 128 43 43 50 (105 113 144), 2048 238 243 303 (249 367 997),
+//   4 and 16: 4096 436 590 (636 1908), 8192 933 1314 (1204 3788), 16384 2225 3306 (3191 8756).
+// Backward errors entry by entry are at or below 1e-14 of |A| |x| where the sweeps' (whose double-float
+// products keep 44 bits and drop what is 2^-74 below its group) reach 1e-13 for ordinary matrices and 1 for
+// ones in mixed units.  Tiles that meet a NaN or an infinity use FP64 FMAs.
 #include <cooperative_groups.h>
 
 #include <climits>
@@ -673,8 +674,8 @@ cudaError_t launch_solve(const double* L, int ldl, double* B, int ldb, int n, in
 }
 
 // Single solves gain at every size (figures above) but with one right-hand side on large factors, whose
-// sweeps read L once and whose links are short: n = 2048 231 us against 248, 4096 about equal (418),
-// 8192 870 against 794.  In a batch, whose systems overlap on streams, the launches count: 24 FP64
+// sweeps read L once and whose links are short: n = 2048 238 us against 249, 4096 about equal (417),
+// 8192 870 against 795.  In a batch, whose systems overlap on streams, the launches count: 24 FP64
 // systems of 64 .. 1024, factored and solved with 4 right-hand sides, take 3.01 ms with the block solve up
 // to 256 rows, 2.91 up to 512, 3.31 up to 1024.  Up to 8 right-hand sides and 1024 rows single solves do as
 // batched ones, so that both agree to the bit there (at 1024 rows that costs a single solve 45 us of
