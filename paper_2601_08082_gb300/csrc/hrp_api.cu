@@ -176,9 +176,12 @@ template <typename T>
 bool ensure_optional(hrp_handle* h, T** p, size_t* cap, size_t need, cudaStream_t s, size_t* refused = nullptr) {
   if (*cap >= need && *p) return true;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if ((refused && need >= *refused) || cudaStreamIsCapturing(s, &capturing) != cudaSuccess ||
-      capturing != cudaStreamCaptureStatusNone)
+  if (refused && need >= *refused) return false;
+  if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) {
+    cudaGetLastError();
     return false;
+  }
+  if (capturing != cudaStreamCaptureStatusNone) return false;
   T* q = nullptr;
   if (need * sizeof(T) >= h->alloc_limit || cudaMalloc(reinterpret_cast<void**>(&q), need * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
